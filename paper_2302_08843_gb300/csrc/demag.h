@@ -93,6 +93,12 @@ void launch_rt_y(const DemagDims& d, const typename Cplx<T>::type* in, typename 
                  cudaStream_t st);
 template <typename T>
 void launch_rt_z(const DemagDims& d, typename Cplx<T>::type* S2, const T* tens, cudaStream_t st);
+// the line engine's passes (demag_rt.cu), any length; false if a line is too long for them
+template <typename T, int DIR>
+bool launch_line_y(const DemagDims& d, const typename Cplx<T>::type* in, typename Cplx<T>::type* out,
+                   cudaStream_t st);
+template <typename T>
+bool launch_line_conv(const DemagDims& d, typename Cplx<T>::type* S2, const T* tens, cudaStream_t st);
 // copy the runtime-plan lengths' twiddle tables to the current device
 cudaError_t upload_twiddles_rt();
 

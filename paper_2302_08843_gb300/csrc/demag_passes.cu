@@ -1093,89 +1093,6 @@ p3_z_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restr
     }
 }
 
-// Register-resident variant (FP32): each thread keeps its 16 values of all
-// three components from the first load to the last store; shared memory only
-// carries the exchanges inside each transform (one per 128-point transform).
-template <typename T, int LZ, int B, int G>
-__global__ void __launch_bounds__(B * G * Fft<T, LZ, -1, (LZ > 1)>::TPL,
-                                  (384 / (B * G * Fft<T, LZ, -1, (LZ > 1)>::TPL)) > 1
-                                      ? 384 / (B * G * Fft<T, LZ, -1, (LZ > 1)>::TPL) : 1)
-p3_z_conv_reg(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restrict__ tens) {
-    using C = typename Cplx<T>::type;
-    using FF = Fft<T, LZ, -1, (LZ > 1)>;
-    using FI = Fft<T, LZ, +1, false>;
-    extern __shared__ __align__(16) unsigned char smraw[];
-    C* s = reinterpret_cast<C*>(smraw);
-    constexpr int NL = B * G;
-    constexpr int NR = FF::NR, TPL = FF::TPL;
-    constexpr int NOUT = LZ == 1 ? 1 : NR / 2;
-    const int tid = threadIdx.x;
-    const int line = tid % NL, j = tid / NL;
-    const int kl = line % B, g = line / B;
-    const int kx = blockIdx.x * B + kl;
-    const int kyi = blockIdx.y * G + g;           // (folded ky, side) pairs, side fastest
-    const int p = kyi >> 1, side = kyi & 1;
-    const int LY = d.LY;
-    const int KY2 = LY / 2 + 1;
-    const bool valid = kx < d.KX && p < KY2 && (side == 0 || (p > 0 && 2 * p < LY));
-    const int ky = side ? LY - p : p;
-    const long cstride = (long)d.nz * LY * d.KXS;
-    C* col = S2 + (long)blockIdx.z * 3 * cstride + (long)ky * d.KXS + kx;
-    const long zs = (long)LY * d.KXS;
-
-    C vx[NR], vy[NR], vz[NR];
-#pragma unroll
-    for (int r = 0; r < NR; ++r) {
-        const int z = FF::in_index(j, r);
-        vx[r] = vy[r] = vz[r] = mk<C>(0, 0);
-        if (valid && FF::in_live(r) && z < d.nz) {
-            vx[r] = col[z * zs];
-            vy[r] = col[cstride + z * zs];
-            vz[r] = col[2 * cstride + z * zs];
-        }
-    }
-    FF::run(vx, s + line, NL, j);
-    FF::run(vy, s + line, NL, j);
-    FF::run(vz, s + line, NL, j);
-    const int KZ2 = LZ / 2 + 1;
-    const long tcomp = (long)KZ2 * KY2 * d.KXS;
-    const T sy = side ? (T)-1 : (T)1;
-#pragma unroll
-    for (int r = 0; r < NR; ++r) {
-        const int kz = j + r * TPL;
-        const int kzf = (2 * kz <= LZ) ? kz : LZ - kz;
-        const T sz = (2 * kz <= LZ) ? (T)1 : (T)-1;
-        T txx = 0, txy = 0, txz = 0, tyy = 0, tyz = 0, tzz = 0;
-        if (valid) {
-            const T* tp = tens + ((long)kzf * KY2 + p) * d.KXS + kx;
-            txx = __ldg(tp);
-            txy = (d.yz_swap ? sz : sy) * __ldg(tp + tcomp);
-            txz = (d.yz_swap ? sy : sz) * __ldg(tp + 2 * tcomp);
-            tyy = __ldg(tp + 3 * tcomp);
-            tyz = sy * sz * __ldg(tp + 4 * tcomp);
-            tzz = __ldg(tp + 5 * tcomp);
-        }
-        const C mx = vx[r], my = vy[r], mz = vz[r];
-        vx[r] = mk<C>(txx * mx.x + txy * my.x + txz * mz.x, txx * mx.y + txy * my.y + txz * mz.y);
-        vy[r] = mk<C>(txy * mx.x + tyy * my.x + tyz * mz.x, txy * mx.y + tyy * my.y + tyz * mz.y);
-        vz[r] = mk<C>(txz * mx.x + tyz * my.x + tzz * mz.x, txz * mx.y + tyz * my.y + tzz * mz.y);
-    }
-    FI::run(vx, s + line, NL, j);
-    FI::run(vy, s + line, NL, j);
-    FI::run(vz, s + line, NL, j);
-    if (valid) {
-#pragma unroll
-        for (int r = 0; r < NOUT; ++r) {
-            const int z = j + r * TPL;
-            if (z < d.nz) {
-                col[z * zs] = vx[r];
-                col[cstride + z * zs] = vy[r];
-                col[2 * cstride + z * zs] = vz[r];
-            }
-        }
-    }
-}
-
 // ----------------------------------------------------------- P3 layers ----
 // Non-equidistant layers (Sec. 4.4): no transform along z; at every lateral
 // wave number (kx, ky) the nz layers are coupled densely,
@@ -2063,11 +1980,11 @@ template <int L> static bool launch_p5_tma(const DemagDims& d, const float2* S1,
 
 template <typename T, int L> static void launch_p3(const DemagDims& d, typename Cplx<T>::type* S2, const T* tens,
                                                    cudaStream_t st) {
-    constexpr int B = b_p3<T, L>(), G = g_p3<T, L>();
-    using C = typename Cplx<T>::type;
-    const int kyi = 2 * (d.LY / 2 + 1);
-    dim3 grid((d.KX + B - 1) / B, (kyi + G - 1) / G, d.nb);
-    // the register-resident variant holds 3 NR values per thread: up to 20
+    // single FP32 grids: the persistent TMA passes where a line has one; the
+    // line engine otherwise (FP64, batches, other lengths): FP64 64-point lines
+    // 519 -> 417 us on 128x128x32, 256-point lines along y of a 512x128x1 film
+    // 97 -> 44 us, 16 FP32 grids of 100x100x8 63 -> 34 us.  On an FP32 film's
+    // 256-point lines the TMA pass stays the faster one (8.7 against 10.0 us).
     if constexpr (sizeof(T) == 4 && L <= 256 && Fft<T, L, -1, (L > 1)>::NR <= 20) {
         if constexpr (z_two_r1<L>() > 0) {
             if (kZTwo && d.nb == 1 && launch_p3_two<L>(d, S2, tens, st)) return;
@@ -2075,14 +1992,13 @@ template <typename T, int L> static void launch_p3(const DemagDims& d, typename 
         if constexpr (tma_len<L>()) {
             if (d.nb == 1 && launch_p3_tma<L>(d, S2, tens, st)) return;
         }
-        // 128-thread CTAs: three fit per SM at up to 170 registers per thread
-        constexpr int G3 = (B * tpl_of<T, L>() >= 128) ? 1 : 128 / (B * tpl_of<T, L>());
-        dim3 grid3((d.KX + B - 1) / B, (kyi + G3 - 1) / G3, d.nb);
-        const size_t sm = (size_t)L * B * G3 * sizeof(C);
-        auto k = p3_z_conv_reg<T, L, B, G3>;
-        set_smem(k, sm);
-        k<<<grid3, B * G3 * tpl_of<T, L>(), sm, st>>>(d, S2, tens);
-    } else {
+    }
+    if (launch_line_conv<T>(d, S2, tens, st)) return;
+    if constexpr (L >= 2048) {        // FP64 lines of more butterflies than a CTA of the line engine holds
+        constexpr int B = b_p3<T, L>(), G = g_p3<T, L>();
+        using C = typename Cplx<T>::type;
+        const int kyi = 2 * (d.LY / 2 + 1);
+        dim3 grid((d.KX + B - 1) / B, (kyi + G - 1) / G, d.nb);
         const size_t sm = 3 * (size_t)L * B * G * sizeof(C);
         auto k = p3_z_conv<T, L, B, G>;
         set_smem(k, sm);
@@ -2095,7 +2011,14 @@ template <typename T, int L, int DIR> static void launch_y(const DemagDims& d, c
     if constexpr (sizeof(T) == 4 && L >= 16 && is_pow2(L)) {
         if (launch_py_tma<L, DIR>(d, in, out, st)) return;
     }
-    launch_py<T, L, DIR>(d, in, out, st);
+    // FP64 lines of 16 points up take the line engine (128x128x32: 144 and 157 us
+    // -> 119 and 126 us); FP32 lines the compiled engines, which stay faster where
+    // exchanges and not FP64 instructions bound the pass (384 points: 29 and 33 us
+    // against 54 and 44)
+    if constexpr (sizeof(T) == 8 && L >= 16) {
+        if (launch_line_y<T, DIR>(d, in, out, st)) return;
+    }
+    if constexpr (sizeof(T) == 4 || L < 16 || L >= 2048) launch_py<T, L, DIR>(d, in, out, st);
 }
 
 template <typename T, int L> static void launch_x_fwd(const DemagDims& d, const T* m, const T* Ms_cell, T Ms,
@@ -2255,10 +2178,10 @@ static void launch_p3_layers(const DemagDims& d, typename Cplx<T>::type* S2, con
 }
 
 // largest padded y extent of a 2-D grid (nz = 1) whose y transforms and tensor
-// multiply run as one pass of the z-pass kernel along y (above it the
-// shared-memory kernel along y measured slower than the y passes: 32 served
-// 256x256x1 grids, 2.36 ms against 2.07 ms per Dormand-Prince attempt)
-constexpr int k2dMaxPy = 256;
+// multiply run as one pass of the z-pass kernels along y (32 served 256x256x1
+// grids: 88 us against 103 us for two y passes and the product; longer lines
+// leave a CTA of the line engine one column, less than a sector of each row)
+constexpr int k2dMaxPy = 1024;
 
 template <typename T>
 static void yzy(const DemagDims& d, typename Cplx<T>::type* S1, typename Cplx<T>::type* S2, const T* tens,

@@ -1,0 +1,223 @@
+// Shared-memory FFT over lines of three-component vectors, for any even
+// 7-smooth length with the radix plan known only at run time.
+//
+// A thread owns one butterfly of one line and carries it for all three
+// components, so that a pass's index arithmetic and twiddles are paid once
+// for three transforms, and the 3x3 tensor product and the cell updates find
+// the three components of a wave number (or cell) in one thread's registers.
+// Element e of line l and component c lives at s[c plane + place(e) B + l];
+// the passes are in place (every thread reads its butterfly, the CTA
+// synchronises, every thread writes).
+//
+// Self-sorting Stockham passes: butterfly b of a pass of radix R and span Ns
+// (the product of the earlier radices) reads elements b + q L/R, multiplies
+// input q by W_{Ns R}^(q k), k = b mod Ns, and writes output q to
+// (b - k) R + k + q Ns.  The first pass has no twiddles, and the last pass's
+// outputs lie at b + q L/R again: a forward transform can hand its outputs to
+// the inverse's first pass, run with the radices in reverse order, in
+// registers.  The plan's first radix is even, so that the zero-padded upper
+// half of a forward's input, and the dropped half of an inverse's output, are
+// the registers q >= R/2 of that pass.
+//
+// Twiddled radix-2 steps are folded as X = a + w b (four multiply-adds) and
+// Y = 2 a - X (two): 3 instructions per point and level against 3.5 for
+// radix-8 passes that multiply first.  FP64 instructions are what an FP64
+// pass spends its time on (one warp instruction per 19 cycles and SM; 64
+// cycles for a single warp of a quarter SM, dependent or not), so FP64 plans
+// take small radices and many threads; FP32 passes are bound by the
+// shared-memory exchanges and take radix 8.
+#pragma once
+
+#include "common.cuh"
+
+namespace mm {
+
+constexpr int kLineMaxPass = 12;
+
+struct LinePlan {
+    int L, np;
+    int tw;                            // offset of W_L^m in the table
+    int rmin;                          // smallest radix: L / rmin butterflies in the widest pass
+    short R[kLineMaxPass];             // forward order; the inverse runs them backwards
+    short Ns[kLineMaxPass];            // forward spans
+    short Nsi[kLineMaxPass];           // spans of the inverse's passes, in its order
+    unsigned mg[kLineMaxPass], mgi[kLineMaxPass];   // ceil(2^32 / span)
+};
+
+// b mod Ns for b < 4096 with mg = ceil(2^32 / Ns): b mg / 2^32 is exact for b Ns < 2^32
+__device__ __forceinline__ int line_mod(int b, int Ns, unsigned mg) {
+    return Ns == 1 ? 0 : b - (int)__umulhi((unsigned)b, mg) * Ns;
+}
+
+// one slot of padding every eight elements spreads the strided writes of the
+// first passes over the banks
+__host__ __device__ __forceinline__ int line_place(int e) { return e + (e >> 3); }
+__host__ __device__ __forceinline__ int line_len(int L) { return L + (L >> 3) + 1; }
+
+// x = a + w b, y = a - w b
+template <typename C> __device__ __forceinline__ void bf2(C& a, C& b, C w) {
+    using T = decltype(C::x);
+    const C x = mk<C>(fma(w.x, b.x, fma(-w.y, b.y, a.x)), fma(w.x, b.y, fma(w.y, b.x, a.y)));
+    b = mk<C>(fma((T)2, a.x, -x.x), fma((T)2, a.y, -x.y));
+    a = x;
+}
+// the same with w replaced by DIR i w
+template <int DIR, typename C> __device__ __forceinline__ void bf2i(C& a, C& b, C w) { bf2(a, b, mul_i<DIR>(w)); }
+
+// DFT of R values, no twiddles; HALF: the upper half of the inputs is zero
+template <int DIR, int R, bool HALF, typename C> __device__ __forceinline__ void line_dft(C (&x)[R]) {
+    if constexpr (R == 2) {
+        if constexpr (HALF) x[1] = x[0]; else dft2<DIR>(x[0], x[1]);
+    } else if constexpr (R == 3) {
+        dft3<DIR>(x[0], x[1], x[2]);
+    } else if constexpr (R == 4) {
+        if constexpr (HALF) {
+            const C a = x[0], b = x[1], ib = mul_i<DIR>(b);
+            x[0] = cadd(a, b); x[2] = csub(a, b); x[1] = cadd(a, ib); x[3] = csub(a, ib);
+        } else {
+            dft4<DIR>(x[0], x[1], x[2], x[3]);
+        }
+    } else if constexpr (R == 5) {
+        dft5<DIR>(x[0], x[1], x[2], x[3], x[4]);
+    } else if constexpr (R == 6) {
+        if constexpr (HALF) x[3] = x[4] = x[5] = mk<C>(0, 0);
+        dft6<DIR>(x);
+    } else if constexpr (R == 7) {
+        dft7<DIR>(x);
+    } else if constexpr (R == 12) {
+        if constexpr (HALF) {
+#pragma unroll
+            for (int q = 6; q < 12; ++q) x[q] = mk<C>(0, 0);
+        }
+        dft12<DIR>(x);
+    } else if constexpr (R == 16) {
+        dft16<DIR, HALF>(x);
+    } else {
+        static_assert(R == 8, "no such radix");
+        if constexpr (HALF) dft8_half<DIR>(x); else dft8<DIR>(x);
+    }
+}
+
+// one butterfly of the three components: twiddles (none for span 1), then the DFT
+template <typename T, int DIR, int R>
+__device__ __forceinline__ void line_butterfly(typename Cplx<T>::type (&x)[3][R], const typename Cplx<T>::type* tw,
+                                               int k, int step, int L) {
+    using C = typename Cplx<T>::type;
+    auto W = [&](int m) {
+        C w = __ldg(tw + m);
+        if (DIR > 0) w.y = -w.y;
+        return w;
+    };
+    if constexpr (R == 2) {
+        const C w = W(k * step);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) bf2(x[c][0], x[c][1], w);
+    } else if constexpr (R == 4) {
+        const C w1 = W(k * step), w2 = W(2 * k * step);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            C* a = x[c];
+            bf2(a[0], a[2], w2);          // t0, t1
+            bf2(a[1], a[3], w2);          // t2, t3
+            bf2(a[0], a[1], w1);          // X0, X2
+            bf2i<DIR>(a[2], a[3], w1);    // X1, X3
+            const C x1 = a[2];
+            a[2] = a[1]; a[1] = x1;
+        }
+    } else if constexpr (R == 8) {
+        // W_8 w1 = W_L^(k step + L/8)
+        const C w1 = W(k * step), w2 = W(2 * k * step), w4 = W(4 * k * step), u = W(k * step + L / 8);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            C* a = x[c];
+            bf2(a[0], a[4], w4); bf2(a[2], a[6], w4);
+            bf2(a[0], a[2], w2); bf2i<DIR>(a[4], a[6], w2);     // E0 E2 | E1 E3 in a0 a2 a4 a6
+            bf2(a[1], a[5], w4); bf2(a[3], a[7], w4);
+            bf2(a[1], a[3], w2); bf2i<DIR>(a[5], a[7], w2);     // O0 O2 | O1 O3 in a1 a3 a5 a7
+            bf2(a[0], a[1], w1);            // X0, X4
+            bf2(a[4], a[5], u);             // X1, X5
+            bf2i<DIR>(a[2], a[3], w1);      // X2, X6
+            bf2i<DIR>(a[6], a[7], u);       // X3, X7
+            const C x4 = a[1], x1 = a[4], x6 = a[3], x3 = a[6];
+            a[1] = x1; a[3] = x3; a[4] = x4; a[6] = x6;
+        }
+    } else {
+#pragma unroll
+        for (int q = 1; q < R; ++q) {
+            const C w = W(q * k * step);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) x[c][q] = cmul(x[c][q], w);
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) line_dft<DIR, R, false>(x[c]);
+    }
+}
+
+template <typename C, int R>
+__device__ __forceinline__ void line_load(C (&x)[3][R], const C* s, int plane, int lb, int b, int M) {
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+        const C* p = s + (line_place(b + q * M) << lb);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) x[c][q] = p[c * plane];
+    }
+}
+template <typename C, int R>
+__device__ __forceinline__ void line_store(const C (&x)[3][R], C* s, int plane, int lb, int b, int k, int Ns) {
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+        C* p = s + (line_place((b - k) * R + k + q * Ns) << lb);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) p[c * plane] = x[c][q];
+    }
+}
+
+// a pass between two others, in place; s is the thread's line.  Every thread of
+// the CTA calls it.
+template <typename T, int DIR, int R>
+__device__ __forceinline__ void line_mid(typename Cplx<T>::type* s, int plane, int lb, int b, int L, int Ns,
+                                         unsigned mg, const typename Cplx<T>::type* tw) {
+    using C = typename Cplx<T>::type;
+    const int M = L / R;
+    // threads without a butterfly compute the first one and store nothing: values
+    // set under a condition would stay live around the loop over passes and spill
+    const bool on = b < M;
+    if (!on) b = 0;
+    C x[3][R];
+    const int k = line_mod(b, Ns, mg);
+    line_load<C, R>(x, s, plane, lb, b, M);
+    line_butterfly<T, DIR, R>(x, tw, k, L / (Ns * R), L);
+    __syncthreads();
+    if (on) line_store<C, R>(x, s, plane, lb, b, k, Ns);
+    __syncthreads();
+}
+
+// CALL with R_ = the radix; the FP64 plans hold none above 7 and no 6
+#define MM_LINE_RADIX(Tv, Rv, CALL)                                       \
+    switch (Rv) {                                                         \
+        case 2: { constexpr int R_ = 2; CALL; } break;                     \
+        case 3: { constexpr int R_ = 3; CALL; } break;                     \
+        case 4: { constexpr int R_ = 4; CALL; } break;                     \
+        case 5: { constexpr int R_ = 5; CALL; } break;                     \
+        case 7: { constexpr int R_ = 7; CALL; } break;                     \
+        case 6: { constexpr int R_ = sizeof(Tv) == 4 ? 6 : 2; CALL; } break; \
+        default: { constexpr int R_ = sizeof(Tv) == 4 ? 8 : 2; CALL; } break; \
+    }
+#define MM_LINE_RADIX_EVEN(Tv, Rv, CALL)                                  \
+    switch (Rv) {                                                         \
+        case 2: { constexpr int R_ = 2; CALL; } break;                     \
+        case 4: { constexpr int R_ = 4; CALL; } break;                     \
+        case 6: { constexpr int R_ = sizeof(Tv) == 4 ? 6 : 2; CALL; } break; \
+        default: { constexpr int R_ = sizeof(Tv) == 4 ? 8 : 2; CALL; } break; \
+    }
+
+template <typename T, int DIR>
+__device__ __forceinline__ void line_mid_any(typename Cplx<T>::type* s, int plane, int lb, int b, const LinePlan& pl,
+                                             int i, const typename Cplx<T>::type* tw) {
+    const int R = DIR < 0 ? pl.R[i] : pl.R[pl.np - 1 - i];
+    const int Ns = DIR < 0 ? pl.Ns[i] : pl.Nsi[i];
+    const unsigned mg = DIR < 0 ? pl.mg[i] : pl.mgi[i];
+    MM_LINE_RADIX(T, R, (line_mid<T, DIR, R_>(s, plane, lb, b, pl.L, Ns, mg, tw)));
+}
+
+}  // namespace mm

@@ -1,0 +1,64 @@
+"""The line engine's passes (any even 7-smooth length, radix plan at run time)
+at the edges of their range, against the oracle's convolution: z lines held in
+one thread (up to 16 points), every radix first and last in a plan, y lines of
+a 2-D grid up to the longest single pass and just beyond it, a last group of
+columns that is nearly empty, lines too long for the engine, and a batch of
+grids.  Tolerances are those of the demag tests: FP32 1e-5 of the largest
+field, FP64 the oracle's own rounding sensitivity but at least 1e-10."""
+import numpy as np
+import pytest
+
+from gpu_util import FP32_TOL, rel, to_host
+
+pytestmark = pytest.mark.gpu
+
+D = (2e-9, 3e-9, 2.5e-9)
+GRIDS = [(9, 8, 2), (9, 8, 3), (17, 6, 4), (33, 7, 6), (10, 12, 8), (5, 3, 49), (6, 4, 35), (7, 5, 63), (8, 9, 27),
+         (3, 245, 1), (20, 257, 1), (5, 512, 1), (6, 525, 1), (2, 3, 1024), (1, 2, 700)]
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("n", GRIDS)
+def test_lines_match_oracle(n, precision):
+    from oracle.demag import demag_fft, magnetization, rounding_sensitivity
+    from oracle.newell import demag_tensor
+    from paper_2302_08843_gb300.binding import State
+    from paper_2302_08843_gb300.workloads import from_soa, to_soa
+    rng = np.random.default_rng(sum(n))
+    m = rng.normal(size=n + (3,))
+    m /= np.linalg.norm(m, axis=-1, keepdims=True)
+    s = State(n, D, precision)
+    s.set_material(Ms=8e5, A=0.0, alpha=0.1)
+    s.demag_setup(20)
+    h = from_soa(to_host(s.heff(m=to_soa(m))))
+    s.close()
+    M = magnetization(m, 8e5)
+    tol = FP32_TOL if precision == "fp32" else max(1e-10, rounding_sensitivity(n, D, 20, M))
+    assert rel(h, demag_fft(demag_tensor(n, D, 20), M)) < tol
+
+
+@pytest.mark.parametrize("n", [(11, 9, 1), (6, 7, 8), (5, 30, 3)])
+def test_batch_lines_match_single_grids(n):
+    """One tiny step of three slots (FP64) against one DP45 step of each alone."""
+    from paper_2302_08843_gb300.binding import Batch, State
+    from paper_2302_08843_gb300.workloads import to_soa
+    rng = np.random.default_rng(5)
+    b = Batch(n, D, "fp64", capacity=4)
+    states = []
+    for slot in (0, 1, 3):
+        m = rng.normal(size=n + (3,))
+        m /= np.linalg.norm(m, axis=-1, keepdims=True)
+        b.set_slot(slot, 7e5 + 1e5 * slot, 1.2e-11, 1.0, to_soa(m), 1e-15)
+        s = State(n, D, "fp64")
+        s.set_material(Ms=7e5 + 1e5 * slot, A=1.2e-11, alpha=1.0)
+        s.demag_setup(20)
+        s.set_m(to_soa(m))
+        s.step(1e-15, 0.0, "dp45", 1e-5)
+        states.append((slot, to_host(s.get_m())))
+        s.close()
+    b.begin(1, 1e-5, 1e-9, 10)
+    st, steps, _ = b.end()
+    for slot, m in states:
+        assert st[slot] == 1 and steps[slot] == 1
+        assert rel(b.get_m(slot), m) < 1e-13
+    b.close()
