@@ -178,7 +178,8 @@ bool fused_stage_supported(const DemagDims& d, const StageParams<float>& p);
 // fill kcT, ckT, dtT, acc_bT and the uniform-material constants from the double fields
 template <typename T> void stage_prepare(StageParams<T>& p);
 template <typename T> int stage_blocks(int nx, int ny, int nz);   // blocks launch_stage will use
-void launch_finalize(const double* partials, int nblocks, double* scalars, cudaStream_t st);
+// host_out: pinned host memory, kNPart scalars and the device error word
+void launch_finalize(const double* partials, int nblocks, const int* dev_err, double* host_out, cudaStream_t st);
 template <typename T> void launch_convert(const double* src, T* dst, long n, cudaStream_t st);
 template <typename T> void launch_renorm_copy(const T* src, T* dst, long N, cudaStream_t st);
 template <typename T> void launch_combine(const T* mn, const T* const* kin, const double* kc, int nk, double dt,
