@@ -19,7 +19,7 @@ LIB = os.path.join(HERE, "libmm.so")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 CU_UNITS = ["mm_api.cu", "demag_passes.cu", "demag_rt.cu", "llg_kernels.cu", "noalloc.cu", "adjoint.cu", "batch.cu",
-            "diag.cu"]
+            "diag.cu", "line_ct0.cu", "line_ct1.cu", "line_ct2.cu", "line_ct3.cu"]
 CPP_UNITS = ["tensor_host.cpp"]
 
 
@@ -61,7 +61,7 @@ def build(verbose=False, force=False, extra_flags=()):
         if force or _stale(obj, [src] + headers):
             jobs.append(["g++", "-c", src, "-o", obj, "-O3", "-std=c++17", "-fPIC", "-fopenmp",
                          "-ffp-contract=off", "-I" + SRC, "-I" + os.path.join(ROOT, "include")])
-    with concurrent.futures.ThreadPoolExecutor(max_workers=max(1, min(8, os.cpu_count() or 1))) as ex:
+    with concurrent.futures.ThreadPoolExecutor(max_workers=max(1, min(16, os.cpu_count() or 1))) as ex:
         outs = list(ex.map(_run, jobs))
     if verbose:
         for o in outs:

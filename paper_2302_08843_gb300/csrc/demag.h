@@ -93,6 +93,23 @@ void launch_rt_y(const DemagDims& d, const typename Cplx<T>::type* in, typename 
                  cudaStream_t st);
 template <typename T>
 void launch_rt_z(const DemagDims& d, typename Cplx<T>::type* S2, const T* tens, cudaStream_t st);
+// input of the x-forward: Ms m, or Ms y with y = m + ca k (ca = dt_b[grid] a for
+// a batch), which is stored too; mask: the grids to work on
+template <typename T> struct LineXIn {
+    const T* m = nullptr;
+    const T* Ms_cell = nullptr;
+    T Ms = 0;
+    const T* k = nullptr;
+    T* y = nullptr;
+    T ca = 0;
+    const double* dt_b = nullptr;
+    double a = 0;
+    const int* mask = nullptr;
+};
+template <typename T>
+bool launch_line_x_fwd(const DemagDims& d, const LineXIn<T>& in, typename Cplx<T>::type* S1, cudaStream_t st);
+template <typename T>
+bool launch_line_x_inv(const DemagDims& d, const typename Cplx<T>::type* S1, T* h, cudaStream_t st);
 // the line engine's passes (demag_rt.cu), any length; false if a line is too long for them
 template <typename T, int DIR>
 bool launch_line_y(const DemagDims& d, const typename Cplx<T>::type* in, typename Cplx<T>::type* out,
@@ -170,6 +187,24 @@ struct StageParams {
     T cex_u, cani_u, gp_u;       // 2/(mu0 Ms), 2 Ku/(mu0 Ms), -gamma/(1+alpha^2) for uniform material
 };
 
+// Per-grid quantities of a batch; mask null: one grid, everything in StageParams.
+struct LineBatch {
+    const int* mask;
+    const float *Ms, *A, *alpha, *D, *pc;
+    const int* kind;
+    const double* dt;
+    float dmi_e[4][9];
+    double* partials;      // [grid][CTAs per grid][3]: torque, error, non-finite
+};
+
+// x-inverse + stage + (fwd) x-forward of the next stage input on the line
+// engine: FP32, every term and output of StageParams (p prepared, p.hd unused)
+// and batches (bt).  gen: the variant with maps, layers, DMI, energies and cells
+// without magnetisation.  CTAs per grid (the partials' blocks): 0 if a line is
+// too long or too short for it.
+int line_fused_blocks(const DemagDims& d, long max_ctas);
+bool launch_line_fused(const DemagDims& d, float2* S1, const StageParams<float>& p, const LineBatch* bt, bool gen,
+                       bool fwd, long max_ctas, cudaStream_t st);
 template <typename T> void launch_stage(const StageParams<T>& p, cudaStream_t st, int* nblocks);
 // fused x-inverse + stage + x-forward of the next stage input (FP32, uniform material, RK stages);
 // the coefficients in the field type (kcT, ckT, dtT, acc_bT) and the uniform constants must be filled

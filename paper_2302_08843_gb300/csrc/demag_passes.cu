@@ -2026,7 +2026,12 @@ template <typename T, int L> static void launch_x_fwd(const DemagDims& d, const 
     if constexpr (sizeof(T) == 4 && L >= 16 && is_pow2(L)) {
         if (launch_p1_tma<L>(d, m, Ms_cell, Ms, S1, st)) return;
     }
-    launch_p1<T, L>(d, m, Ms_cell, Ms, S1, st);
+    LineXIn<T> in;
+    in.m = m;
+    in.Ms_cell = Ms_cell;
+    in.Ms = Ms;
+    if (launch_line_x_fwd<T>(d, in, S1, st)) return;
+    if constexpr (L < 16 || L >= 2048) launch_p1<T, L>(d, m, Ms_cell, Ms, S1, st);   // too short or long for the engine
 }
 
 template <typename T, int L> static void launch_x_inv(const DemagDims& d, const typename Cplx<T>::type* S1, T* h,
@@ -2034,7 +2039,8 @@ template <typename T, int L> static void launch_x_inv(const DemagDims& d, const 
     if constexpr (sizeof(T) == 4 && L >= 16 && is_pow2(L)) {
         if (launch_p5_tma<L>(d, S1, h, st)) return;
     }
-    launch_p5<T, L>(d, S1, h, st);
+    if (launch_line_x_inv<T>(d, S1, h, st)) return;
+    if constexpr (L < 16 || L >= 2048) launch_p5<T, L>(d, S1, h, st);
 }
 
 // fused K5 launcher (see k5_fused): false if the shape or material does not qualify

@@ -21,7 +21,7 @@
 #include <vector>
 
 #include "demag.h"
-#include "line_engine.cuh"
+#include "line_kernels.cuh"
 #include "tensor_host.h"
 #include "tma.cuh"
 
@@ -62,62 +62,26 @@ const RtTable& rt_table() {
     return t;
 }
 
-// the factors of L for the line engine, as few as radices up to rmax (and 3, 5,
-// 7) allow and among those the largest smallest one: factors of `L` from
-// `radix[at]` on, appended to cur
-void line_factors(int L, int rmax, int at, std::vector<int>& cur, std::vector<int>& best) {
-    static const int radix[7] = {8, 7, 6, 5, 4, 3, 2};
-    if (L == 1) {
-        if (best.empty() || cur.size() < best.size() || (cur.size() == best.size() && cur.back() > best.back()))
-            best = cur;
-        return;
-    }
-    if (!best.empty() && cur.size() >= best.size()) return;
-    for (int i = at; i < 7; ++i) {
-        const int r = radix[i];
-        if (L % r || (r > rmax && r % 2 == 0)) continue;
-        cur.push_back(r);
-        line_factors(L / r, rmax, i, cur, best);
-        cur.pop_back();
-    }
-}
-
-// The line engine's plan of a length in the table (or 1): an even radix first,
-// the largest of the others last.  one: a single pass of radix L.
-LinePlan line_plan(int L, int rmax, bool one) {
-    LinePlan p{};
-    p.L = L;
-    if (L == 1) {
-        p.np = p.rmin = p.R[0] = p.Ns[0] = p.Nsi[0] = 1;
-        return p;
-    }
-    if (one) {
-        p.np = 1;
-        p.rmin = p.R[0] = (short)L;
-        return p;
-    }
-    std::vector<int> cur, f;
-    line_factors(L, rmax, 0, cur, f);
-    if (f.empty() || (int)f.size() > kLineMaxPass) return p;      // np = 0: not a length of the engine
-    p.np = (int)f.size();
-    p.rmin = f.back();
-    size_t first = 0;
-    while (f[first] % 2) ++first;      // factors come largest first; L is even
-    p.R[0] = (short)f[first];
-    f.erase(f.begin() + first);
-    for (int i = 1; i < p.np; ++i) p.R[i] = (short)f[p.np - 1 - i];
-    for (int i = 0, a = 1, b = 1; i < p.np; ++i) {
-        p.Ns[i] = (short)a;
-        p.Nsi[i] = (short)b;
-        p.mg[i] = (unsigned)(((1ull << 32) + a - 1) / a);
-        p.mgi[i] = (unsigned)(((1ull << 32) + b - 1) / b);
-        a *= p.R[i];
-        b *= p.R[p.np - 1 - i];
-    }
+// offset of W_L^m in the table, -1 for a length that is not in it
+int rt_offset(int L) {
     const RtTable& t = rt_table();
     const auto it = std::lower_bound(t.lengths.begin(), t.lengths.end(), L);
-    if (it == t.lengths.end() || *it != L) p.np = 0;
-    else p.tw = t.offsets[it - t.lengths.begin()];
+    return it == t.lengths.end() || *it != L ? -1 : t.offsets[it - t.lengths.begin()];
+}
+
+// the engine's plan of a length; one: a single pass of radix L
+LinePlan host_plan(int L, int rmax, bool one) {
+    LinePlan p{};
+    if (one) {
+        p.L = L;
+        p.np = 1;
+        p.rmin = p.R[0] = (short)L;
+        p.Ns[0] = p.Nsi[0] = 1;
+        return p;
+    }
+    p = line_plan(L, rmax);
+    p.tw = rt_offset(L);
+    if (p.tw < 0) p.np = 0;
     return p;
 }
 
@@ -128,6 +92,17 @@ LinePlan line_plan(int L, int rmax, bool one) {
 constexpr int kTwRt = 173884;
 static __device__ double2 g_twrt64[kTwRt];
 static __device__ float2 g_twrt32[kTwRt];
+
+// device addresses of the tables, per device (set by the upload)
+constexpr int kMaxDevices = 128;
+static const double2* g_tab64[kMaxDevices];
+static const float2* g_tab32[kMaxDevices];
+template <typename T> const typename Cplx<T>::type* line_table(const LinePlan& pl) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if constexpr (sizeof(T) == 4) return g_tab32[dev] + pl.tw;
+    else return g_tab64[dev] + pl.tw;
+}
 
 template <typename T> struct TwRt;
 template <> struct TwRt<float> {
@@ -190,6 +165,16 @@ cudaError_t upload_twiddles_rt() {
     }
     cudaError_t e = cudaMemcpyToSymbol(g_twrt64, h64.data(), sizeof(double2) * kTwRt);
     if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_twrt32, h32.data(), sizeof(float2) * kTwRt);
+    int dev = 0;
+    void *p64 = nullptr, *p32 = nullptr;
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess && (dev < 0 || dev >= kMaxDevices)) e = cudaErrorInvalidDevice;
+    if (e == cudaSuccess) e = cudaGetSymbolAddress(&p64, g_twrt64);
+    if (e == cudaSuccess) e = cudaGetSymbolAddress(&p32, g_twrt32);
+    if (e == cudaSuccess) {
+        g_tab64[dev] = static_cast<const double2*>(p64);
+        g_tab32[dev] = static_cast<const float2*>(p32);
+    }
     return e;
 }
 
@@ -445,243 +430,6 @@ rt_z_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restr
         }
 }
 
-// ---------------------------------------------------- y passes, z pass ----
-// Line engine (line_engine.cuh): a CTA takes 2^lb columns, one thread per
-// butterfly of a column, all three components.
-template <typename T> struct LineTab;
-template <> struct LineTab<float> {
-    static __device__ __forceinline__ const float2* get() { return g_twrt32; }
-};
-template <> struct LineTab<double> {
-    static __device__ __forceinline__ const double2* get() { return g_twrt64; }
-};
-// threads of a CTA at most.  FP32 passes wait on memory: three CTAs of 256
-// threads per SM (85 registers); the 512-thread variant takes the lines with
-// more butterflies.
-constexpr int kLineThreads = 512, kLineThreads32 = 256;
-template <typename T, int MAXT> constexpr int line_blocks() { return sizeof(T) == 4 && MAXT == kLineThreads32 ? 3 : 1; }
-
-__device__ __forceinline__ void cp_async(float* dst, const float* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async(double* dst, const double* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-// first pass of a transform along a strided line: elements b + q M straight
-// from global memory (at g[e es + c cs]; e < n, the rest zero)
-template <typename T, int DIR, int R, bool HALF>
-__device__ __forceinline__ void line_first(const typename Cplx<T>::type* g, long es, long cs, int n,
-                                           typename Cplx<T>::type* s, int plane, int lb, int b, int L) {
-    using C = typename Cplx<T>::type;
-    const int M = L / R;
-    if (b >= M) return;
-    C x[3][R];
-#pragma unroll
-    for (int q = 0; q < (HALF ? R / 2 : R); ++q) {
-        const int e = b + q * M;
-        const bool in = !HALF || e < n;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) x[c][q] = in ? g[c * cs + e * es] : mk<C>(0, 0);
-    }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) line_dft<DIR, R, HALF>(x[c]);
-    line_store<C, R>(x, s, plane, lb, b, 0, 1);
-}
-
-// last pass: outputs b + q M to global memory; HALF: only e < n
-template <typename T, int DIR, int R, bool HALF>
-__device__ __forceinline__ void line_last(const typename Cplx<T>::type* s, int plane, int lb, int b, int L, int Ns,
-                                          unsigned mg, const typename Cplx<T>::type* tw,
-                                          typename Cplx<T>::type* g, long es, long cs, int n, bool valid) {
-    using C = typename Cplx<T>::type;
-    const int M = L / R;
-    if (b >= M) return;
-    C x[3][R];
-    line_load<C, R>(x, s, plane, lb, b, M);
-    line_butterfly<T, DIR, R>(x, tw, line_mod(b, Ns, mg), L / (Ns * R), L);
-#pragma unroll
-    for (int q = 0; q < (HALF ? R / 2 : R); ++q) {
-        const int e = b + q * M;
-        if (valid && (!HALF || e < n)) {
-#pragma unroll
-            for (int c = 0; c < 3; ++c) g[c * cs + e * es] = x[c][q];
-        }
-    }
-}
-
-// h^ = T M^ at the R wave numbers b + q M of one column; tp points at the
-// column's folded ky row, tz between kz planes, tc between components
-template <typename T, int R>
-__device__ __forceinline__ void line_tensor(typename Cplx<T>::type (&x)[3][R], const T* __restrict__ tp, long tz,
-                                            long tc, int b, int M, int L, T sy, int swap) {
-    using C = typename Cplx<T>::type;
-#pragma unroll
-    for (int q = 0; q < R; ++q) {
-        const int kz = b + q * M;
-        const bool up = 2 * kz > L;
-        const T* t = tp + (up ? L - kz : kz) * tz;
-        const T sz = up ? (T)-1 : (T)1;
-        const T txx = t[0], tyy = t[3 * tc], tzz = t[5 * tc];
-        const T txy = (swap ? sz : sy) * t[tc], txz = (swap ? sy : sz) * t[2 * tc];
-        const T tyz = sy * sz * t[4 * tc];
-        const C mx = x[0][q], my = x[1][q], mz = x[2][q];
-        x[0][q] = mk<C>(txx * mx.x + txy * my.x + txz * mz.x, txx * mx.y + txy * my.y + txz * mz.y);
-        x[1][q] = mk<C>(txy * mx.x + tyy * my.x + tyz * mz.x, txy * mx.y + tyy * my.y + tyz * mz.y);
-        x[2][q] = mk<C>(txz * mx.x + tyz * my.x + tzz * mz.x, txz * mx.y + tyz * my.y + tzz * mz.y);
-    }
-}
-
-// the forward's last pass, the tensor product and the inverse's first pass
-template <typename T, int R>
-__device__ __forceinline__ void line_product(typename Cplx<T>::type* s, int plane, int lb, int b, int L, int Ns,
-                                             unsigned mg, const typename Cplx<T>::type* tw, const T* tp, int tz,
-                                             int tc, T sy, int swap) {
-    using C = typename Cplx<T>::type;
-    const int M = L / R;
-    const bool on = b < M;
-    if (!on) b = 0;
-    C x[3][R];
-    line_load<C, R>(x, s, plane, lb, b, M);
-    line_butterfly<T, -1, R>(x, tw, line_mod(b, Ns, mg), L / (Ns * R), L);
-    line_tensor<T, R>(x, tp, tz, tc, b, M, L, sy, swap);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) line_dft<+1, R, false>(x[c]);
-    __syncthreads();
-    if (on) line_store<C, R>(x, s, plane, lb, b, 0, 1);
-    __syncthreads();
-}
-
-// the whole column in one thread's registers (L = R)
-template <typename T, int R>
-__device__ __forceinline__ void line_product_one(typename Cplx<T>::type* g, long es, long cs, int n, const T* tp,
-                                                 long tz, long tc, T sy, int swap) {
-    using C = typename Cplx<T>::type;
-    constexpr int H = R == 1 ? 1 : R / 2;
-    C x[3][R];
-#pragma unroll
-    for (int q = 0; q < H; ++q)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) x[c][q] = q < n ? g[c * cs + q * es] : mk<C>(0, 0);
-    if constexpr (R > 1) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) line_dft<-1, R, true>(x[c]);
-    }
-    line_tensor<T, R>(x, tp, tz, tc, 0, 1, R, sy, swap);
-    if constexpr (R > 1) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) line_dft<+1, R, false>(x[c]);
-    }
-#pragma unroll
-    for (int q = 0; q < H; ++q)
-        if (q < n) {
-#pragma unroll
-            for (int c = 0; c < 3; ++c) g[c * cs + q * es] = x[c][q];
-        }
-}
-
-// z pass: per (kx, ky) column z-forward (z < nz, the rest zero), h^ = T M^ with
-// the octant-folded real tensor (sign flips of the odd components from the
-// parity of ky and kz, or of the transformed axis on 2-D grids), z-inverse,
-// keep z < nz; in place.  Columns are numbered kx-fastest over (ky, kx <= Px/2);
-// blockIdx.y is the grid of a batch.
-// The column's tensor slice is copied to shared memory while the forward passes run.
-template <typename T, bool ONE, int MAXT>
-__global__ void __launch_bounds__(MAXT, line_blocks<T, MAXT>())
-line_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restrict__ tens,
-          const __grid_constant__ LinePlan pl, int lb, int ncol, int early) {
-    using C = typename Cplx<T>::type;
-    extern __shared__ __align__(16) unsigned char smraw[];
-    const int L = pl.L, tid = threadIdx.x;
-    const int l = tid & ((1 << lb) - 1), b = tid >> lb;
-    const int col = (blockIdx.x << lb) + l;
-    const bool valid = col < ncol;
-    const int cc = valid ? col : ncol - 1;      // columns past the end follow the last one and store nothing
-    const int ky = cc / d.KX, kx = cc - ky * d.KX;
-    const int LY = d.LY, KY2 = LY / 2 + 1;
-    const bool up = 2 * ky > LY;
-    const long zs = (long)LY * d.KXS, cs = (long)d.nz * zs;
-    C* g = S2 + (long)blockIdx.y * 3 * cs + (long)ky * d.KXS + kx;
-    const long tz = (long)KY2 * d.KXS, tc = (long)(L / 2 + 1) * tz;
-    const T* tp = tens + (long)(up ? LY - ky : ky) * d.KXS + kx;
-    const T sy = up ? (T)-1 : (T)1;
-    if (early) grid_dep_launch();
-    grid_dep_wait();
-    if constexpr (ONE) {
-        if (!valid) return;
-        switch (L) {
-            case 1: line_product_one<T, 1>(g, zs, cs, d.nz, tp, tz, tc, sy, d.yz_swap); break;
-            case 2: line_product_one<T, 2>(g, zs, cs, d.nz, tp, tz, tc, sy, d.yz_swap); break;
-            case 4: line_product_one<T, 4>(g, zs, cs, d.nz, tp, tz, tc, sy, d.yz_swap); break;
-            case 6: line_product_one<T, sizeof(T) == 4 ? 6 : 1>(g, zs, cs, d.nz, tp, tz, tc, sy, d.yz_swap); break;
-            case 8: line_product_one<T, sizeof(T) == 4 ? 8 : 1>(g, zs, cs, d.nz, tp, tz, tc, sy, d.yz_swap); break;
-            case 12: line_product_one<T, sizeof(T) == 4 ? 12 : 1>(g, zs, cs, d.nz, tp, tz, tc, sy, d.yz_swap); break;
-            default: line_product_one<T, sizeof(T) == 4 ? 16 : 1>(g, zs, cs, d.nz, tp, tz, tc, sy, d.yz_swap); break;
-        }
-    } else {
-        C* s = reinterpret_cast<C*>(smraw) + l;
-        const int plane = line_len(L) << lb;
-        const C* tw = LineTab<T>::get() + pl.tw;
-        const int KZ2 = L / 2 + 1, B = 1 << lb;
-        T* ts = reinterpret_cast<T*>(reinterpret_cast<C*>(smraw) + 3 * plane) + l;     // [6][KZ2][B]
-        for (int c = 0; c < 6; ++c)
-            for (int k = b; k < KZ2; k += blockDim.x >> lb)
-                cp_async(ts + (c * KZ2 + k) * B, tp + c * tc + k * tz);
-        MM_LINE_RADIX_EVEN(T, pl.R[0], (line_first<T, -1, R_, true>(g, zs, cs, d.nz, s, plane, lb, b, L)));
-        __syncthreads();
-        const int np = pl.np;
-        for (int i = 1; i < np - 1; ++i) line_mid_any<T, -1>(s, plane, lb, b, pl, i, tw);
-        cp_async_wait_all();
-        __syncthreads();
-        MM_LINE_RADIX(T, pl.R[np - 1], (line_product<T, R_>(s, plane, lb, b, L, pl.Ns[np - 1], pl.mg[np - 1], tw, ts,
-                                                            B, KZ2 << lb, sy, d.yz_swap)));
-        for (int i = 1; i < np - 1; ++i) line_mid_any<T, +1>(s, plane, lb, b, pl, i, tw);
-        MM_LINE_RADIX_EVEN(T, pl.R[0], (line_last<T, +1, R_, true>(s, plane, lb, b, L, pl.Nsi[np - 1], pl.mgi[np - 1], tw,
-                                                                g, zs, cs, d.nz, valid)));
-    }
-}
-
-// y passes.  DIR = -1: S1 (ny rows) -> S2 (Py rows), forward, zero upper half;
-// DIR = +1: S2 -> S1, keep y < ny.  Columns kx-fastest over (z, kx <= Px/2).
-template <typename T, int DIR, int MAXT>
-__global__ void __launch_bounds__(MAXT, line_blocks<T, MAXT>())
-line_y(DemagDims d, const typename Cplx<T>::type* __restrict__ in, typename Cplx<T>::type* __restrict__ out,
-       const __grid_constant__ LinePlan pl, int lb, int ncol, int early) {
-    using C = typename Cplx<T>::type;
-    extern __shared__ __align__(16) unsigned char smraw[];
-    const int L = pl.L, tid = threadIdx.x;
-    const int l = tid & ((1 << lb) - 1), b = tid >> lb;
-    const int col = (blockIdx.x << lb) + l;
-    const bool valid = col < ncol;
-    const int cc = valid ? col : ncol - 1;
-    const int z = cc / d.KX, kx = cc - z * d.KX;
-    const int rin = DIR < 0 ? d.ny : L, rout = DIR < 0 ? L : d.ny;
-    const long cin = (long)d.nz * rin * d.KXS, cout = (long)d.nz * rout * d.KXS;
-    const C* gi = in + (long)blockIdx.y * 3 * cin + (long)z * rin * d.KXS + kx;
-    C* go = out + (long)blockIdx.y * 3 * cout + (long)z * rout * d.KXS + kx;
-    if (early) grid_dep_launch();
-    grid_dep_wait();
-    C* s = reinterpret_cast<C*>(smraw) + l;
-    const int plane = line_len(L) << lb;
-    const C* tw = LineTab<T>::get() + pl.tw;
-    const int np = pl.np;
-    if constexpr (DIR < 0) {
-        MM_LINE_RADIX_EVEN(T, pl.R[0], (line_first<T, -1, R_, true>(gi, d.KXS, cin, d.ny, s, plane, lb, b, L)));
-    } else {
-        MM_LINE_RADIX(T, pl.R[np - 1], (line_first<T, +1, R_, false>(gi, d.KXS, cin, L, s, plane, lb, b, L)));
-    }
-    __syncthreads();
-    for (int i = 1; i < np - 1; ++i) line_mid_any<T, DIR>(s, plane, lb, b, pl, i, tw);
-    if constexpr (DIR < 0) {
-        MM_LINE_RADIX(T, pl.R[np - 1], (line_last<T, -1, R_, false>(s, plane, lb, b, L, pl.Ns[np - 1], pl.mg[np - 1], tw,
-                                                                 go, d.KXS, cout, L, valid)));
-    } else {
-        MM_LINE_RADIX_EVEN(T, pl.R[0], (line_last<T, +1, R_, true>(s, plane, lb, b, L, pl.Nsi[np - 1], pl.mgi[np - 1], tw,
-                                                                go, d.KXS, cout, d.ny, valid)));
-    }
-}
-
 // ------------------------------------------------------------- launchers ----
 namespace {
 template <typename K> void rt_smem(K kernel, size_t bytes) {
@@ -699,6 +447,9 @@ int rt_lines(int L, size_t csz, int nbuf, int cap) {
 template <typename T>
 void launch_rt_x_fwd(const DemagDims& d, const T* m, const T* Ms_cell, T Ms, typename Cplx<T>::type* S1,
                      cudaStream_t st) {
+    LineXIn<T> in;
+    in.m = m; in.Ms_cell = Ms_cell; in.Ms = Ms;
+    if (launch_line_x_fwd<T>(d, in, S1, st)) return;
     using C = typename Cplx<T>::type;
     const RtPlan pl = make_plan(d.LX);
     const int NL = rt_lines(d.LX, sizeof(C), 2, kRtMaxLines);
@@ -711,6 +462,7 @@ void launch_rt_x_fwd(const DemagDims& d, const T* m, const T* Ms_cell, T Ms, typ
 
 template <typename T>
 void launch_rt_x_inv(const DemagDims& d, const typename Cplx<T>::type* S1, T* h, cudaStream_t st) {
+    if (launch_line_x_inv<T>(d, S1, h, st)) return;
     using C = typename Cplx<T>::type;
     const RtPlan pl = make_plan(d.LX);
     const int NL = rt_lines(d.LX, sizeof(C), 2, kRtMaxLines);
@@ -734,22 +486,23 @@ struct LineShape {
 
 // Radices are bounded by 8 (FP32, which shared-memory exchanges bound) or 4
 // (FP64, whose instructions bound it: small radices cost no more of them and
-// put more warps on them).  An FP64 launch that would leave quarter SMs idle
-// takes radix 2.  Then as many columns per CTA (at least one 32-byte sector of
+// put more warps on them).  An FP64 grid that would leave quarter SMs idle
+// takes radix 2; the grids of a batch do not count, so that a grid's rounding
+// does not depend on the others.  Then as many columns per CTA (at least one 32-byte sector of
 // each row) as leave two CTAs for every SM.
-template <typename T> bool line_shape(int L, long ncol, int nb, bool conv, LineShape* o) {
+template <typename T> bool line_shape(int L, long ncol, int nb, int nc, bool conv, LineShape* o) {
     constexpr int kSms = 152;
     constexpr int full = 128 / (2 * sizeof(T)), sector = 32 / (2 * sizeof(T));
     int rmax = sizeof(T) == 4 ? 8 : 4;
-    if (sizeof(T) == 8 && L > 2 && ncol * nb * (L / 4) < kSms * 128L) rmax = 2;
+    if (sizeof(T) == 8 && L > 2 && ncol * (L / 4) < kSms * 128L) rmax = 2;
     // FP32 z lines of up to 16 points stay in one thread's registers
     const bool one = conv && (L <= 2 || L == 4 || (sizeof(T) == 4 && (L == 6 || L == 8 || L == 12 || L == 16)));
-    o->pl = line_plan(L, rmax, one);
+    o->pl = host_plan(L, rmax, one);
     const int M = L / o->pl.rmin;
     if (o->pl.np < 1 || o->pl.np > kLineMaxPass) return false;
     int lb = 0;
     while ((1 << lb) < full) ++lb;
-    const size_t column = 2 * sizeof(T) * 3 * line_len(L) + (conv ? sizeof(T) * 6 * (L / 2 + 1) : 0);
+    const size_t column = 2 * sizeof(T) * nc * line_len(L);
     auto fits = [&](int q) { return ((long)M << q) <= kLineThreads && column << q <= 160 * 1024; };
     while (lb > 0 && (!fits(lb) || (M << lb) > 256)) --lb;
     while (lb > 0 && (2 << lb) > 2 * sector && (M << lb) > 32 && ((ncol + (1 << lb) - 1) >> lb) * nb < 2 * kSms) --lb;
@@ -779,17 +532,139 @@ void line_launch(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, 
     cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
+// the kernel of a compiled length in place of the run-time one, if there is one
+template <typename... KArgs> bool line_ct_use(LineKind kind, int L, void (**kernel)(KArgs...)) {
+    const void* k = line_ct_kernel0(kind, L);
+    if (!k) k = line_ct_kernel1(kind, L);
+    if (!k) k = line_ct_kernel2(kind, L);
+    if (!k) k = line_ct_kernel3(kind, L);
+    if (!k) return false;
+    *kernel = reinterpret_cast<void (*)(KArgs...)>(const_cast<void*>(k));
+    return true;
+}
+
 }  // namespace
+
+namespace {
+
+// A launch of the x passes: nt threads for each of a CTA's lines.
+struct LineXShape {
+    LinePlan pl;
+    int nt, lines, threads;
+    bool ct;             // a compiled length's kernel holds that many threads
+    size_t smem;
+    long ctas;
+};
+
+// As many lines per CTA (up to 256 threads) as leave two CTAs for every SM
+// (nb = 1 for the fused stage: its block partials must not depend on a batch's
+// other grids); never more CTAs than max_ctas for each grid.  nc: lines of a row
+// pair (3: the fused stage's components).  FP64 radices as in line_shape.
+template <typename T> bool line_x_shape(int L, long pairs, int nb, int nc, long max_ctas, LineXShape* o) {
+    constexpr int kSms = 152;
+    int rmax = line_rmax<T>();
+    if (sizeof(T) == 8 && pairs * (L / 4) < kSms * 128L) rmax = 2;
+    o->pl = host_plan(L, rmax, false);
+    if (o->pl.np < 2) return false;
+    o->nt = L / o->pl.rmin;
+    const int per = nc * o->nt, most = nc == 3 ? 1024 : kLineThreads;
+    // (the fused stage parks up to 6 float2 values for each x of a row pair besides)
+    const size_t one = 2 * sizeof(T) * nc * line_len(L) + (nc == 3 ? 6 * sizeof(float2) * (L / 2) : 0);
+    if (per > most || one > 200 * 1024) return false;
+    long lines = per >= 256 ? 1 : 256 / per;
+    while (lines > 1 && (lines * (long)one > 100 * 1024 || (pairs + lines - 1) / lines * nb < 2 * kSms)) --lines;
+    while ((pairs + lines - 1) / lines > max_ctas) ++lines;
+    if (lines * per > most || lines * (long)one > 200 * 1024) return false;
+    o->lines = (int)lines;
+    o->threads = (int)((lines * per + 31) / 32 * 32);
+    o->ct = o->threads <= (nc == 1 || per <= 256 ? 256 : (per + 31) / 32 * 32);
+    o->smem = lines * 2 * sizeof(T) * nc * line_len(L);
+    o->ctas = (pairs + lines - 1) / lines;
+    return true;
+}
+constexpr long kAnyCtas = 1L << 40;
+
+long line_x_pairs(const DemagDims& d) { return (3L * d.ny * d.nz + 1) / 2; }
+long line_fused_pairs(const DemagDims& d) { return (long)d.nz * ((d.ny + 1) / 2); }
+
+}  // namespace
+
+template <typename T>
+bool launch_line_x_fwd(const DemagDims& d, const LineXIn<T>& in, typename Cplx<T>::type* S1, cudaStream_t st) {
+    constexpr int NC = 1;
+    LineXShape o;
+    if (d.nb > 65535 || !line_x_shape<T>(d.LX, line_x_pairs(d), d.nb, 1, kAnyCtas, &o)) return false;
+    LineForward<T> f{in.m, in.Ms_cell, in.Ms, in.k, in.y, in.ca, in.dt_b, in.a, in.mask};
+    auto k = o.threads <= 256 ? line_x_forward<T, NC, 256, 0> : line_x_forward<T, NC, kLineThreads, 0>;
+    if constexpr (sizeof(T) == 4) {
+        if (o.ct) line_ct_use(kLineXFwd, d.LX, &k);
+    }
+    line_launch(k, dim3((unsigned)o.ctas, d.nb), o.threads, o.smem, st, d, f, S1, o.pl, line_table<T>(o.pl), o.nt, o.lines,
+                (int)(o.ctas * d.nb <= 304));
+    return true;
+}
+
+template <typename T>
+bool launch_line_x_inv(const DemagDims& d, const typename Cplx<T>::type* S1, T* h, cudaStream_t st) {
+    constexpr int NC = 1;
+    LineXShape o;
+    if (d.nb > 65535 || !line_x_shape<T>(d.LX, line_x_pairs(d), d.nb, 1, kAnyCtas, &o)) return false;
+    auto k = o.threads <= 256 ? line_x_inverse<T, NC, 256, 0> : line_x_inverse<T, NC, kLineThreads, 0>;
+    if constexpr (sizeof(T) == 4) {
+        if (o.ct) line_ct_use(kLineXInv, d.LX, &k);
+    }
+    line_launch(k, dim3((unsigned)o.ctas, d.nb), o.threads, o.smem, st, d, S1, h, o.pl, line_table<T>(o.pl), o.nt, o.lines,
+                (int)(o.ctas * d.nb <= 304));
+    return true;
+}
+
+int line_fused_blocks(const DemagDims& d, long max_ctas) {
+    LineXShape o;
+    if (d.nb > 65535 || !line_x_shape<float>(d.LX, line_fused_pairs(d), 1, 3, max_ctas, &o)) return 0;
+    return (int)o.ctas;
+}
+
+bool launch_line_fused(const DemagDims& d, float2* S1, const StageParams<float>& p, const LineBatch* bt, bool gen,
+                       bool fwd, long max_ctas, cudaStream_t st) {
+    LineXShape o;
+    if (d.nb > 65535 || !line_x_shape<float>(d.LX, line_fused_pairs(d), 1, 3, max_ctas, &o)) return false;
+    LineBatch b{};
+    if (bt) b = *bt;
+    auto k = gen ? (o.threads <= 256 ? line_fused<true, 256, 0> : line_fused<true, 1024, 0>)
+                 : (o.threads <= 256 ? line_fused<false, 256, 0> : line_fused<false, 1024, 0>);
+    if (o.ct) line_ct_use(gen ? kLineFusedGen : kLineFused, d.LX, &k);
+    // parked float2 values per x of a row pair (line_fused)
+    const int park = (p.next ? 3 : 0) + (p.want_err ? 3 : 0);
+    const size_t smem = o.smem + (size_t)o.lines * park * d.nx * sizeof(float2);
+    line_launch(k, dim3((unsigned)o.ctas, d.nb), o.threads, smem, st, d, S1, p, b, o.pl, line_table<float>(o.pl), o.nt,
+                o.lines, park, (int)fwd,
+                (int)(o.ctas * d.nb <= 304));
+    return true;
+}
+
+// the column shape a compiled length's kernel is built for
+static void line_ct_shape(int L, long ncol, LineShape* o) {
+    o->lb = line_ct_lb<float>(L);
+    const int M = L / o->pl.rmin;
+    o->threads = ((M << o->lb) + 31) / 32 * 32;
+    o->smem = (size_t)3 * line_len(L) * (sizeof(float2) << o->lb);
+    o->ctas = (ncol + (1 << o->lb) - 1) >> o->lb;
+}
 
 template <typename T, int DIR>
 bool launch_line_y(const DemagDims& d, const typename Cplx<T>::type* in, typename Cplx<T>::type* out,
                    cudaStream_t st) {
+    constexpr int NC = sizeof(T) == 8 ? 1 : 3;
     LineShape o;
-    const long ncol = (long)d.KX * d.nz;
-    if (d.nb > 65535 || !line_shape<T>(d.LY, ncol, d.nb, false, &o) || o.pl.np < 2) return false;
-    auto k = sizeof(T) == 4 && o.threads <= kLineThreads32 ? line_y<T, DIR, sizeof(T) == 4 ? kLineThreads32 : kLineThreads>
-                                                           : line_y<T, DIR, kLineThreads>;
-    line_launch(k, dim3((unsigned)o.ctas, d.nb), o.threads, o.smem, st, d, in, out, o.pl, o.lb, (int)ncol,
+    const long ncol = (long)d.KX * d.nz * (3 / NC);
+    if (d.nb > 65535 || !line_shape<T>(d.LY, ncol, d.nb, NC, false, &o) || o.pl.np < 2) return false;
+    auto k = sizeof(T) == 4 && o.threads <= kLineThreads32
+                 ? line_y<T, DIR, NC, sizeof(T) == 4 ? kLineThreads32 : kLineThreads, 0>
+                 : line_y<T, DIR, NC, kLineThreads, 0>;
+    if constexpr (sizeof(T) == 4) {
+        if (line_ct_use(DIR < 0 ? kLineYFwd : kLineYInv, d.LY, &k)) line_ct_shape(d.LY, ncol, &o);
+    }
+    line_launch(k, dim3((unsigned)o.ctas, d.nb), o.threads, o.smem, st, d, in, out, o.pl, line_table<T>(o.pl), o.lb, (int)ncol,
                 (int)(o.ctas * d.nb <= 304));
     return true;
 }
@@ -798,13 +673,16 @@ template <typename T>
 bool launch_line_conv(const DemagDims& d, typename Cplx<T>::type* S2, const T* tens, cudaStream_t st) {
     LineShape o;
     const long ncol = (long)d.KX * d.LY;
-    if (d.nb > 65535 || !line_shape<T>(d.LZ, ncol, d.nb, true, &o)) return false;
+    if (d.nb > 65535 || !line_shape<T>(d.LZ, ncol, d.nb, 3, true, &o)) return false;
+    constexpr int kSmall = sizeof(T) == 4 ? kLineThreads32 : kLineThreads;
+    auto k = o.pl.np == 1 ? line_conv<T, true, kLineThreads, 0>
+             : o.threads > kSmall ? line_conv<T, false, kLineThreads, 0> : line_conv<T, false, kSmall, 0>;
+    if constexpr (sizeof(T) == 4) {
+        if (o.pl.np > 1 && line_ct_use(kLineConv, d.LZ, &k)) line_ct_shape(d.LZ, ncol, &o);
+    }
     const dim3 grid((unsigned)o.ctas, d.nb);
-    const int early = o.ctas * d.nb <= 304;
-    auto k = o.pl.np == 1 ? line_conv<T, true, kLineThreads>
-             : sizeof(T) == 4 && o.threads <= kLineThreads32 ? line_conv<T, false, sizeof(T) == 4 ? kLineThreads32 : kLineThreads>
-                                                             : line_conv<T, false, kLineThreads>;
-    line_launch(k, grid, o.threads, o.smem, st, d, S2, tens, o.pl, o.lb, (int)ncol, early);
+    line_launch(k, grid, o.threads, o.smem, st, d, S2, tens, o.pl, line_table<T>(o.pl), o.lb, (int)ncol,
+                (int)(o.ctas * d.nb <= 304));
     return true;
 }
 
@@ -853,5 +731,10 @@ template void launch_rt_y<double, -1>(const DemagDims&, const double2*, double2*
 template void launch_rt_y<double, +1>(const DemagDims&, const double2*, double2*, cudaStream_t);
 template void launch_rt_z<float>(const DemagDims&, float2*, const float*, cudaStream_t);
 template void launch_rt_z<double>(const DemagDims&, double2*, const double*, cudaStream_t);
+
+template bool launch_line_x_fwd<float>(const DemagDims&, const LineXIn<float>&, float2*, cudaStream_t);
+template bool launch_line_x_fwd<double>(const DemagDims&, const LineXIn<double>&, double2*, cudaStream_t);
+template bool launch_line_x_inv<float>(const DemagDims&, const float2*, float*, cudaStream_t);
+template bool launch_line_x_inv<double>(const DemagDims&, const double2*, double*, cudaStream_t);
 
 }  // namespace mm

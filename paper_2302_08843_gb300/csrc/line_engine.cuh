@@ -1,10 +1,11 @@
-// Shared-memory FFT over lines of three-component vectors, for any even
+// Shared-memory FFT over lines of vectors of NC components, for any even
 // 7-smooth length with the radix plan known only at run time.
 //
-// A thread owns one butterfly of one line and carries it for all three
-// components, so that a pass's index arithmetic and twiddles are paid once
-// for three transforms, and the 3x3 tensor product and the cell updates find
-// the three components of a wave number (or cell) in one thread's registers.
+// A thread owns one butterfly of one line and carries it for NC components
+// (three or one); with three, a pass's index arithmetic and twiddles are paid once
+// for three transforms, and the 3x3 tensor product finds the components of a
+// wave number in one thread's registers; with one, three times the threads
+// share the work (FP64 passes other than the tensor product).
 // Element e of line l and component c lives at s[c plane + place(e) B + l];
 // the passes are in place (every thread reads its butterfly, the CTA
 // synchronises, every thread writes).
@@ -33,6 +34,7 @@
 namespace mm {
 
 constexpr int kLineMaxPass = 12;
+constexpr int kLineIdle = 1 << 20;       // butterfly number of a thread without a line: past every pass's count
 
 struct LinePlan {
     int L, np;
@@ -44,14 +46,75 @@ struct LinePlan {
     unsigned mg[kLineMaxPass], mgi[kLineMaxPass];   // ceil(2^32 / span)
 };
 
-// b mod Ns for b < 4096 with mg = ceil(2^32 / Ns): b mg / 2^32 is exact for b Ns < 2^32
-__device__ __forceinline__ int line_mod(int b, int Ns, unsigned mg) {
-    return Ns == 1 ? 0 : b - (int)__umulhi((unsigned)b, mg) * Ns;
+// The factors of L, as few as radices up to rmax (and 3, 5, 7) allow and among
+// those the largest smallest one, largest first: from radix number `at` on,
+// appended to cur[0..n).
+struct LineFactors {
+    int n = 0, f[kLineMaxPass] = {};
+};
+constexpr void line_factors(int L, int rmax, int at, LineFactors cur, LineFactors& best) {
+    constexpr int radix[7] = {8, 7, 6, 5, 4, 3, 2};
+    if (L == 1) {
+        if (best.n == 0 || cur.n < best.n || (cur.n == best.n && cur.f[cur.n - 1] > best.f[best.n - 1])) best = cur;
+        return;
+    }
+    if (cur.n == kLineMaxPass || (best.n && cur.n >= best.n)) return;
+    for (int i = at; i < 7; ++i) {
+        const int r = radix[i];
+        if (L % r || (r > rmax && r % 2 == 0)) continue;
+        LineFactors next = cur;
+        next.f[next.n++] = r;
+        line_factors(L / r, rmax, i, next, best);
+    }
 }
 
-// one slot of padding every eight elements spreads the strided writes of the
-// first passes over the banks
-__host__ __device__ __forceinline__ int line_place(int e) { return e + (e >> 3); }
+// The plan of an even length (np = 0: not one of the engine's): an even radix
+// first, the largest of the others last.
+constexpr LinePlan line_plan(int L, int rmax) {
+    LinePlan p{};
+    p.L = L;
+    LineFactors f;
+    line_factors(L, rmax, 0, LineFactors(), f);
+    if (f.n == 0) return p;
+    p.np = f.n;
+    p.rmin = f.f[f.n - 1];
+    int first = 0;
+    while (f.f[first] % 2) ++first;
+    p.R[0] = (short)f.f[first];
+    for (int i = 0, at = f.n - 1; i < f.n; ++i)
+        if (i != first) p.R[at--] = (short)f.f[i];
+    for (int i = 0, a = 1, b = 1; i < p.np; ++i) {
+        p.Ns[i] = (short)a;
+        p.Nsi[i] = (short)b;
+        p.mg[i] = (unsigned)(((1ull << 32) + a - 1) / a);
+        p.mgi[i] = (unsigned)(((1ull << 32) + b - 1) / b);
+        a *= p.R[i];
+        b *= p.R[p.np - 1 - i];
+    }
+    return p;
+}
+template <typename T> constexpr int line_rmax() { return sizeof(T) == 4 ? 8 : 4; }
+template <typename T> __host__ __device__ constexpr LinePlan line_ct(int L) { return line_plan(L, line_rmax<T>()); }
+// columns per CTA (log2) of a compiled length: a sector of each row at least, and two warps
+template <typename T> __host__ __device__ constexpr int line_ct_lb(int L) {
+    const LinePlan p = line_ct<T>(L);
+    int lb = sizeof(T) == 4 ? 2 : 1;
+    while (lb < 5 && ((L / p.rmin) << lb) < 64) ++lb;
+    while (lb > 0 && ((L / p.rmin) << lb) > 512) --lb;
+    return lb;
+}
+
+// b mod Ns for b < 4096 with mg = ceil(2^32 / Ns): b mg / 2^32 is exact for b Ns < 2^32
+// (mg = 0: Ns is a constant)
+__device__ __forceinline__ int line_mod(int b, int Ns, unsigned mg) {
+    return mg == 0 ? b % Ns : Ns == 1 ? 0 : b - (int)__umulhi((unsigned)b, mg) * Ns;
+}
+
+// One slot of padding every 2^SH elements spreads the strided writes of the
+// first passes over the banks: every eight where several lines lie side by side
+// (a warp reads eight elements of four lines), every sixteen where one line
+// does (a half warp reads sixteen elements).
+template <int SH> __host__ __device__ __forceinline__ int line_place(int e) { return e + (e >> SH); }
 __host__ __device__ __forceinline__ int line_len(int L) { return L + (L >> 3) + 1; }
 
 // x = a + w b, y = a - w b
@@ -98,9 +161,9 @@ template <int DIR, int R, bool HALF, typename C> __device__ __forceinline__ void
     }
 }
 
-// one butterfly of the three components: twiddles (none for span 1), then the DFT
-template <typename T, int DIR, int R>
-__device__ __forceinline__ void line_butterfly(typename Cplx<T>::type (&x)[3][R], const typename Cplx<T>::type* tw,
+// one butterfly of NC components: twiddles (none for span 1), then the DFT
+template <typename T, int DIR, int R, int NC>
+__device__ __forceinline__ void line_butterfly(typename Cplx<T>::type (&x)[NC][R], const typename Cplx<T>::type* tw,
                                                int k, int step, int L) {
     using C = typename Cplx<T>::type;
     auto W = [&](int m) {
@@ -111,11 +174,11 @@ __device__ __forceinline__ void line_butterfly(typename Cplx<T>::type (&x)[3][R]
     if constexpr (R == 2) {
         const C w = W(k * step);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) bf2(x[c][0], x[c][1], w);
+        for (int c = 0; c < NC; ++c) bf2(x[c][0], x[c][1], w);
     } else if constexpr (R == 4) {
         const C w1 = W(k * step), w2 = W(2 * k * step);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
+        for (int c = 0; c < NC; ++c) {
             C* a = x[c];
             bf2(a[0], a[2], w2);          // t0, t1
             bf2(a[1], a[3], w2);          // t2, t3
@@ -128,7 +191,7 @@ __device__ __forceinline__ void line_butterfly(typename Cplx<T>::type (&x)[3][R]
         // W_8 w1 = W_L^(k step + L/8)
         const C w1 = W(k * step), w2 = W(2 * k * step), w4 = W(4 * k * step), u = W(k * step + L / 8);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
+        for (int c = 0; c < NC; ++c) {
             C* a = x[c];
             bf2(a[0], a[4], w4); bf2(a[2], a[6], w4);
             bf2(a[0], a[2], w2); bf2i<DIR>(a[4], a[6], w2);     // E0 E2 | E1 E3 in a0 a2 a4 a6
@@ -146,35 +209,35 @@ __device__ __forceinline__ void line_butterfly(typename Cplx<T>::type (&x)[3][R]
         for (int q = 1; q < R; ++q) {
             const C w = W(q * k * step);
 #pragma unroll
-            for (int c = 0; c < 3; ++c) x[c][q] = cmul(x[c][q], w);
+            for (int c = 0; c < NC; ++c) x[c][q] = cmul(x[c][q], w);
         }
 #pragma unroll
-        for (int c = 0; c < 3; ++c) line_dft<DIR, R, false>(x[c]);
+        for (int c = 0; c < NC; ++c) line_dft<DIR, R, false>(x[c]);
     }
 }
 
-template <typename C, int R>
-__device__ __forceinline__ void line_load(C (&x)[3][R], const C* s, int plane, int lb, int b, int M) {
+template <int SH, typename C, int R, int NC>
+__device__ __forceinline__ void line_load(C (&x)[NC][R], const C* s, int plane, int lb, int b, int M) {
 #pragma unroll
     for (int q = 0; q < R; ++q) {
-        const C* p = s + (line_place(b + q * M) << lb);
+        const C* p = s + (line_place<SH>(b + q * M) << lb);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) x[c][q] = p[c * plane];
+        for (int c = 0; c < NC; ++c) x[c][q] = p[c * plane];
     }
 }
-template <typename C, int R>
-__device__ __forceinline__ void line_store(const C (&x)[3][R], C* s, int plane, int lb, int b, int k, int Ns) {
+template <int SH, typename C, int R, int NC>
+__device__ __forceinline__ void line_store(const C (&x)[NC][R], C* s, int plane, int lb, int b, int k, int Ns) {
 #pragma unroll
     for (int q = 0; q < R; ++q) {
-        C* p = s + (line_place((b - k) * R + k + q * Ns) << lb);
+        C* p = s + (line_place<SH>((b - k) * R + k + q * Ns) << lb);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) p[c * plane] = x[c][q];
+        for (int c = 0; c < NC; ++c) p[c * plane] = x[c][q];
     }
 }
 
 // a pass between two others, in place; s is the thread's line.  Every thread of
 // the CTA calls it.
-template <typename T, int DIR, int R>
+template <typename T, int DIR, int R, int NC, int SH>
 __device__ __forceinline__ void line_mid(typename Cplx<T>::type* s, int plane, int lb, int b, int L, int Ns,
                                          unsigned mg, const typename Cplx<T>::type* tw) {
     using C = typename Cplx<T>::type;
@@ -183,12 +246,12 @@ __device__ __forceinline__ void line_mid(typename Cplx<T>::type* s, int plane, i
     // set under a condition would stay live around the loop over passes and spill
     const bool on = b < M;
     if (!on) b = 0;
-    C x[3][R];
+    C x[NC][R];
     const int k = line_mod(b, Ns, mg);
-    line_load<C, R>(x, s, plane, lb, b, M);
-    line_butterfly<T, DIR, R>(x, tw, k, L / (Ns * R), L);
+    line_load<SH>(x, s, plane, lb, b, M);
+    line_butterfly<T, DIR>(x, tw, k, L / (Ns * R), L);
     __syncthreads();
-    if (on) line_store<C, R>(x, s, plane, lb, b, k, Ns);
+    if (on) line_store<SH>(x, s, plane, lb, b, k, Ns);
     __syncthreads();
 }
 
@@ -211,13 +274,25 @@ __device__ __forceinline__ void line_mid(typename Cplx<T>::type* s, int plane, i
         default: { constexpr int R_ = sizeof(Tv) == 4 ? 8 : 2; CALL; } break; \
     }
 
-template <typename T, int DIR>
+template <typename T, int DIR, int NC, int SH>
 __device__ __forceinline__ void line_mid_any(typename Cplx<T>::type* s, int plane, int lb, int b, const LinePlan& pl,
                                              int i, const typename Cplx<T>::type* tw) {
     const int R = DIR < 0 ? pl.R[i] : pl.R[pl.np - 1 - i];
     const int Ns = DIR < 0 ? pl.Ns[i] : pl.Nsi[i];
     const unsigned mg = DIR < 0 ? pl.mg[i] : pl.mgi[i];
-    MM_LINE_RADIX(T, R, (line_mid<T, DIR, R_>(s, plane, lb, b, pl.L, Ns, mg, tw)));
+    MM_LINE_RADIX(T, R, (line_mid<T, DIR, R_, NC, SH>(s, plane, lb, b, pl.L, Ns, mg, tw)));
+}
+
+// passes I .. END-1 of a compiled length
+template <typename T, int DIR, int NC, int SH, int LC, int I, int END>
+__device__ __forceinline__ void line_mids_ct(typename Cplx<T>::type* s, int plane, int lb, int b,
+                                             const typename Cplx<T>::type* tw) {
+    if constexpr (I < END) {
+        constexpr LinePlan P = line_ct<T>(LC);
+        constexpr int R = DIR < 0 ? P.R[I] : P.R[P.np - 1 - I], Ns = DIR < 0 ? P.Ns[I] : P.Nsi[I];
+        line_mid<T, DIR, R, NC, SH>(s, plane, lb, b, LC, Ns, 0, tw);
+        line_mids_ct<T, DIR, NC, SH, LC, I + 1, END>(s, plane, lb, b, tw);
+    }
 }
 
 }  // namespace mm

@@ -348,19 +348,91 @@ mm_status read_scalars(mm_state* s) {
     return MM_OK;
 }
 
+// whether this state's evaluations run the line engine's fused stage (FP32
+// with a demag term and x lines the engine takes)
+template <typename T> bool line_path(const mm_state* s) {
+    if constexpr (sizeof(T) == 4) return !s->demag_off && s->demag_ready && line_fused_blocks(s->d, 1L << 40) > 0;
+    return false;
+}
+
+// One field evaluation at the stage input p.m with the outputs p asks for.
+// FP32 (line_path): S1 through the y and z passes (s1_ready: S1 already holds
+// the x-spectrum of Ms p.m), then the fused stage, which leaves the x-spectrum
+// of Ms p.next in S1 when fwd is set.  Otherwise demag field, then stage.
+template <typename T> mm_status run_eval(mm_state* s, StageParams<T>& p, bool reduce, bool s1_ready, bool fwd) {
+    if constexpr (sizeof(T) == 4) {
+        if (line_path<T>(s)) {
+            s->s1_fresh = false;
+            demag_front<float>(s->d, p.m, (const float*)s->Ms_cell, (float)s->Ms, !s1_ready, (float2*)s->S1,
+                               (float2*)s->S2, (const float*)s->tens, s->st, &s->timer);
+            MM_LAUNCHED();
+            p.hd = nullptr;
+            p.partials = nullptr;
+            const int nb = line_fused_blocks(s->d, 1L << 40);
+            if (reduce) {
+                MM_TRY(ensure_partials(s, nb));
+                p.partials = s->partials;
+            }
+            stage_prepare(p);
+            const bool gen = p.Ms_cell || p.A_cell || p.Ku_cell || p.alpha_cell || p.zw || p.D_cell || p.lay || p.dmi ||
+                             p.want_energy || p.Ms == 0.f;
+            s->timer.begin(s->st, "line_fused");
+            const bool ok = launch_line_fused(s->d, (float2*)s->S1, p, nullptr, gen, fwd, 1L << 40, s->st);
+            s->timer.end(s->st);
+            if (!ok) return fail(MM_ECUDA, "fused line kernel could not be launched for this grid");
+            MM_LAUNCHED();
+            if (reduce) {
+                s->timer.begin(s->st, "finalize_reduce");
+                launch_finalize(s->partials, nb, s->dev_err, s->h_scalars, s->st);
+                s->timer.end(s->st);
+                MM_LAUNCHED();
+            }
+            return MM_OK;
+        }
+    }
+    MM_TRY(run_demag<T>(s, p.m));
+    return run_stage<T>(s, p, reduce);
+}
+
+// y = m + dt a k, a stage input without a field evaluation; FP32 (line_path)
+// with the x-spectrum of Ms y left in S1 by the same pass
+template <typename T> mm_status run_combine(mm_state* s, const void* k, double a, double dt, void* y) {
+    if constexpr (sizeof(T) == 4) {
+        if (line_path<T>(s)) {
+            LineXIn<float> in;
+            in.m = (const float*)s->m;
+            in.Ms_cell = (const float*)s->Ms_cell;
+            in.Ms = (float)s->Ms;
+            in.k = (const float*)k;
+            in.y = (float*)y;
+            in.ca = (float)(dt * a);
+            s->s1_fresh = false;
+            s->timer.begin(s->st, "p1_x_forward");
+            const bool ok = launch_line_x_fwd<float>(s->d, in, (float2*)s->S1, s->st);
+            s->timer.end(s->st);
+            if (!ok) return fail(MM_ECUDA, "x-forward pass could not be launched for this grid");
+            MM_LAUNCHED();
+            return MM_OK;
+        }
+    }
+    const T* k0 = (const T*)k;
+    launch_combine<T>((const T*)s->m, &k0, &a, 1, dt, (T*)y, s->N, s->st);
+    MM_LAUNCHED();
+    return MM_OK;
+}
+
 template <typename T>
 mm_status heff_impl(mm_state* s, const void* m, void* h_out, double* E_out, double t, double* torque_out) {
     MM_TRY(ready_for_fields(s));
     if (!m && !s->have_m) return fail(MM_ENOTSETUP, "no magnetisation: call mm_set_m or pass m");
     const void* mm_ = m ? m : s->m;
-    MM_TRY(run_demag<T>(s, mm_));
     StageParams<T> p;
     fill_common<T>(s, p, mm_, t);
     p.h_out = (T*)h_out;
     p.want_energy = E_out != nullptr;
     p.want_torque = torque_out != nullptr;
     const bool reduce = E_out || torque_out;
-    MM_TRY(run_stage<T>(s, p, reduce));
+    MM_TRY(run_eval<T>(s, p, reduce, false, false));
     if (reduce) {
         MM_TRY(read_scalars(s));
         if (E_out) {
@@ -403,11 +475,10 @@ template <typename T> mm_status rhs_impl(mm_state* s, const void* m, void* k_out
             return MM_OK;
         }
     }
-    MM_TRY(run_demag<T>(s, mm_));
     StageParams<T> p;
     fill_common<T>(s, p, mm_, t);
     p.k_out = (T*)k_out;
-    return run_stage<T>(s, p, false);
+    return run_eval<T>(s, p, false, false, false);
 }
 
 const double kRK4_C[4] = {0.0, 0.5, 0.5, 1.0};
@@ -468,8 +539,9 @@ template <typename T> mm_status rk4_impl(mm_state* s, double dt, double t) {
     const double anext[3] = {0.5, 0.5, 1.0};
     void* in[4] = {s->m, s->mA, s->mB, s->mA};
     void* out[4] = {s->mA, s->mB, s->mA, s->m};
+    const bool fresh = s->s1_fresh;         // S1 from the last step's end
+    const bool line = line_path<T>(s);
     for (int st = 0; st < 4; ++st) {
-        MM_TRY(run_demag<T>(s, in[st]));
         StageParams<T> p;
         fill_common<T>(s, p, in[st], t + kRK4_C[st] * dt);
         p.dt = dt;
@@ -486,8 +558,9 @@ template <typename T> mm_status rk4_impl(mm_state* s, double dt, double t) {
             p.ck = b[3];
             p.renorm = 1;
         }
-        MM_TRY(run_stage<T>(s, p, false));
+        MM_TRY(run_eval<T>(s, p, false, line && (st > 0 || fresh), true));
     }
+    s->s1_fresh = line;
     s->fsal = s->k1_exact = false;
     return MM_OK;
 }
@@ -514,12 +587,11 @@ mm_status ensure_dp_buffers(mm_state* s) {
 
 // k1 = f(m, t) into K[0]; optional torque readback
 template <typename T> mm_status dp_first_stage(mm_state* s, double t, double* torque) {
-    MM_TRY(run_demag<T>(s, s->m));
     StageParams<T> p;
     fill_common<T>(s, p, s->m, t);
     p.k_out = (T*)s->K[0];
     p.want_torque = torque != nullptr;
-    MM_TRY(run_stage<T>(s, p, torque != nullptr));
+    MM_TRY(run_eval<T>(s, p, torque != nullptr, false, false));
     if (torque) {
         MM_TRY(read_scalars(s));
         *torque = s->h_scalars[R_TORQUE];
@@ -534,14 +606,12 @@ template <typename T> mm_status dp_first_stage(mm_state* s, double t, double* to
 template <typename T>
 mm_status dp_attempt(mm_state* s, double t, double dt, double rtol, double* err, double* torque, void** y5buf) {
     // y2 = m + dt a21 k1
-    const T* k0 = (const T*)s->K[0];
-    launch_combine<T>((const T*)s->m, &k0, &kDP_A[1][0], 1, dt, (T*)s->mA, s->N, s->st);
-    MM_LAUNCHED();
+    MM_TRY(run_combine<T>(s, s->K[0], kDP_A[1][0], dt, s->mA));
+    const bool line = line_path<T>(s);
     void* ybuf[2] = {s->mA, s->mB};
     int cur = 0;
     for (int st = 1; st <= 6; ++st) {     // stage st computes K[st] from y_{st+1} (0-based K)
         void* yin = ybuf[cur];
-        MM_TRY(run_demag<T>(s, yin));
         StageParams<T> p;
         fill_common<T>(s, p, yin, t + kDP_C[st] * dt);
         p.dt = dt;
@@ -551,7 +621,7 @@ mm_status dp_attempt(mm_state* s, double t, double dt, double rtol, double* err,
             for (int q = 0; q < st; ++q) { p.kin[q] = (const T*)s->K[q]; p.kc[q] = kDP_A[st + 1][q]; }
             p.nk = st;
             p.ck = kDP_A[st + 1][st];
-            MM_TRY(run_stage<T>(s, p, false));
+            MM_TRY(run_eval<T>(s, p, false, line, true));
             cur = 1 - cur;
         } else {
             // last stage: k7 = f(y7), error estimate, torque at y7
@@ -562,7 +632,7 @@ mm_status dp_attempt(mm_state* s, double t, double dt, double rtol, double* err,
             p.rtol = rtol;
             p.atol = rtol;
             p.want_torque = 1;
-            MM_TRY(run_stage<T>(s, p, true));
+            MM_TRY(run_eval<T>(s, p, true, line, false));
             *y5buf = yin;
         }
     }
@@ -593,8 +663,8 @@ mm_status adjoint_impl(mm_state* s, const void* m_n, const void* lam_np1, void* 
     T* Apart = A[18];
     const T* ms[4] = {(const T*)m_n, Am[0], Am[1], Am[2]};
     // forward recompute of the stage inputs, fields and derivatives
+    const bool line = line_path<T>(s);
     for (int st = 0; st < 4; ++st) {
-        MM_TRY(run_demag<T>(s, ms[st]));
         StageParams<T> p;
         fill_common<T>(s, p, ms[st], t + kRK4_C[st] * dt);
         p.mn = (const T*)m_n;
@@ -605,7 +675,7 @@ mm_status adjoint_impl(mm_state* s, const void* m_n, const void* lam_np1, void* 
             p.next = Am[st];
             p.ck = kRK4_C[st + 1];
         }
-        MM_TRY(run_stage<T>(s, p, false));
+        MM_TRY(run_eval<T>(s, p, false, line && st > 0, st < 3));
     }
     const T* kin[4] = {Ak[0], Ak[1], Ak[2], Ak[3]};
     launch_combine<T>((const T*)m_n, kin, b, 4, dt, Ay, s->N, s->st);
@@ -710,14 +780,12 @@ const double kRKF_B5[6] = {16.0 / 135.0, 0.0, 6656.0 / 12825.0, 28561.0 / 56430.
 // (returned in *y4buf, not renormalised) and the error norm against it
 template <typename T>
 mm_status rkf_attempt(mm_state* s, double t, double dt, double rtol, double* err, void** y4buf) {
-    const T* k0 = (const T*)s->K[0];
-    launch_combine<T>((const T*)s->m, &k0, &kRKF_A[1][0], 1, dt, (T*)s->mA, s->N, s->st);
-    MM_LAUNCHED();
+    MM_TRY(run_combine<T>(s, s->K[0], kRKF_A[1][0], dt, s->mA));
+    const bool line = line_path<T>(s);
     void* ybuf[2] = {s->mA, s->mB};
     int cur = 0;
     for (int st = 1; st <= 5; ++st) {     // stage st computes K[st] from y_{st+1}
         void* yin = ybuf[cur];
-        MM_TRY(run_demag<T>(s, yin));
         StageParams<T> p;
         fill_common<T>(s, p, yin, t + kRKF_C[st] * dt);
         p.dt = dt;
@@ -727,7 +795,7 @@ mm_status rkf_attempt(mm_state* s, double t, double dt, double rtol, double* err
             for (int q = 0; q < st; ++q) { p.kin[q] = (const T*)s->K[q]; p.kc[q] = kRKF_A[st + 1][q]; }
             p.nk = st;
             p.ck = kRKF_A[st + 1][st];
-            MM_TRY(run_stage<T>(s, p, false));
+            MM_TRY(run_eval<T>(s, p, false, line, true));
         } else {
             // last stage: k6, y4 = m + dt sum b4 k, error sum (b5 - b4) k against y4
             for (int q = 0; q < 5; ++q) {
@@ -742,7 +810,7 @@ mm_status rkf_attempt(mm_state* s, double t, double dt, double rtol, double* err
             p.err_on_next = 1;
             p.rtol = rtol;
             p.atol = rtol;
-            MM_TRY(run_stage<T>(s, p, true));
+            MM_TRY(run_eval<T>(s, p, true, line, false));
             *y4buf = ybuf[1 - cur];
         }
         cur = 1 - cur;
@@ -804,6 +872,7 @@ struct mm_batch {
     void* D_d = nullptr;
     void* pc_d = nullptr;
     int* kind_d = nullptr;
+    std::vector<char> special;     // slots with DMI or Ms = 0: the general variant of the fused stage
     std::vector<char> unstarted;   // loaded and not yet in an mm_batch_begin
     // per-slot controller state, on the device: status, steps, fresh, dt, t, torque
     int* ctl_i = nullptr;        // [3][cap] ints
@@ -820,8 +889,10 @@ struct mm_batch {
     int nact = 0;                // slots [0, nact) are launched (highest running slot + 1)
     bool pending = false;
     bool fresh_any = false;
+    bool gen = false;            // this call's launches take the general variant of the fused stage
     std::vector<int> status;     // host mirror of the last report
     // cached CUDA graphs of `attempts` consecutive attempts, per (nact, attempts)
+    // (negative attempts: with the general variant of the fused stage)
     std::map<std::pair<int, int>, cudaGraphExec_t> graphs;
     double g_rtol = -1, g_tol = -1;
     int g_max_steps = -1;
@@ -852,6 +923,68 @@ size_t batch_bytes(const mm_grid* g, mm_precision prec, int cap, int* LXo, int* 
     return bytes;
 }
 
+// FP32 batches whose x lines the line engine takes run its fused stage
+template <typename T> bool batch_line(const mm_batch* b) {
+    if constexpr (sizeof(T) == 4) return line_fused_blocks(b->d, b->nblk) > 0;
+    return false;
+}
+
+// x-forward of Ms m, or of Ms y with y = m + dt a k per grid (stored), into S1
+mm_status batch_line_forward(mm_batch* b, const void* m, const void* k, double a, void* y, const int* mask) {
+    LineXIn<float> in;
+    in.m = (const float*)m;
+    in.k = (const float*)k;
+    in.y = (float*)y;
+    in.dt_b = b->dt_d();
+    in.a = a;
+    in.mask = mask;
+    if (!launch_line_x_fwd<float>(b->d, in, (float2*)b->S1, b->st))
+        return fail(MM_ECUDA, "x-forward pass could not be launched for this grid");
+    MM_LAUNCHED();
+    return MM_OK;
+}
+
+// y and z passes on S1, then the fused stage of batch_stage's parameters; S1
+// becomes the x-spectrum of Ms next where there is a next stage input
+mm_status batch_line_stage(mm_batch* b, const BatchStageParams<float>& q, bool gen) {
+    KernelTimer off;
+    demag_front<float>(b->d, nullptr, nullptr, 0.f, false, (float2*)b->S1, (float2*)b->S2, (const float*)b->tens, b->st,
+                       &off);
+    MM_LAUNCHED();
+    StageParams<float> p;
+    std::memset(&p, 0, sizeof(p));
+    p.nx = q.nx; p.ny = q.ny; p.nz = q.nz; p.N = q.N;
+    p.idx2 = q.idx2; p.idy2 = q.idy2; p.idz2 = q.idz2;
+    p.i2dx = q.i2dx; p.i2dy = q.i2dy; p.i2dz = q.i2dz;
+    p.hx0 = q.hx0; p.hy0 = q.hy0; p.hz0 = q.hz0;
+    p.m = q.m; p.mn = q.mn; p.k_out = q.k_out; p.next = q.next;
+    p.nk = q.nk;
+    for (int i = 0; i < 7; ++i) { p.kin[i] = q.kin[i]; p.kcT[i] = q.kc[i]; p.ebT[i] = q.eb[i]; }
+    p.ckT = q.ck; p.eb_kT = q.eb_k;
+    p.rtolT = p.atolT = q.rtol;
+    p.want_err = q.want_err; p.want_torque = q.want_torque;
+    LineBatch bt;
+    std::memset(&bt, 0, sizeof(bt));
+    bt.mask = q.mask;
+    bt.Ms = q.Ms; bt.A = q.A; bt.alpha = q.alpha; bt.D = q.D; bt.pc = q.pc; bt.kind = q.dmi_kind; bt.dt = q.dt;
+    std::memcpy(bt.dmi_e, q.dmi_e, sizeof(bt.dmi_e));
+    bt.partials = q.partials;
+    if (!launch_line_fused(b->d, (float2*)b->S1, p, &bt, gen, q.next != nullptr, b->nblk, b->st))
+        return fail(MM_ECUDA, "fused line kernel could not be launched for this grid");
+    MM_LAUNCHED();
+    return MM_OK;
+}
+
+template <typename T> mm_status batch_demag(mm_batch* b, const void* m) {
+    using C = typename Cplx<T>::type;
+    KernelTimer off;
+    demag_apply<T>(b->d, (const T*)m, nullptr, (T)0, (C*)b->S1, (C*)b->S2, (const T*)b->tens, (T*)b->hd, b->st, &off);
+    MM_LAUNCHED();
+    return MM_OK;
+}
+
+// one field evaluation of the launched grids at stage input m (for the line
+// path S1 holds its x-spectrum), and the stage's outputs
 template <typename T> mm_status batch_stage(mm_batch* b, const void* m, const void* mn, void* k_out, void* next,
                                             const int* mask, int st, bool err, bool torque, double* partials,
                                             double rtol) {
@@ -885,15 +1018,11 @@ template <typename T> mm_status batch_stage(mm_batch* b, const void* m, const vo
     p.want_torque = torque;
     p.partials = partials;
     p.rtol = rtol;
+    if constexpr (sizeof(T) == 4) {
+        if (batch_line<T>(b)) return batch_line_stage(b, p, b->gen);
+    }
+    MM_TRY(batch_demag<T>(b, m));
     launch_batch_stage<T>(p, b->st);
-    MM_LAUNCHED();
-    return MM_OK;
-}
-
-template <typename T> mm_status batch_demag(mm_batch* b, const void* m) {
-    using C = typename Cplx<T>::type;
-    KernelTimer off;
-    demag_apply<T>(b->d, (const T*)m, nullptr, (T)0, (C*)b->S1, (C*)b->S2, (const T*)b->tens, (T*)b->hd, b->st, &off);
     MM_LAUNCHED();
     return MM_OK;
 }
@@ -903,9 +1032,10 @@ template <typename T> mm_status batch_first(mm_batch* b, double rtol, double tol
     const int cap = b->cap;
     launch_batch_masks(b->status_d(), b->fresh_d(), b->mask_d, cap, b->st);
     MM_LAUNCHED();
-    MM_TRY(batch_demag<T>(b, b->m));
+    if (batch_line<T>(b)) MM_TRY(batch_line_forward(b, b->m, nullptr, 0.0, nullptr, b->mask_d));
     MM_TRY(batch_stage<T>(b, b->m, b->m, b->K[0], nullptr, b->mask_d, 0, false, true, b->partials, rtol));
-    launch_batch_finalize(b->partials, b->nblk, b->nact, b->scal_d, b->st);
+    const int nblk = batch_line<T>(b) ? line_fused_blocks(b->d, b->nblk) : b->nblk;
+    launch_batch_finalize(b->partials, nblk, b->nact, b->scal_d, b->st);
     MM_LAUNCHED();
     launch_batch_first(b->scal_d, b->mask_d, b->status_d(), b->fresh_d(), b->torque_d(), tol, cap, b->st);
     MM_LAUNCHED();
@@ -917,15 +1047,20 @@ template <typename T> mm_status batch_attempts(mm_batch* b, int attempts, double
     const int cap = b->cap;
     int* run = b->mask_d + cap;
     double* p1 = b->partials + (size_t)cap * b->nblk * 3;
+    const bool line = batch_line<T>(b);
+    const int nblk = line ? line_fused_blocks(b->d, b->nblk) : b->nblk;
     launch_batch_masks(b->status_d(), b->fresh_d(), b->mask_d, cap, b->st);
     MM_LAUNCHED();
     for (int a = 0; a < attempts; ++a) {
-        launch_batch_combine<T>((const T*)b->m, (const T*)b->K[0], b->dt_d(), kDP_A[1][0], run, (T*)b->Y[0],
-                                (int)b->N, b->nact, b->st);
-        MM_LAUNCHED();
+        if (line) {
+            MM_TRY(batch_line_forward(b, b->m, b->K[0], kDP_A[1][0], b->Y[0], run));
+        } else {
+            launch_batch_combine<T>((const T*)b->m, (const T*)b->K[0], b->dt_d(), kDP_A[1][0], run, (T*)b->Y[0],
+                                    (int)b->N, b->nact, b->st);
+            MM_LAUNCHED();
+        }
         int cur = 0;
         for (int st = 1; st <= 6; ++st) {
-            MM_TRY(batch_demag<T>(b, b->Y[cur]));
             if (st < 6) {
                 MM_TRY(batch_stage<T>(b, b->Y[cur], b->m, b->K[st], b->Y[1 - cur], run, st, false, false, nullptr,
                                       rtol));
@@ -935,7 +1070,7 @@ template <typename T> mm_status batch_attempts(mm_batch* b, int attempts, double
                 b->y5 = cur;
             }
         }
-        launch_batch_finalize(p1, b->nblk, b->nact, b->scal_d + 3 * cap, b->st);
+        launch_batch_finalize(p1, nblk, b->nact, b->scal_d + 3 * cap, b->st);
         MM_LAUNCHED();
         launch_batch_control(b->scal_d + 3 * cap, run, b->status_d(), b->steps_d(), b->dt_d(), b->t_d(),
                              b->torque_d(), b->acc_d, tol, max_steps, cap, b->st);
@@ -964,6 +1099,9 @@ mm_status batch_begin_impl(mm_batch* b, int attempts, double rtol, double tol, i
         // masked ones below it cost one early-exiting block per tile
         b->nact = hi;
         b->d.nb = hi;
+        b->gen = false;
+        for (int i = 0; i < hi; ++i)
+            if (b->status[i] == 1 && b->special[i]) b->gen = true;
         if (b->fresh_any) {
             MM_TRY(batch_first<T>(b, rtol, tol));
             b->fresh_any = false;
@@ -972,7 +1110,7 @@ mm_status batch_begin_impl(mm_batch* b, int attempts, double rtol, double tol, i
             batch_drop_graphs(b);
             b->g_rtol = rtol; b->g_tol = tol; b->g_max_steps = max_steps;
         }
-        const auto key = std::make_pair(hi, attempts);
+        const auto key = std::make_pair(hi, b->gen ? -attempts : attempts);
         auto it = b->graphs.find(key);
         cudaGraphExec_t exec = it == b->graphs.end() ? nullptr : it->second;
         if (!exec) {
@@ -1471,6 +1609,7 @@ mm_status mm_batch_create(const mm_grid* grid, mm_precision precision, int capac
     if (e != cudaSuccess) return bail(fail(MM_ECUDA, "batch set-up: %s", cudaGetErrorString(e)));
     b->status.assign(capacity, 0);
     b->unstarted.assign(capacity, 0);
+    b->special.assign(capacity, 0);
     *out = b;
     return MM_OK;
 }
@@ -1508,6 +1647,7 @@ mm_status mm_batch_set_slot(mm_batch* b, int slot, double Ms, double A, double a
     MM_CUDA(cudaMemcpyAsync(b->torque_d() + slot, &dz, sizeof(double), cudaMemcpyHostToDevice, b->st));
     MM_CUDA(cudaStreamSynchronize(b->st));   // the host values above are stack copies
     b->status[slot] = 1;
+    b->special[slot] = Ms == 0.0 || (float)Ms == 0.f;
     b->unstarted[slot] = 1;
     b->fresh_any = true;
     return MM_OK;
@@ -1534,6 +1674,7 @@ mm_status mm_batch_set_slot_terms(mm_batch* b, int slot, int dmi_kind, double D,
     }
     MM_CUDA(cudaMemcpyAsync(b->kind_d + slot, &kind, sizeof(int), cudaMemcpyHostToDevice, b->st));
     MM_CUDA(cudaStreamSynchronize(b->st));   // the host values above are stack copies
+    if (kind != MM_DMI_NONE) b->special[slot] = 1;
     return MM_OK;
 }
 

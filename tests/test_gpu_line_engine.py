@@ -62,3 +62,30 @@ def test_batch_lines_match_single_grids(n):
         assert st[slot] == 1 and steps[slot] == 1
         assert rel(b.get_m(slot), m) < 1e-13
     b.close()
+
+
+@pytest.mark.parametrize("n", [(25, 25, 1), (24, 9, 2), (32, 16, 3), (50, 7, 1), (18, 1, 5)])
+def test_fused_stage_steps_match_fp64(n):
+    """FP32 DP45 and RKF45 steps through the fused stage, rows of y paired and the
+    last one alone, against the FP64 passes: the step sizes (error norm) to 1e-3,
+    the states to 20 times the FP32 field bound."""
+    from paper_2302_08843_gb300.binding import State
+    from paper_2302_08843_gb300.workloads import to_soa
+    rng = np.random.default_rng(3)
+    m = rng.normal(size=n + (3,))
+    m = to_soa(m / np.linalg.norm(m, axis=-1, keepdims=True))
+    for method in ("dp45", "rkf45"):
+        out = []
+        for precision in ("fp64", "fp32"):
+            s = State(n, D, precision)
+            s.set_material(Ms=8e5, A=1.3e-11, alpha=0.5, Ku1=1e5, ku_axis=(0.0, 0.6, 0.8))
+            s.demag_setup(20)
+            s.set_m(m)
+            t, dt, dts = 0.0, 2e-14, []
+            for _ in range(3):
+                t, dt = s.step(dt, t, method, 1e-3)
+                dts.append(dt)
+            out.append((np.array(dts), to_host(s.get_m())))
+            s.close()
+        assert np.max(np.abs(out[1][0] / out[0][0] - 1)) < 1e-3
+        assert rel(out[1][1], out[0][1]) < 20 * FP32_TOL
