@@ -47,6 +47,12 @@ struct DemagDims {
     // 2-D grids: the z-pass kernels run along y (nz' = ny, Pz' = Py); the
     // odd components' mirror signs then come from the transformed axis
     int yz_swap = 0;
+    // FP32: the separate passes with the compiled and the ping-pong engines, and
+    // none of the line engine's.  RK4 steps driven through per-cell Zeeman weights
+    // keep them: such runs read small signals out of a nearly uniform state, and
+    // the rounding of their demag field is the signal's noise (1e-6 of it), so
+    // another order of operations, though no less exact, moves every such signal.
+    int classic = 0;
     // non-equidistant layers (Sec. 4.4): no transform along z; the nz layers
     // are coupled densely at every lateral wave number (p3_layers).  lh holds
     // the nz thicknesses in the real type of the passes.

@@ -1093,6 +1093,89 @@ p3_z_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restr
     }
 }
 
+// Register-resident variant (FP32): each thread keeps its 16 values of all
+// three components from the first load to the last store; shared memory only
+// carries the exchanges inside each transform (one per 128-point transform).
+template <typename T, int LZ, int B, int G>
+__global__ void __launch_bounds__(B * G * Fft<T, LZ, -1, (LZ > 1)>::TPL,
+                                  (384 / (B * G * Fft<T, LZ, -1, (LZ > 1)>::TPL)) > 1
+                                      ? 384 / (B * G * Fft<T, LZ, -1, (LZ > 1)>::TPL) : 1)
+p3_z_conv_reg(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restrict__ tens) {
+    using C = typename Cplx<T>::type;
+    using FF = Fft<T, LZ, -1, (LZ > 1)>;
+    using FI = Fft<T, LZ, +1, false>;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    C* s = reinterpret_cast<C*>(smraw);
+    constexpr int NL = B * G;
+    constexpr int NR = FF::NR, TPL = FF::TPL;
+    constexpr int NOUT = LZ == 1 ? 1 : NR / 2;
+    const int tid = threadIdx.x;
+    const int line = tid % NL, j = tid / NL;
+    const int kl = line % B, g = line / B;
+    const int kx = blockIdx.x * B + kl;
+    const int kyi = blockIdx.y * G + g;           // (folded ky, side) pairs, side fastest
+    const int p = kyi >> 1, side = kyi & 1;
+    const int LY = d.LY;
+    const int KY2 = LY / 2 + 1;
+    const bool valid = kx < d.KX && p < KY2 && (side == 0 || (p > 0 && 2 * p < LY));
+    const int ky = side ? LY - p : p;
+    const long cstride = (long)d.nz * LY * d.KXS;
+    C* col = S2 + (long)blockIdx.z * 3 * cstride + (long)ky * d.KXS + kx;
+    const long zs = (long)LY * d.KXS;
+
+    C vx[NR], vy[NR], vz[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        const int z = FF::in_index(j, r);
+        vx[r] = vy[r] = vz[r] = mk<C>(0, 0);
+        if (valid && FF::in_live(r) && z < d.nz) {
+            vx[r] = col[z * zs];
+            vy[r] = col[cstride + z * zs];
+            vz[r] = col[2 * cstride + z * zs];
+        }
+    }
+    FF::run(vx, s + line, NL, j);
+    FF::run(vy, s + line, NL, j);
+    FF::run(vz, s + line, NL, j);
+    const int KZ2 = LZ / 2 + 1;
+    const long tcomp = (long)KZ2 * KY2 * d.KXS;
+    const T sy = side ? (T)-1 : (T)1;
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        const int kz = j + r * TPL;
+        const int kzf = (2 * kz <= LZ) ? kz : LZ - kz;
+        const T sz = (2 * kz <= LZ) ? (T)1 : (T)-1;
+        T txx = 0, txy = 0, txz = 0, tyy = 0, tyz = 0, tzz = 0;
+        if (valid) {
+            const T* tp = tens + ((long)kzf * KY2 + p) * d.KXS + kx;
+            txx = __ldg(tp);
+            txy = (d.yz_swap ? sz : sy) * __ldg(tp + tcomp);
+            txz = (d.yz_swap ? sy : sz) * __ldg(tp + 2 * tcomp);
+            tyy = __ldg(tp + 3 * tcomp);
+            tyz = sy * sz * __ldg(tp + 4 * tcomp);
+            tzz = __ldg(tp + 5 * tcomp);
+        }
+        const C mx = vx[r], my = vy[r], mz = vz[r];
+        vx[r] = mk<C>(txx * mx.x + txy * my.x + txz * mz.x, txx * mx.y + txy * my.y + txz * mz.y);
+        vy[r] = mk<C>(txy * mx.x + tyy * my.x + tyz * mz.x, txy * mx.y + tyy * my.y + tyz * mz.y);
+        vz[r] = mk<C>(txz * mx.x + tyz * my.x + tzz * mz.x, txz * mx.y + tyz * my.y + tzz * mz.y);
+    }
+    FI::run(vx, s + line, NL, j);
+    FI::run(vy, s + line, NL, j);
+    FI::run(vz, s + line, NL, j);
+    if (valid) {
+#pragma unroll
+        for (int r = 0; r < NOUT; ++r) {
+            const int z = j + r * TPL;
+            if (z < d.nz) {
+                col[z * zs] = vx[r];
+                col[cstride + z * zs] = vy[r];
+                col[2 * cstride + z * zs] = vz[r];
+            }
+        }
+    }
+}
+
 // ----------------------------------------------------------- P3 layers ----
 // Non-equidistant layers (Sec. 4.4): no transform along z; at every lateral
 // wave number (kx, ky) the nz layers are coupled densely,
@@ -1980,24 +2063,37 @@ template <int L> static bool launch_p5_tma(const DemagDims& d, const float2* S1,
 
 template <typename T, int L> static void launch_p3(const DemagDims& d, typename Cplx<T>::type* S2, const T* tens,
                                                    cudaStream_t st) {
-    // single FP32 grids: the persistent TMA passes where a line has one; the
-    // line engine otherwise (FP64, batches, other lengths): FP64 64-point lines
-    // 519 -> 417 us on 128x128x32, 256-point lines along y of a 512x128x1 film
-    // 97 -> 44 us, 16 FP32 grids of 100x100x8 63 -> 34 us.  On an FP32 film's
-    // 256-point lines the TMA pass stays the faster one (8.7 against 10.0 us).
+    // Single FP32 grids with tiles enough for the persistent TMA passes (16
+    // columns of one ky each; two-factor lines: always) take those: 2304 tiles of
+    // 32-point lines 14.6 against 16.5 us, 128-point lines 43 against 70.  The line
+    // engine takes the others, where a tile's latency is what counts (33 tiles of
+    // a film's 256 points 8.6 -> 5.8 us, 640 of 32 points 10.5 -> 9.0; lines up to
+    // 16 points, one thread each, are level up to 8704 tiles), FP64 (64-point
+    // lines of 128x128x32 519 -> 393 us, 256 points of a 512x128x1 film 97 -> 44)
+    // and batches (16 grids of 100x100x8 63 -> 34 us).
     if constexpr (sizeof(T) == 4 && L <= 256 && Fft<T, L, -1, (L > 1)>::NR <= 20) {
         if constexpr (z_two_r1<L>() > 0) {
             if (kZTwo && d.nb == 1 && launch_p3_two<L>(d, S2, tens, st)) return;
         }
         if constexpr (tma_len<L>()) {
-            if (d.nb == 1 && launch_p3_tma<L>(d, S2, tens, st)) return;
+            const long tiles = (long)((d.KX + 15) / 16) * d.LY;
+            if (d.nb == 1 && (d.classic || tiles >= (L <= 16 ? 8192 : 1024)) && launch_p3_tma<L>(d, S2, tens, st)) return;
         }
     }
-    if (launch_line_conv<T>(d, S2, tens, st)) return;
-    if constexpr (L >= 2048) {        // FP64 lines of more butterflies than a CTA of the line engine holds
-        constexpr int B = b_p3<T, L>(), G = g_p3<T, L>();
-        using C = typename Cplx<T>::type;
-        const int kyi = 2 * (d.LY / 2 + 1);
+    if (!d.classic && launch_line_conv<T>(d, S2, tens, st)) return;
+    constexpr int B = b_p3<T, L>(), G = g_p3<T, L>();
+    using C = typename Cplx<T>::type;
+    const int kyi = 2 * (d.LY / 2 + 1);
+    if constexpr (sizeof(T) == 4 && L <= 256 && Fft<T, L, -1, (L > 1)>::NR <= 20) {     // classic
+        // 128-thread CTAs: three fit per SM at up to 170 registers per thread
+        constexpr int G3 = (B * tpl_of<T, L>() >= 128) ? 1 : 128 / (B * tpl_of<T, L>());
+        dim3 grid3((d.KX + B - 1) / B, (kyi + G3 - 1) / G3, d.nb);
+        const size_t sm = (size_t)L * B * G3 * sizeof(C);
+        auto k = p3_z_conv_reg<T, L, B, G3>;
+        set_smem(k, sm);
+        k<<<grid3, B * G3 * tpl_of<T, L>(), sm, st>>>(d, S2, tens);
+    } else if constexpr (sizeof(T) == 4 || L >= 2048) {
+        // classic, and lines of more butterflies than a CTA of the line engine holds
         dim3 grid((d.KX + B - 1) / B, (kyi + G - 1) / G, d.nb);
         const size_t sm = 3 * (size_t)L * B * G * sizeof(C);
         auto k = p3_z_conv<T, L, B, G>;
@@ -2030,8 +2126,9 @@ template <typename T, int L> static void launch_x_fwd(const DemagDims& d, const 
     in.m = m;
     in.Ms_cell = Ms_cell;
     in.Ms = Ms;
-    if (launch_line_x_fwd<T>(d, in, S1, st)) return;
-    if constexpr (L < 16 || L >= 2048) launch_p1<T, L>(d, m, Ms_cell, Ms, S1, st);   // too short or long for the engine
+    if (!d.classic && launch_line_x_fwd<T>(d, in, S1, st)) return;
+    // lines too short or too long for the engine, and the classic FP32 passes
+    if constexpr (sizeof(T) == 4 || L < 16 || L >= 2048) launch_p1<T, L>(d, m, Ms_cell, Ms, S1, st);
 }
 
 template <typename T, int L> static void launch_x_inv(const DemagDims& d, const typename Cplx<T>::type* S1, T* h,
@@ -2039,8 +2136,8 @@ template <typename T, int L> static void launch_x_inv(const DemagDims& d, const 
     if constexpr (sizeof(T) == 4 && L >= 16 && is_pow2(L)) {
         if (launch_p5_tma<L>(d, S1, h, st)) return;
     }
-    if (launch_line_x_inv<T>(d, S1, h, st)) return;
-    if constexpr (L < 16 || L >= 2048) launch_p5<T, L>(d, S1, h, st);
+    if (!d.classic && launch_line_x_inv<T>(d, S1, h, st)) return;
+    if constexpr (sizeof(T) == 4 || L < 16 || L >= 2048) launch_p5<T, L>(d, S1, h, st);
 }
 
 // fused K5 launcher (see k5_fused): false if the shape or material does not qualify
@@ -2187,7 +2284,7 @@ static void launch_p3_layers(const DemagDims& d, typename Cplx<T>::type* S2, con
 // multiply run as one pass of the z-pass kernels along y (32 served 256x256x1
 // grids: 88 us against 103 us for two y passes and the product; longer lines
 // leave a CTA of the line engine one column, less than a sector of each row)
-constexpr int k2dMaxPy = 1024;
+constexpr int k2dMaxPy = 1024, k2dClassicPy = 256;
 
 template <typename T>
 static void yzy(const DemagDims& d, typename Cplx<T>::type* S1, typename Cplx<T>::type* S2, const T* tens,
@@ -2210,7 +2307,7 @@ static void yzy(const DemagDims& d, typename Cplx<T>::type* S1, typename Cplx<T>
         }
         return;
     }
-    if (d.nz == 1 && d.LY > 1 && d.LY <= k2dMaxPy) {
+    if (d.nz == 1 && d.LY > 1 && d.LY <= (d.classic ? k2dClassicPy : k2dMaxPy)) {
         DemagDims d2 = d;
         d2.ny = 1; d2.nz = d.ny; d2.LY = 1; d2.LZ = d.LY; d2.yz_swap = 1;
         tm->begin(st, "p3_z_conv");

@@ -449,7 +449,7 @@ void launch_rt_x_fwd(const DemagDims& d, const T* m, const T* Ms_cell, T Ms, typ
                      cudaStream_t st) {
     LineXIn<T> in;
     in.m = m; in.Ms_cell = Ms_cell; in.Ms = Ms;
-    if (launch_line_x_fwd<T>(d, in, S1, st)) return;
+    if (!d.classic && launch_line_x_fwd<T>(d, in, S1, st)) return;
     using C = typename Cplx<T>::type;
     const RtPlan pl = make_plan(d.LX);
     const int NL = rt_lines(d.LX, sizeof(C), 2, kRtMaxLines);
@@ -462,7 +462,7 @@ void launch_rt_x_fwd(const DemagDims& d, const T* m, const T* Ms_cell, T Ms, typ
 
 template <typename T>
 void launch_rt_x_inv(const DemagDims& d, const typename Cplx<T>::type* S1, T* h, cudaStream_t st) {
-    if (launch_line_x_inv<T>(d, S1, h, st)) return;
+    if (!d.classic && launch_line_x_inv<T>(d, S1, h, st)) return;
     using C = typename Cplx<T>::type;
     const RtPlan pl = make_plan(d.LX);
     const int NL = rt_lines(d.LX, sizeof(C), 2, kRtMaxLines);
@@ -515,6 +515,11 @@ template <typename T> bool line_shape(int L, long ncol, int nb, int nc, bool con
     o->ctas = (ncol + (1 << lb) - 1) >> lb;
     return true;
 }
+
+// Whether a launch lets the next one start beside it at once: FP32 grids that
+// leave room on the chip.  FP64 CTAs placed while the previous grid still runs
+// crowd on the SMs that finish first, and FP64 time is the fullest SM's.
+template <typename T> int line_early(long ctas) { return sizeof(T) == 4 && ctas <= 304; }
 
 template <typename... KArgs, typename... Args>
 void line_launch(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args&&... args) {
@@ -600,7 +605,7 @@ bool launch_line_x_fwd(const DemagDims& d, const LineXIn<T>& in, typename Cplx<T
         if (o.ct) line_ct_use(kLineXFwd, d.LX, &k);
     }
     line_launch(k, dim3((unsigned)o.ctas, d.nb), o.threads, o.smem, st, d, f, S1, o.pl, line_table<T>(o.pl), o.nt, o.lines,
-                (int)(o.ctas * d.nb <= 304));
+                line_early<T>(o.ctas * d.nb));
     return true;
 }
 
@@ -614,7 +619,7 @@ bool launch_line_x_inv(const DemagDims& d, const typename Cplx<T>::type* S1, T* 
         if (o.ct) line_ct_use(kLineXInv, d.LX, &k);
     }
     line_launch(k, dim3((unsigned)o.ctas, d.nb), o.threads, o.smem, st, d, S1, h, o.pl, line_table<T>(o.pl), o.nt, o.lines,
-                (int)(o.ctas * d.nb <= 304));
+                line_early<T>(o.ctas * d.nb));
     return true;
 }
 
@@ -638,7 +643,7 @@ bool launch_line_fused(const DemagDims& d, float2* S1, const StageParams<float>&
     const size_t smem = o.smem + (size_t)o.lines * park * d.nx * sizeof(float2);
     line_launch(k, dim3((unsigned)o.ctas, d.nb), o.threads, smem, st, d, S1, p, b, o.pl, line_table<float>(o.pl), o.nt,
                 o.lines, park, (int)fwd,
-                (int)(o.ctas * d.nb <= 304));
+                line_early<float>(o.ctas * d.nb));
     return true;
 }
 
@@ -665,7 +670,7 @@ bool launch_line_y(const DemagDims& d, const typename Cplx<T>::type* in, typenam
         if (line_ct_use(DIR < 0 ? kLineYFwd : kLineYInv, d.LY, &k)) line_ct_shape(d.LY, ncol, &o);
     }
     line_launch(k, dim3((unsigned)o.ctas, d.nb), o.threads, o.smem, st, d, in, out, o.pl, line_table<T>(o.pl), o.lb, (int)ncol,
-                (int)(o.ctas * d.nb <= 304));
+                line_early<T>(o.ctas * d.nb));
     return true;
 }
 
@@ -675,21 +680,31 @@ bool launch_line_conv(const DemagDims& d, typename Cplx<T>::type* S2, const T* t
     const long ncol = (long)d.KX * d.LY;
     if (d.nb > 65535 || !line_shape<T>(d.LZ, ncol, d.nb, 3, true, &o)) return false;
     constexpr int kSmall = sizeof(T) == 4 ? kLineThreads32 : kLineThreads;
-    auto k = o.pl.np == 1 ? line_conv<T, true, kLineThreads, 0>
-             : o.threads > kSmall ? line_conv<T, false, kLineThreads, 0> : line_conv<T, false, kSmall, 0>;
+    const int M = o.pl.np ? d.LZ / o.pl.rmin : 0;
+    const bool split = o.pl.np > 1 && line_split<T>(M);
+    if (split) {
+        o.lb = line_split_lb<T>(M);
+        o.threads = (((3 * M) << o.lb) + 31) / 32 * 32;
+        o.smem = (size_t)3 * line_len(d.LZ) * (2 * sizeof(T) << o.lb);
+        o.ctas = (ncol + (1 << o.lb) - 1) >> o.lb;
+    }
+    auto k = o.pl.np == 1 ? line_conv<T, kConvOne, 256, 0>
+             : o.threads > kSmall ? line_conv<T, kConvThree, kLineThreads, 0> : line_conv<T, kConvThree, kSmall, 0>;
     if constexpr (sizeof(T) == 4) {
         if (o.pl.np > 1 && line_ct_use(kLineConv, d.LZ, &k)) line_ct_shape(d.LZ, ncol, &o);
+    } else if (split) {
+        k = o.threads <= 384 ? line_conv<T, kConvSplit, 384, 0> : line_conv<T, kConvSplit, 768, 0>;
     }
     const dim3 grid((unsigned)o.ctas, d.nb);
     line_launch(k, grid, o.threads, o.smem, st, d, S2, tens, o.pl, line_table<T>(o.pl), o.lb, (int)ncol,
-                (int)(o.ctas * d.nb <= 304));
+                line_early<T>(o.ctas * d.nb));
     return true;
 }
 
 template <typename T, int DIR>
 void launch_rt_y(const DemagDims& d, const typename Cplx<T>::type* in, typename Cplx<T>::type* out,
                  cudaStream_t st) {
-    if (launch_line_y<T, DIR>(d, in, out, st)) return;
+    if (!d.classic && launch_line_y<T, DIR>(d, in, out, st)) return;
     using C = typename Cplx<T>::type;
     const RtPlan pl = make_plan(d.LY);
     const int B = rt_lines(d.LY, sizeof(C), 2, (int)(128 / sizeof(C)));
@@ -702,7 +717,7 @@ void launch_rt_y(const DemagDims& d, const typename Cplx<T>::type* in, typename 
 
 template <typename T>
 void launch_rt_z(const DemagDims& d, typename Cplx<T>::type* S2, const T* tens, cudaStream_t st) {
-    if (launch_line_conv<T>(d, S2, tens, st)) return;
+    if (!d.classic && launch_line_conv<T>(d, S2, tens, st)) return;
     using C = typename Cplx<T>::type;
     const RtPlan pl = make_plan(d.LZ);
     const int B = rt_lines(d.LZ, sizeof(C), 4, (int)(128 / sizeof(C)));

@@ -20,8 +20,8 @@
 // half of a forward's input, and the dropped half of an inverse's output, are
 // the registers q >= R/2 of that pass.
 //
-// Twiddled radix-2 steps are folded as X = a + w b (four multiply-adds) and
-// Y = 2 a - X (two): 3 instructions per point and level against 3.5 for
+// Twiddled radix-2 steps are folded into multiply-adds: X = a + w b (four) and,
+// in FP64, Y = 2 a - X (two), 3 instructions per point and level against 3.5 for
 // radix-8 passes that multiply first.  FP64 instructions are what an FP64
 // pass spends its time on (one warp instruction per 19 cycles and SM; 64
 // cycles for a single warp of a quarter SM, dependent or not), so FP64 plans
@@ -95,7 +95,18 @@ constexpr LinePlan line_plan(int L, int rmax) {
 }
 template <typename T> constexpr int line_rmax() { return sizeof(T) == 4 ? 8 : 4; }
 template <typename T> __host__ __device__ constexpr LinePlan line_ct(int L) { return line_plan(L, line_rmax<T>()); }
-// columns per CTA (log2) of a compiled length: a sector of each row at least, and two warps
+// FP64 z lines whose three components fit a CTA side by side take a thread per
+// butterfly and component (32x32x4: 9.5 -> 6.6 us, 128x128x32: 416 -> 393 us; in
+// FP32 the extra exchange costs more than the threads bring: 32 grids of
+// 256x256x1 105 against 68 us).  M: butterflies of the widest pass.
+template <typename T> __host__ __device__ constexpr bool line_split(int M) { return sizeof(T) == 8 && M <= 128; }
+// their columns per CTA (log2): a sector of each row at least, and three warps
+template <typename T> __host__ __device__ constexpr int line_split_lb(int M) {
+    int lb = sizeof(T) == 4 ? 2 : 1;
+    while (lb < 5 && ((3 * M) << lb) < 96) ++lb;
+    return lb;
+}
+// columns per CTA (log2) of a compiled length otherwise: a sector of each row at least, and two warps
 template <typename T> __host__ __device__ constexpr int line_ct_lb(int L) {
     const LinePlan p = line_ct<T>(L);
     int lb = sizeof(T) == 4 ? 2 : 1;
@@ -117,11 +128,15 @@ __device__ __forceinline__ int line_mod(int b, int Ns, unsigned mg) {
 template <int SH> __host__ __device__ __forceinline__ int line_place(int e) { return e + (e >> SH); }
 __host__ __device__ __forceinline__ int line_len(int L) { return L + (L >> 3) + 1; }
 
-// x = a + w b, y = a - w b
+// x = a + w b, y = a - w b.  FP64 forms y = 2 a - x (six instructions in all);
+// FP32, which is not bound by them, forms both directly: 2 a - x would carry the
+// rounding of a large x into a small y, as the spectrum of a nearly uniform
+// magnetisation has them side by side.
 template <typename C> __device__ __forceinline__ void bf2(C& a, C& b, C w) {
     using T = decltype(C::x);
     const C x = mk<C>(fma(w.x, b.x, fma(-w.y, b.y, a.x)), fma(w.x, b.y, fma(w.y, b.x, a.y)));
-    b = mk<C>(fma((T)2, a.x, -x.x), fma((T)2, a.y, -x.y));
+    if constexpr (sizeof(T) == 4) b = mk<C>(fma(-w.x, b.x, fma(w.y, b.y, a.x)), fma(-w.x, b.y, fma(-w.y, b.x, a.y)));
+    else b = mk<C>(fma((T)2, a.x, -x.x), fma((T)2, a.y, -x.y));
     a = x;
 }
 // the same with w replaced by DIR i w
@@ -252,6 +267,22 @@ __device__ __forceinline__ void line_mid(typename Cplx<T>::type* s, int plane, i
     line_butterfly<T, DIR>(x, tw, k, L / (Ns * R), L);
     __syncthreads();
     if (on) line_store<SH>(x, s, plane, lb, b, k, Ns);
+    __syncthreads();
+}
+
+// a first pass in place: no twiddles, any input
+template <typename T, int DIR, int R, int NC, int SH>
+__device__ __forceinline__ void line_start(typename Cplx<T>::type* s, int plane, int lb, int b, int L) {
+    using C = typename Cplx<T>::type;
+    const int M = L / R;
+    const bool on = b < M;
+    if (!on) b = 0;
+    C x[NC][R];
+    line_load<SH>(x, s, plane, lb, b, M);
+#pragma unroll
+    for (int c = 0; c < NC; ++c) line_dft<DIR, R, false>(x[c]);
+    __syncthreads();
+    if (on) line_store<SH>(x, s, plane, lb, b, 0, 1);
     __syncthreads();
 }
 

@@ -739,25 +739,35 @@ __device__ __forceinline__ void line_last(const typename Cplx<T>::type* s, int p
     }
 }
 
+// -v or v; FP64 on the integer side (FP64 instructions are what an FP64 pass is made of)
+__device__ __forceinline__ float line_flip(float v, bool neg) { return neg ? -v : v; }
+__device__ __forceinline__ double line_flip(double v, bool neg) {
+    return __hiloint2double(__double2hiint(v) ^ (neg ? (int)0x80000000 : 0), __double2loint(v));
+}
+
+// h^ = T M^ of one wave number; t: the octant's xx, xy, xz, yy, yz, zz; ny, nz:
+// whether the odd components along y and along z change sign here
+template <typename T, typename C>
+__device__ __forceinline__ void line_mul(const T (&t)[6], bool ny, bool nz, C& x, C& y, C& z) {
+    const T txy = line_flip(t[1], ny), txz = line_flip(t[2], nz), tyz = line_flip(t[4], ny != nz);
+    const C mx = x, my = y, mz = z;
+    x = mk<C>(t[0] * mx.x + txy * my.x + txz * mz.x, t[0] * mx.y + txy * my.y + txz * mz.y);
+    y = mk<C>(txy * mx.x + t[3] * my.x + tyz * mz.x, txy * mx.y + t[3] * my.y + tyz * mz.y);
+    z = mk<C>(txz * mx.x + tyz * my.x + t[5] * mz.x, txz * mx.y + tyz * my.y + t[5] * mz.y);
+}
+
 // h^ = T M^ at the R wave numbers b + q M of one column; tp points at the
 // column's folded ky row, tz between kz planes, tc between components
 template <typename T, int R>
 __device__ __forceinline__ void line_tensor(typename Cplx<T>::type (&x)[3][R], const T* __restrict__ tp, long tz, long tc,
-                                            int b, int M, int L, T sy, int swap) {
-    using C = typename Cplx<T>::type;
+                                            int b, int M, int L, bool sy, int swap) {
 #pragma unroll
     for (int q = 0; q < R; ++q) {
         const int kz = b + q * M;
-        const bool up = 2 * kz > L;
-        const T* t = tp + (up ? L - kz : kz) * tz;
-        const T sz = up ? (T)-1 : (T)1;
-        const T txx = t[0], tyy = t[3 * tc], tzz = t[5 * tc];
-        const T txy = (swap ? sz : sy) * t[tc], txz = (swap ? sy : sz) * t[2 * tc];
-        const T tyz = sy * sz * t[4 * tc];
-        const C mx = x[0][q], my = x[1][q], mz = x[2][q];
-        x[0][q] = mk<C>(txx * mx.x + txy * my.x + txz * mz.x, txx * mx.y + txy * my.y + txz * mz.y);
-        x[1][q] = mk<C>(txy * mx.x + tyy * my.x + tyz * mz.x, txy * mx.y + tyy * my.y + tyz * mz.y);
-        x[2][q] = mk<C>(txz * mx.x + tyz * my.x + tzz * mz.x, txz * mx.y + tyz * my.y + tzz * mz.y);
+        const bool sz = 2 * kz > L;
+        const T* g = tp + (sz ? L - kz : kz) * tz;
+        const T t[6] = {g[0], g[tc], g[2 * tc], g[3 * tc], g[4 * tc], g[5 * tc]};
+        line_mul(t, swap ? sz : sy, swap ? sy : sz, x[0][q], x[1][q], x[2][q]);
     }
 }
 
@@ -765,7 +775,7 @@ __device__ __forceinline__ void line_tensor(typename Cplx<T>::type (&x)[3][R], c
 template <typename T, int R>
 __device__ __forceinline__ void line_product(typename Cplx<T>::type* s, int plane, int lb, int b, int L, int Ns,
                                              unsigned mg, const typename Cplx<T>::type* tw, const T* tp, long tz, long tc,
-                                             T sy, int swap) {
+                                             bool sy, int swap) {
     using C = typename Cplx<T>::type;
     const int M = L / R;
     const bool on = b < M;
@@ -784,7 +794,7 @@ __device__ __forceinline__ void line_product(typename Cplx<T>::type* s, int plan
 // the whole column in one thread's registers (L = R)
 template <typename T, int R>
 __device__ __forceinline__ void line_product_one(typename Cplx<T>::type* g, long es, long cs, int n, const T* tp,
-                                                 long tz, long tc, T sy, int swap) {
+                                                 long tz, long tc, bool sy, int swap) {
     using C = typename Cplx<T>::type;
     constexpr int H = R == 1 ? 1 : R / 2;
     C x[3][R];
@@ -816,18 +826,27 @@ __device__ __forceinline__ void line_product_one(typename Cplx<T>::type* g, long
 // blockIdx.y is the grid of a batch.
 // (The tensor slice copied to shared memory during the forward passes measured
 // slower, 90 against 80 us on 32 grids of 256x256x1: fewer CTAs per SM.)
-template <typename T, bool ONE, int MAXT, int LC>
-__global__ void __launch_bounds__(MAXT, LC > 0 && MAXT == kLineThreads32 ? 2 : line_blocks<T, MAXT>())
+// FORM: kConvOne, a column in one thread's registers; kConvThree, a thread per
+// butterfly of all three components; kConvSplit, a thread per butterfly and
+// component, the product then taken wave number by wave number by all of them.
+enum { kConvOne, kConvThree, kConvSplit };
+template <typename T, int FORM, int MAXT, int LC>
+__global__ void __launch_bounds__(MAXT, FORM == kConvSplit ? (MAXT <= 384 ? 2 : 1) : FORM == kConvOne ? 2 : LC > 0 && MAXT == kLineThreads32 ? 2 : line_blocks<T, MAXT>())
 line_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restrict__ tens,
           const __grid_constant__ LinePlan pl, const typename Cplx<T>::type* __restrict__ tw, int lb, int ncol, int early) {
     using C = typename Cplx<T>::type;
     extern __shared__ __align__(16) unsigned char smraw[];
     const int L = LC ? LC : pl.L, tid = threadIdx.x;
+    int M = L / pl.rmin;
     if constexpr (LC > 0) {
-        constexpr int kLb = line_ct_lb<T>(LC);
+        constexpr int kM = LC / line_ct<T>(LC).rmin;
+        constexpr int kLb = FORM == kConvSplit ? line_split_lb<T>(kM) : line_ct_lb<T>(LC);
+        M = kM;
         lb = kLb;
     }
-    const int l = tid & ((1 << lb) - 1), b = tid >> lb;
+    const int l = tid & ((1 << lb) - 1), u = tid >> lb;
+    const int c = FORM == kConvSplit ? min(u / M, 2) : 0;
+    const int b = FORM != kConvSplit ? u : u < 3 * M ? u - c * M : kLineIdle;
     const int col = (blockIdx.x << lb) + l;
     const bool valid = col < ncol;
     const int cc = valid ? col : ncol - 1;      // columns past the end follow the last one and store nothing
@@ -838,19 +857,72 @@ line_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restr
     C* g = S2 + (long)blockIdx.y * 3 * cs + (long)ky * d.KXS + kx;
     const long tz = (long)KY2 * d.KXS, tc = (long)(L / 2 + 1) * tz;
     const T* tp = tens + (long)(up ? LY - ky : ky) * d.KXS + kx;
-    const T sy = up ? (T)-1 : (T)1;
     if (early) grid_dep_launch();
+    if constexpr (FORM == kConvSplit) {
+        // this thread's wave numbers u + 3 M i; their tensor entries (written long
+        // before the previous pass) are on their way from the start
+        constexpr int KP = sizeof(T) == 4 ? 3 : 2;      // the smallest radix of a plan is 8, or 4, at most
+        T t[KP][6];
+#pragma unroll
+        for (int i = 0; i < KP; ++i) {
+            const int kz = min(u + 3 * M * i, L - 1);
+            const T* q = tp + (2 * kz > L ? L - kz : kz) * tz;
+#pragma unroll
+            for (int j = 0; j < 6; ++j) t[i][j] = __ldg(q + j * tc);
+        }
+        grid_dep_wait();
+        C* s0 = reinterpret_cast<C*>(smraw) + l;
+        const int plane = line_len(L) << lb;
+        C* s = s0 + c * plane;
+        g += c * cs;
+        auto product = [&]() {
+#pragma unroll
+            for (int i = 0; i < KP; ++i) {
+                const int kz = u + 3 * M * i;
+                if (u < 3 * M && kz < L) {
+                    C* q = s0 + (line_place<3>(kz) << lb);
+                    const bool sz = 2 * kz > L;
+                    C x = q[0], y = q[plane], z = q[2 * plane];
+                    line_mul(t[i], d.yz_swap ? sz : up, d.yz_swap ? up : sz, x, y, z);
+                    q[0] = x; q[plane] = y; q[2 * plane] = z;
+                }
+            }
+            __syncthreads();
+        };
+        if constexpr (LC > 0) {
+            constexpr LinePlan P = line_ct<T>(LC);
+            constexpr int np = P.np;
+            line_first<T, -1, P.R[0], true, 1>(g, zs, 0, d.nz, s, 0, lb, b, L);
+            __syncthreads();
+            line_mids_ct<T, -1, 1, 3, LC, 1, np>(s, 0, lb, b, tw);
+            product();
+            line_start<T, +1, P.R[np - 1], 1, 3>(s, 0, lb, b, L);
+            line_mids_ct<T, +1, 1, 3, LC, 1, np - 1>(s, 0, lb, b, tw);
+            line_last<T, +1, P.R[0], true, 1>(s, 0, lb, b, L, P.Nsi[np - 1], 0, tw, g, zs, 0, d.nz, valid);
+        } else {
+            const int np = pl.np;
+            MM_LINE_RADIX_EVEN(T, pl.R[0], (line_first<T, -1, R_, true, 1>(g, zs, 0, d.nz, s, 0, lb, b, L)));
+            __syncthreads();
+            for (int i = 1; i < np; ++i) line_mid_any<T, -1, 1, 3>(s, 0, lb, b, pl, i, tw);
+            product();
+            MM_LINE_RADIX(T, pl.R[np - 1], (line_start<T, +1, R_, 1, 3>(s, 0, lb, b, L)));
+            for (int i = 1; i < np - 1; ++i) line_mid_any<T, +1, 1, 3>(s, 0, lb, b, pl, i, tw);
+            MM_LINE_RADIX_EVEN(T, pl.R[0], (line_last<T, +1, R_, true, 1>(s, 0, lb, b, L, pl.Nsi[np - 1], pl.mgi[np - 1],
+                                                                          tw, g, zs, 0, d.nz, valid)));
+        }
+        return;
+    }
     grid_dep_wait();
-    if constexpr (ONE) {
+    if constexpr (FORM == kConvOne) {
         if (!valid) return;
         switch (L) {
-            case 1: line_product_one<T, 1>(g, zs, cs, d.nz, tp, tz, tc, sy, d.yz_swap); break;
-            case 2: line_product_one<T, 2>(g, zs, cs, d.nz, tp, tz, tc, sy, d.yz_swap); break;
-            case 4: line_product_one<T, 4>(g, zs, cs, d.nz, tp, tz, tc, sy, d.yz_swap); break;
-            case 6: line_product_one<T, sizeof(T) == 4 ? 6 : 1>(g, zs, cs, d.nz, tp, tz, tc, sy, d.yz_swap); break;
-            case 8: line_product_one<T, sizeof(T) == 4 ? 8 : 1>(g, zs, cs, d.nz, tp, tz, tc, sy, d.yz_swap); break;
-            case 12: line_product_one<T, sizeof(T) == 4 ? 12 : 1>(g, zs, cs, d.nz, tp, tz, tc, sy, d.yz_swap); break;
-            default: line_product_one<T, sizeof(T) == 4 ? 16 : 1>(g, zs, cs, d.nz, tp, tz, tc, sy, d.yz_swap); break;
+            case 1: line_product_one<T, 1>(g, zs, cs, d.nz, tp, tz, tc, up, d.yz_swap); break;
+            case 2: line_product_one<T, 2>(g, zs, cs, d.nz, tp, tz, tc, up, d.yz_swap); break;
+            case 4: line_product_one<T, 4>(g, zs, cs, d.nz, tp, tz, tc, up, d.yz_swap); break;
+            case 6: line_product_one<T, sizeof(T) == 4 ? 6 : 1>(g, zs, cs, d.nz, tp, tz, tc, up, d.yz_swap); break;
+            case 8: line_product_one<T, sizeof(T) == 4 ? 8 : 1>(g, zs, cs, d.nz, tp, tz, tc, up, d.yz_swap); break;
+            case 12: line_product_one<T, sizeof(T) == 4 ? 12 : 1>(g, zs, cs, d.nz, tp, tz, tc, up, d.yz_swap); break;
+            default: line_product_one<T, sizeof(T) == 4 ? 16 : 1>(g, zs, cs, d.nz, tp, tz, tc, up, d.yz_swap); break;
         }
     } else {
         C* s = reinterpret_cast<C*>(smraw) + l;
@@ -861,7 +933,7 @@ line_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restr
             line_first<T, -1, P.R[0], true, 3>(g, zs, cs, d.nz, s, plane, lb, b, L);
             __syncthreads();
             line_mids_ct<T, -1, 3, 3, LC, 1, np - 1>(s, plane, lb, b, tw);
-            line_product<T, P.R[np - 1]>(s, plane, lb, b, L, P.Ns[np - 1], 0, tw, tp, tz, tc, sy, d.yz_swap);
+            line_product<T, P.R[np - 1]>(s, plane, lb, b, L, P.Ns[np - 1], 0, tw, tp, tz, tc, up, d.yz_swap);
             line_mids_ct<T, +1, 3, 3, LC, 1, np - 1>(s, plane, lb, b, tw);
             line_last<T, +1, P.R[0], true, 3>(s, plane, lb, b, L, P.Nsi[np - 1], 0, tw, g, zs, cs, d.nz, valid);
         } else {
@@ -870,7 +942,7 @@ line_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restr
             const int np = pl.np;
             for (int i = 1; i < np - 1; ++i) line_mid_any<T, -1, 3, 3>(s, plane, lb, b, pl, i, tw);
             MM_LINE_RADIX(T, pl.R[np - 1], (line_product<T, R_>(s, plane, lb, b, L, pl.Ns[np - 1], pl.mg[np - 1], tw, tp,
-                                                                tz, tc, sy, d.yz_swap)));
+                                                                tz, tc, up, d.yz_swap)));
             for (int i = 1; i < np - 1; ++i) line_mid_any<T, +1, 3, 3>(s, plane, lb, b, pl, i, tw);
             MM_LINE_RADIX_EVEN(T, pl.R[0], (line_last<T, +1, R_, true, 3>(s, plane, lb, b, L, pl.Nsi[np - 1],
                                                                           pl.mgi[np - 1], tw, g, zs, cs, d.nz, valid)));
@@ -947,7 +1019,7 @@ template <int LC> const void* line_ct_pick(LineKind kind) {
         case kLineFusedGen: return (const void*)line_fused<true, FT, LC>;
         case kLineXFwd: return (const void*)line_x_forward<float, 1, 256, LC>;
         case kLineXInv: return (const void*)line_x_inverse<float, 1, 256, LC>;
-        case kLineConv: return (const void*)line_conv<float, false, YT, LC>;
+        case kLineConv: return (const void*)line_conv<float, kConvThree, YT, LC>;
         case kLineYFwd: return (const void*)line_y<float, -1, 3, YT, LC>;
         default: return (const void*)line_y<float, +1, 3, YT, LC>;
     }

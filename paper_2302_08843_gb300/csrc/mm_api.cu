@@ -351,7 +351,7 @@ mm_status read_scalars(mm_state* s) {
 // whether this state's evaluations run the line engine's fused stage (FP32
 // with a demag term and x lines the engine takes)
 template <typename T> bool line_path(const mm_state* s) {
-    if constexpr (sizeof(T) == 4) return !s->demag_off && s->demag_ready && line_fused_blocks(s->d, 1L << 40) > 0;
+    if constexpr (sizeof(T) == 4) return !s->d.classic && !s->demag_off && s->demag_ready && line_fused_blocks(s->d, 1L << 40) > 0;
     return false;
 }
 
@@ -540,6 +540,11 @@ template <typename T> mm_status rk4_impl(mm_state* s, double dt, double t) {
     void* in[4] = {s->m, s->mA, s->mB, s->mA};
     void* out[4] = {s->mA, s->mB, s->mA, s->m};
     const bool fresh = s->s1_fresh;         // S1 from the last step's end
+    struct Classic {                        // for this step only (see DemagDims)
+        DemagDims& d;
+        ~Classic() { d.classic = 0; }
+    } classic{s->d};
+    s->d.classic = sizeof(T) == 4 && s->zw != nullptr;
     const bool line = line_path<T>(s);
     for (int st = 0; st < 4; ++st) {
         StageParams<T> p;
