@@ -248,6 +248,33 @@ __global__ void batch_control_kernel(const double* __restrict__ scal, int* __res
     }
 }
 
+// A slot's control state, material and field terms in one launch, from its
+// arguments, where there were a dozen copies of a few bytes (loading 32 slots of
+// 64x64x1 from the host 1000 -> 610 us, clearing them 307 -> 81 us).
+template <typename T> __global__ void batch_slot_kernel(BatchSlot<T> p) {
+    const int i = p.slot;
+    if (p.what != kSlotClear) {
+        p.D[i] = p.vD;
+        p.pc[i] = p.vpc;
+        p.kind[i] = p.vkind;
+    }
+    if (p.what == kSlotTerms) return;
+    p.status[i] = p.fresh[i] = p.what == kSlotLoad;
+    if (p.what == kSlotClear) return;
+    p.Ms[i] = p.vMs;
+    p.A[i] = p.vA;
+    p.alpha[i] = p.valpha;
+    p.steps[i] = 0;
+    p.dt[i] = p.vdt;
+    p.t[i] = p.torque[i] = 0.0;
+}
+
+template <typename T> void launch_batch_slot(const BatchSlot<T>& p, cudaStream_t st) {
+    batch_slot_kernel<T><<<1, 1, 0, st>>>(p);
+}
+template void launch_batch_slot<float>(const BatchSlot<float>&, cudaStream_t);
+template void launch_batch_slot<double>(const BatchSlot<double>&, cudaStream_t);
+
 void launch_batch_masks(const int* status, const int* fresh, int* mask, int cap, cudaStream_t st) {
     batch_masks_kernel<<<(cap + 127) / 128, 128, 0, st>>>(status, fresh, mask, cap);
 }

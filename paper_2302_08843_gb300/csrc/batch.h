@@ -52,4 +52,17 @@ void launch_batch_control(const double* scal, int* run, int* status, int* steps,
 template <typename T> void launch_batch_accept(const T* y5, const T* k7, const int* acc, T* m, T* k1, int N, int nb,
                                                cudaStream_t st);
 
+// one slot's device-side entries and the values to put there
+enum { kSlotLoad, kSlotTerms, kSlotClear };
+template <typename T> struct BatchSlot {
+    int slot, what;
+    T *Ms, *A, *alpha, *D, *pc;
+    int *kind, *status, *steps, *fresh;
+    double *dt, *t, *torque;
+    T vMs, vA, valpha, vD, vpc;
+    int vkind;
+    double vdt;
+};
+template <typename T> void launch_batch_slot(const BatchSlot<T>& p, cudaStream_t st);
+
 }  // namespace mm

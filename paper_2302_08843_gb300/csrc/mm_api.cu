@@ -1087,6 +1087,29 @@ template <typename T> mm_status batch_attempts(mm_batch* b, int attempts, double
     return MM_OK;
 }
 
+template <typename T>
+void batch_slot_as(mm_batch* b, int slot, int what, double Ms, double A, double alpha, double D, double pc, int kind,
+                   double dt) {
+    BatchSlot<T> p;
+    p.slot = slot; p.what = what;
+    p.Ms = (T*)b->Ms_d; p.A = (T*)b->A_d; p.alpha = (T*)b->alpha_d; p.D = (T*)b->D_d; p.pc = (T*)b->pc_d;
+    p.kind = b->kind_d; p.status = b->status_d(); p.steps = b->steps_d(); p.fresh = b->fresh_d();
+    p.dt = b->dt_d(); p.t = b->t_d(); p.torque = b->torque_d();
+    p.vMs = (T)Ms; p.vA = (T)A; p.valpha = (T)alpha; p.vD = (T)D; p.vpc = (T)pc;
+    p.vkind = kind;
+    p.vdt = dt;
+    launch_batch_slot<T>(p, b->st);
+}
+
+// a slot's device-side entries, on the batch's stream
+mm_status batch_slot(mm_batch* b, int slot, int what, double Ms, double A, double alpha, double D, double pc, int kind,
+                     double dt) {
+    if (b->prec == MM_FP64) batch_slot_as<double>(b, slot, what, Ms, A, alpha, D, pc, kind, dt);
+    else batch_slot_as<float>(b, slot, what, Ms, A, alpha, D, pc, kind, dt);
+    MM_LAUNCHED();
+    return MM_OK;
+}
+
 void batch_drop_graphs(mm_batch* b) {
     for (auto& kv : b->graphs) cudaGraphExecDestroy(kv.second);
     b->graphs.clear();
@@ -1631,26 +1654,8 @@ mm_status mm_batch_set_slot(mm_batch* b, int slot, double Ms, double A, double a
     MM_CUDA(cudaMemcpyAsync(static_cast<char*>(b->m) + slot * v, m0, v,
                             on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, b->st));
     // the slot's material; no DMI and the precession term on until mm_batch_set_slot_terms
-    const double mat[5] = {Ms, A, alpha, 0.0, 1.0};
-    void* dst[5] = {b->Ms_d, b->A_d, b->alpha_d, b->D_d, b->pc_d};
-    MM_CUDA(cudaMemsetAsync(b->kind_d + slot, 0, sizeof(int), b->st));
-    for (int q = 0; q < 5; ++q) {
-        if (b->prec == MM_FP64) {
-            MM_CUDA(cudaMemcpyAsync(static_cast<double*>(dst[q]) + slot, &mat[q], 8, cudaMemcpyHostToDevice, b->st));
-        } else {
-            const float f = (float)mat[q];
-            MM_CUDA(cudaMemcpyAsync(static_cast<float*>(dst[q]) + slot, &f, 4, cudaMemcpyHostToDevice, b->st));
-        }
-    }
-    const int one = 1, zero = 0;
-    const double dt = dt0 > 0 ? dt0 : 1e-13, dz = 0.0;
-    MM_CUDA(cudaMemcpyAsync(b->status_d() + slot, &one, sizeof(int), cudaMemcpyHostToDevice, b->st));
-    MM_CUDA(cudaMemcpyAsync(b->steps_d() + slot, &zero, sizeof(int), cudaMemcpyHostToDevice, b->st));
-    MM_CUDA(cudaMemcpyAsync(b->fresh_d() + slot, &one, sizeof(int), cudaMemcpyHostToDevice, b->st));
-    MM_CUDA(cudaMemcpyAsync(b->dt_d() + slot, &dt, sizeof(double), cudaMemcpyHostToDevice, b->st));
-    MM_CUDA(cudaMemcpyAsync(b->t_d() + slot, &dz, sizeof(double), cudaMemcpyHostToDevice, b->st));
-    MM_CUDA(cudaMemcpyAsync(b->torque_d() + slot, &dz, sizeof(double), cudaMemcpyHostToDevice, b->st));
-    MM_CUDA(cudaStreamSynchronize(b->st));   // the host values above are stack copies
+    MM_TRY(batch_slot(b, slot, kSlotLoad, Ms, A, alpha, 0.0, 1.0, 0, dt0 > 0 ? dt0 : 1e-13));
+    MM_CUDA(cudaStreamSynchronize(b->st));   // the caller may reuse m0
     b->status[slot] = 1;
     b->special[slot] = Ms == 0.0 || (float)Ms == 0.f;
     b->unstarted[slot] = 1;
@@ -1667,18 +1672,8 @@ mm_status mm_batch_set_slot_terms(mm_batch* b, int slot, int dmi_kind, double D,
         return fail(MM_EINVAL, "bad DMI kind or strength");
     MM_CUDA(cudaSetDevice(b->device));
     const int kind = D != 0.0 ? dmi_kind : MM_DMI_NONE;
-    const double v[2] = {D, precession ? 1.0 : 0.0};
-    void* dst[2] = {b->D_d, b->pc_d};
-    for (int q = 0; q < 2; ++q) {
-        if (b->prec == MM_FP64) {
-            MM_CUDA(cudaMemcpyAsync(static_cast<double*>(dst[q]) + slot, &v[q], 8, cudaMemcpyHostToDevice, b->st));
-        } else {
-            const float f = (float)v[q];
-            MM_CUDA(cudaMemcpyAsync(static_cast<float*>(dst[q]) + slot, &f, 4, cudaMemcpyHostToDevice, b->st));
-        }
-    }
-    MM_CUDA(cudaMemcpyAsync(b->kind_d + slot, &kind, sizeof(int), cudaMemcpyHostToDevice, b->st));
-    MM_CUDA(cudaStreamSynchronize(b->st));   // the host values above are stack copies
+    MM_TRY(batch_slot(b, slot, kSlotTerms, 0.0, 0.0, 0.0, D, precession ? 1.0 : 0.0, kind, 0.0));
+    MM_CUDA(cudaStreamSynchronize(b->st));
     if (kind != MM_DMI_NONE) b->special[slot] = 1;
     return MM_OK;
 }
@@ -1688,10 +1683,7 @@ mm_status mm_batch_clear_slot(mm_batch* b, int slot) {
     if (slot < 0 || slot >= b->cap) return fail(MM_EINVAL, "slot %d out of range", slot);
     if (b->pending) return fail(MM_EINVAL, "attempts are in flight: call mm_batch_end first");
     MM_CUDA(cudaSetDevice(b->device));
-    const int zero = 0;
-    MM_CUDA(cudaMemcpyAsync(b->status_d() + slot, &zero, sizeof(int), cudaMemcpyHostToDevice, b->st));
-    MM_CUDA(cudaMemcpyAsync(b->fresh_d() + slot, &zero, sizeof(int), cudaMemcpyHostToDevice, b->st));
-    MM_CUDA(cudaStreamSynchronize(b->st));
+    MM_TRY(batch_slot(b, slot, kSlotClear, 0.0, 0.0, 0.0, 0.0, 0.0, 0, 0.0));
     b->status[slot] = 0;
     b->unstarted[slot] = 0;
     return MM_OK;
