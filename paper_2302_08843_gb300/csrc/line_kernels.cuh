@@ -326,8 +326,22 @@ __device__ __forceinline__ float line_davg(float a, float b) {
 struct LineRed {
     float tq2, tq, en, ed;     // largest |m x h|^2 (uniform Ms) and |m x h| / Ms, error ratio en / ed
     int nf;
-    double e[5];
+    float2 e[5];               // energy sums, sum Ms m.h per term, as high and low parts
 };
+
+// Sums of FP32 products kept exact to 48 bits as high and low parts (products
+// and sums with their rounding errors: Dekker 1971, Knuth's two-sum): FP64
+// instructions run at 1/64 of the FP32 rate here, and an energy of 100x65x27
+// cells spent 20 of 35 us on them.
+__device__ __forceinline__ void line_acc(float2& s, float p, float e) {
+    const float t = __fadd_rn(s.x, p), z = __fsub_rn(t, s.x);
+    s.y = __fadd_rn(s.y, __fadd_rn(__fadd_rn(__fsub_rn(s.x, __fsub_rn(t, z)), __fsub_rn(p, z)), e));
+    s.x = t;
+}
+__device__ __forceinline__ void line_acc_prod(float2& s, float a, float b) {
+    const float p = __fmul_rn(a, b);
+    line_acc(s, p, __fmaf_rn(a, b, -p));
+}
 
 // One item: the cells (x, ya) and (x, yb) of the line's two rows as the lanes
 // of paired FP32 instructions.  ia, ib: their indices in the grid (ib = ia for
@@ -467,22 +481,25 @@ __device__ __forceinline__ void line_cells(const StageParams<float>& p, const Li
         }
     }
     if (GEN && p.want_energy) {
-        const double V = p.lvol ? p.lvol[z] : p.V;
-        auto dot = [&](int lane, float2 a, float2 b, float2 c) {
-            return lane ? (double)mx.y * a.y + (double)my.y * b.y + (double)mz.y * c.y
-                        : (double)mx.x * a.x + (double)my.x * b.x + (double)mz.x * c.x;
-        };
+        auto add = [&](int q, float2 a, float2 b, float2 c) {
 #pragma unroll
-        for (int lane = 0; lane < 2; ++lane) {
-            const float ms = lane ? Ms.y : Ms.x;
-            if ((lane && !two) || ms == 0.f) continue;
-            const double f = -0.5 * kMu0 * V * (double)ms;
-            red.e[0] += f * dot(lane, v[0], v[1], v[2]);
-            red.e[1] += f * dot(lane, hex, hey, hez);
-            red.e[2] += f * dot(lane, hax, hay, haz);
-            red.e[3] += 2.0 * f * dot(lane, hzx, hzy, hzz);
-            if (dmi) red.e[4] += f * dot(lane, hmx, hmy, hmz);
-        }
+            for (int lane = 0; lane < 2; ++lane) {
+                if (lane && !two) break;
+                float2 dot = f2s(0.f);
+                line_acc_prod(dot, lane ? mx.y : mx.x, lane ? a.y : a.x);
+                line_acc_prod(dot, lane ? my.y : my.x, lane ? b.y : b.x);
+                line_acc_prod(dot, lane ? mz.y : mz.x, lane ? c.y : c.x);
+                const float ms = lane ? Ms.y : Ms.x, h = __fadd_rn(dot.x, dot.y), l = __fadd_rn(__fsub_rn(dot.x, h), dot.y);
+                if (ms == 0.f) continue;
+                const float w = __fmul_rn(ms, h);
+                line_acc(red.e[q], w, __fadd_rn(__fmaf_rn(ms, h, -w), __fmul_rn(ms, l)));
+            }
+        };
+        add(0, v[0], v[1], v[2]);
+        add(1, hex, hey, hez);
+        add(2, hax, hay, haz);
+        add(3, hzx, hzy, hzz);
+        if (dmi) add(4, hmx, hmy, hmz);
     }
     if (p.h_out) st(p.h_out + off, hx, hy, hz);
     if (p.k_out) st(p.k_out + off, kx, ky, kz);
@@ -624,7 +641,7 @@ line_fused(DemagDims d, float2* __restrict__ S1, const __grid_constant__ StagePa
     red.tq2 = red.tq = red.en = 0.f;
     red.ed = 1.f;
     red.nf = 0;
-    for (int q = 0; q < 5; ++q) red.e[q] = 0.0;
+    for (int q = 0; q < 5; ++q) red.e[q] = f2s(0.f);
     if (r.on && t.in) {
 #pragma unroll 1
         for (int x = c * nt + t.b; x < nx; x += 3 * nt) {
@@ -645,6 +662,12 @@ line_fused(DemagDims d, float2* __restrict__ S1, const __grid_constant__ StagePa
         __shared__ int rn[MAXT / 32];
         __shared__ double re[MAXT / 32][5];
         const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+        double en[5] = {0, 0, 0, 0, 0};
+        if (GEN && p.want_energy) {
+            const double f = -0.5 * kMu0 * (p.lvol ? p.lvol[min(r.z, d.nz - 1)] : p.V);
+#pragma unroll
+            for (int q = 0; q < 5; ++q) en[q] = (q == 3 ? 2.0 : 1.0) * f * ((double)red.e[q].x + (double)red.e[q].y);
+        }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             const float n2 = __shfl_down_sync(0xffffffffu, red.en, o), d2 = __shfl_down_sync(0xffffffffu, red.ed, o);
@@ -653,14 +676,14 @@ line_fused(DemagDims d, float2* __restrict__ S1, const __grid_constant__ StagePa
             red.tq = fmaxf(red.tq, __shfl_down_sync(0xffffffffu, red.tq, o));
             if (GEN && p.want_energy) {
 #pragma unroll
-                for (int q = 0; q < 5; ++q) red.e[q] += __shfl_down_sync(0xffffffffu, red.e[q], o);
+                for (int q = 0; q < 5; ++q) en[q] += __shfl_down_sync(0xffffffffu, en[q], o);
             }
         }
         const int nf = __any_sync(0xffffffffu, red.nf);
         if (lane == 0) {
             rt[w][0] = red.tq2; rt[w][1] = red.tq; rt[w][2] = red.en; rt[w][3] = red.ed;
             rn[w] = nf;
-            for (int q = 0; q < 5; ++q) re[w][q] = red.e[q];
+            for (int q = 0; q < 5; ++q) re[w][q] = en[q];
         }
         __syncthreads();
         if (threadIdx.x == 0) {

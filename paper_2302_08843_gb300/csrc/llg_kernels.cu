@@ -74,8 +74,8 @@ template <typename T> struct Vec<T, 1> {
 
 constexpr int kBX = 64, kBY = 4;   // threads per block: 64 along x, 4 rows of y
 
-// 3-D launch: blockIdx.z = z, blockIdx.y * kBY + threadIdx.y = y,
-// (blockIdx.x * kBX + threadIdx.x) * VEC = first x of the thread's cells.
+// 3-D launch: blockIdx.z = z, blockIdx.y * blockDim.y + threadIdx.y = y,
+// (blockIdx.x * blockDim.x + threadIdx.x) * VEC = first x of the thread's cells.
 // Requires nx % VEC == 0 (all of a thread's cells in one row).
 // UNI: Ms, A, Ku and alpha are uniform scalars (easy axes may still vary by
 // grain); the per-cell branches for material maps then compile away.
@@ -104,8 +104,8 @@ __global__ void __launch_bounds__(kStageThreads, stage_min_blocks<T, DMI>()) sta
     using LV = Vec<T, VEC>;
     const int nx = p.nx, ny = p.ny, nz = p.nz;
     const int N = (int)p.N;
-    const int x0 = (blockIdx.x * kBX + threadIdx.x) * VEC;
-    const int y = blockIdx.y * kBY + threadIdx.y;
+    const int x0 = (blockIdx.x * blockDim.x + threadIdx.x) * VEC;
+    const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
     double red_e0 = 0.0, red_e1 = 0.0, red_e2 = 0.0, red_e3 = 0.0, red_e4 = 0.0;
     int red_nf = 0;
@@ -360,7 +360,8 @@ __global__ void __launch_bounds__(kStageThreads, stage_min_blocks<T, DMI>()) sta
         constexpr int NW = kStageThreads / 32;
         __shared__ double red[NW][kNPart];
         __shared__ T redt[NW][3];
-        const int tid = threadIdx.y * kBX + threadIdx.x;
+        const int nw = (blockDim.x * blockDim.y) >> 5;
+        const int tid = threadIdx.y * blockDim.x + threadIdx.x;
         const int lane = tid & 31, wid = tid >> 5;
         double vals[kNPart] = {0.0, red_e0, red_e1, red_e2, red_e3, 0.0, 0.0, red_e4};
         if (p.want_energy) {
@@ -387,13 +388,13 @@ __global__ void __launch_bounds__(kStageThreads, stage_min_blocks<T, DMI>()) sta
             double acc = red[0][q];
             if (q == R_TORQUE || q == R_ERR) {
                 T t = redt[0][0], n = redt[0][1], d = redt[0][2];
-                for (int w = 1; w < NW; ++w) {
+                for (int w = 1; w < nw; ++w) {
                     t = fmax(t, redt[w][0]);
                     if (redt[w][1] * d > n * redt[w][2]) { n = redt[w][1]; d = redt[w][2]; }
                 }
                 acc = q == R_TORQUE ? (double)t : (double)(n / d);
             } else {
-                for (int w = 1; w < NW; ++w) acc = q == R_NONFINITE ? fmax(acc, red[w][q]) : acc + red[w][q];
+                for (int w = 1; w < nw; ++w) acc = q == R_NONFINITE ? fmax(acc, red[w][q]) : acc + red[w][q];
             }
             const long b = ((long)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
             p.partials[b * kNPart + q] = acc;
@@ -477,15 +478,41 @@ template <typename T> void launch_combine(const T* mn, const T* const* kin, cons
     combine_kernel<T><<<(unsigned)((3 * N + 255) / 256), 256, 0, st>>>(p);
 }
 
-template <typename T> int stage_vec(int nx);
-template <> int stage_vec<float>(int nx) { return nx % 2 == 0 ? 2 : 1; }
-template <> int stage_vec<double>(int nx) { return nx % 2 == 0 ? 2 : 1; }
+// Cells per thread along x and the block of a launch.  FP32: 64 x 4 threads, two
+// cells each.  FP64 is bound by its instructions (64 cycles for a lone warp of a
+// quarter SM, 16 per warp and SM at best), so they are spread: one cell per
+// thread unless there are 16 warps for every SM anyway, and blocks of one warp's
+// width with as many rows as leave six blocks for every SM (32x32x4: 10.0 ->
+// 5.6 us a stage, 512x128x1 18.2 -> 15.4 us).
+struct StageShape {
+    int vec;
+    dim3 block, grid;
+};
+template <typename T> static StageShape stage_shape(int nx, int ny, int nz, bool vec_ok) {
+    constexpr int kSms = 152;
+    StageShape s;
+    s.vec = vec_ok && nx % 2 == 0 ? 2 : 1;
+    int bx = kBX, by = kBY;
+    if (sizeof(T) == 8) {
+        auto warps = [&](int v) { return (long)((nx / v + 31) / 32) * ny * nz; };
+        if (s.vec == 2 && warps(2) < 16 * kSms) s.vec = 1;
+        bx = 32;
+        by = 8;
+        while (by > 1 && (long)((nx / s.vec + bx - 1) / bx) * ((ny + by - 1) / by) * nz < 6 * kSms) by >>= 1;
+    }
+    s.block = dim3(bx, by);
+    s.grid = dim3((nx / s.vec + bx - 1) / bx, (ny + by - 1) / by, nz);
+    return s;
+}
 
-// an upper bound on the blocks launch_stage uses (the scalar path has the most)
+// an upper bound on the blocks launch_stage uses
 template <typename T> int stage_blocks(int nx, int ny, int nz) {
-    const int gx = (nx + kBX - 1) / kBX;
-    const int gy = (ny + kBY - 1) / kBY;
-    return gx * gy * nz;
+    int most = 0;
+    for (int v = 0; v < 2; ++v) {
+        const StageShape s = stage_shape<T>(nx, ny, nz, v != 0);
+        most = max(most, (int)(s.grid.x * s.grid.y * s.grid.z));
+    }
+    return most;
 }
 
 static bool al16(const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; }
@@ -521,9 +548,9 @@ template void stage_prepare<double>(StageParams<double>&);
 template <typename T> void launch_stage(const StageParams<T>& p0, cudaStream_t st, int* nblocks) {
     StageParams<T> p = p0;
     stage_prepare(p);
-    const int vec = all_aligned(p) ? stage_vec<T>(p.nx) : 1;
-    dim3 block(kBX, kBY);
-    dim3 grid((p.nx / vec + kBX - 1) / kBX, (p.ny + kBY - 1) / kBY, p.nz);
+    const StageShape shape = stage_shape<T>(p.nx, p.ny, p.nz, all_aligned(p));
+    const int vec = shape.vec;
+    const dim3 block = shape.block, grid = shape.grid;
     *nblocks = (int)(grid.x * grid.y * grid.z);
     // uniform material needs Ms != 0 too (the Ms = 0 test is compiled away)
     const bool uni = !p.Ms_cell && !p.A_cell && !p.Ku_cell && !p.alpha_cell && !p.zw && p.Ms != (T)0;
