@@ -596,11 +596,10 @@ long line_fused_pairs(const DemagDims& d) { return (long)d.nz * ((d.ny + 1) / 2)
 
 template <typename T>
 bool launch_line_x_fwd(const DemagDims& d, const LineXIn<T>& in, typename Cplx<T>::type* S1, cudaStream_t st) {
-    constexpr int NC = 1;
     LineXShape o;
     if (d.nb > 65535 || !line_x_shape<T>(d.LX, line_x_pairs(d), d.nb, 1, kAnyCtas, &o)) return false;
     LineForward<T> f{in.m, in.Ms_cell, in.Ms, in.k, in.y, in.ca, in.dt_b, in.a, in.mask};
-    auto k = o.threads <= 256 ? line_x_forward<T, NC, 256, 0> : line_x_forward<T, NC, kLineThreads, 0>;
+    auto k = o.threads <= 256 ? line_x_forward<T, 256, 0> : line_x_forward<T, kLineThreads, 0>;
     if constexpr (sizeof(T) == 4) {
         if (o.ct) line_ct_use(kLineXFwd, d.LX, &k);
     }
@@ -611,10 +610,9 @@ bool launch_line_x_fwd(const DemagDims& d, const LineXIn<T>& in, typename Cplx<T
 
 template <typename T>
 bool launch_line_x_inv(const DemagDims& d, const typename Cplx<T>::type* S1, T* h, cudaStream_t st) {
-    constexpr int NC = 1;
     LineXShape o;
     if (d.nb > 65535 || !line_x_shape<T>(d.LX, line_x_pairs(d), d.nb, 1, kAnyCtas, &o)) return false;
-    auto k = o.threads <= 256 ? line_x_inverse<T, NC, 256, 0> : line_x_inverse<T, NC, kLineThreads, 0>;
+    auto k = o.threads <= 256 ? line_x_inverse<T, 256, 0> : line_x_inverse<T, kLineThreads, 0>;
     if constexpr (sizeof(T) == 4) {
         if (o.ct) line_ct_use(kLineXInv, d.LX, &k);
     }
@@ -659,18 +657,12 @@ static void line_ct_shape(int L, long ncol, LineShape* o) {
 template <typename T, int DIR>
 bool launch_line_y(const DemagDims& d, const typename Cplx<T>::type* in, typename Cplx<T>::type* out,
                    cudaStream_t st) {
-    constexpr int NC = sizeof(T) == 8 ? 1 : 3;
     LineShape o;
-    const long ncol = (long)d.KX * d.nz * (3 / NC);
-    if (d.nb > 65535 || !line_shape<T>(d.LY, ncol, d.nb, NC, false, &o) || o.pl.np < 2) return false;
-    auto k = sizeof(T) == 4 && o.threads <= kLineThreads32
-                 ? line_y<T, DIR, NC, sizeof(T) == 4 ? kLineThreads32 : kLineThreads, 0>
-                 : line_y<T, DIR, NC, kLineThreads, 0>;
-    if constexpr (sizeof(T) == 4) {
-        if (line_ct_use(DIR < 0 ? kLineYFwd : kLineYInv, d.LY, &k)) line_ct_shape(d.LY, ncol, &o);
-    }
-    line_launch(k, dim3((unsigned)o.ctas, d.nb), o.threads, o.smem, st, d, in, out, o.pl, line_table<T>(o.pl), o.lb, (int)ncol,
-                line_early<T>(o.ctas * d.nb));
+    const long ncol = 3L * d.KX * d.nz;
+    if (d.nb > 65535 || !line_shape<T>(d.LY, ncol, d.nb, 1, false, &o) || o.pl.np < 2) return false;
+    auto k = o.threads <= 256 ? line_y<T, DIR, 256> : line_y<T, DIR, kLineThreads>;
+    line_launch(k, dim3((unsigned)o.ctas, d.nb), o.threads, o.smem, st, d, in, out, o.pl, line_table<T>(o.pl), o.lb,
+                (int)ncol, line_early<T>(o.ctas * d.nb));
     return true;
 }
 

@@ -207,10 +207,11 @@ template <typename T> struct LineForward {
     const int* mask;      // grids to work on, or null
 };
 
-template <typename T, int NC, int MAXT, int LC>
+template <typename T, int MAXT, int LC>
 __global__ void __launch_bounds__(MAXT)
 line_x_forward(DemagDims d, LineForward<T> f, typename Cplx<T>::type* __restrict__ S1,
                const __grid_constant__ LinePlan pl, const typename Cplx<T>::type* __restrict__ tw, int nt, int lines, int early) {
+    constexpr int NC = 1;                            // components per line
     using C = typename Cplx<T>::type;
     extern __shared__ __align__(16) unsigned char smraw[];
     if constexpr (LC > 0) {
@@ -275,10 +276,11 @@ line_x_forward(DemagDims d, LineForward<T> f, typename Cplx<T>::type* __restrict
                         r.on && t.in, r.two);
 }
 
-template <typename T, int NC, int MAXT, int LC>
+template <typename T, int MAXT, int LC>
 __global__ void __launch_bounds__(MAXT)
 line_x_inverse(DemagDims d, const typename Cplx<T>::type* __restrict__ S1, T* __restrict__ h,
                const __grid_constant__ LinePlan pl, const typename Cplx<T>::type* __restrict__ tw, int nt, int lines, int early) {
+    constexpr int NC = 1;                            // components per line
     using C = typename Cplx<T>::type;
     extern __shared__ __align__(16) unsigned char smraw[];
     if constexpr (LC > 0) {
@@ -331,8 +333,8 @@ struct LineRed {
 
 // Sums of FP32 products kept exact to 48 bits as high and low parts (products
 // and sums with their rounding errors: Dekker 1971, Knuth's two-sum): FP64
-// instructions run at 1/64 of the FP32 rate here, and an energy of 100x65x27
-// cells spent 20 of 35 us on them.
+// instructions run at 1/64 of the FP32 rate here, and a field of 100x65x27 cells
+// with its energies took 35.6 us in FP64 sums, 30.8 us so.
 __device__ __forceinline__ void line_acc(float2& s, float p, float e) {
     const float t = __fadd_rn(s.x, p), z = __fsub_rn(t, s.x);
     s.y = __fadd_rn(s.y, __fadd_rn(__fadd_rn(__fsub_rn(s.x, __fsub_rn(t, z)), __fsub_rn(p, z)), e));
@@ -863,7 +865,7 @@ line_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restr
     int M = L / pl.rmin;
     if constexpr (LC > 0) {
         constexpr int kM = LC / line_ct<T>(LC).rmin;
-        constexpr int kLb = FORM == kConvSplit ? line_split_lb<T>(kM) : line_ct_lb<T>(LC);
+        constexpr int kLb = line_ct_lb<T>(LC);
         M = kM;
         lb = kLb;
     }
@@ -884,7 +886,8 @@ line_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restr
     if constexpr (FORM == kConvSplit) {
         // this thread's wave numbers u + 3 M i; their tensor entries (written long
         // before the previous pass) are on their way from the start
-        constexpr int KP = sizeof(T) == 4 ? 3 : 2;      // the smallest radix of a plan is 8, or 4, at most
+        static_assert(LC == 0 && sizeof(T) == 8, "the split form is FP64's");
+        constexpr int KP = 2;                           // the smallest radix of an FP64 plan is 4 at most
         T t[KP][6];
 #pragma unroll
         for (int i = 0; i < KP; ++i) {
@@ -912,27 +915,15 @@ line_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restr
             }
             __syncthreads();
         };
-        if constexpr (LC > 0) {
-            constexpr LinePlan P = line_ct<T>(LC);
-            constexpr int np = P.np;
-            line_first<T, -1, P.R[0], true, 1>(g, zs, 0, d.nz, s, 0, lb, b, L);
-            __syncthreads();
-            line_mids_ct<T, -1, 1, 3, LC, 1, np>(s, 0, lb, b, tw);
-            product();
-            line_start<T, +1, P.R[np - 1], 1, 3>(s, 0, lb, b, L);
-            line_mids_ct<T, +1, 1, 3, LC, 1, np - 1>(s, 0, lb, b, tw);
-            line_last<T, +1, P.R[0], true, 1>(s, 0, lb, b, L, P.Nsi[np - 1], 0, tw, g, zs, 0, d.nz, valid);
-        } else {
-            const int np = pl.np;
-            MM_LINE_RADIX_EVEN(T, pl.R[0], (line_first<T, -1, R_, true, 1>(g, zs, 0, d.nz, s, 0, lb, b, L)));
-            __syncthreads();
-            for (int i = 1; i < np; ++i) line_mid_any<T, -1, 1, 3>(s, 0, lb, b, pl, i, tw);
-            product();
-            MM_LINE_RADIX(T, pl.R[np - 1], (line_start<T, +1, R_, 1, 3>(s, 0, lb, b, L)));
-            for (int i = 1; i < np - 1; ++i) line_mid_any<T, +1, 1, 3>(s, 0, lb, b, pl, i, tw);
-            MM_LINE_RADIX_EVEN(T, pl.R[0], (line_last<T, +1, R_, true, 1>(s, 0, lb, b, L, pl.Nsi[np - 1], pl.mgi[np - 1],
-                                                                          tw, g, zs, 0, d.nz, valid)));
-        }
+        const int np = pl.np;
+        MM_LINE_RADIX_EVEN(T, pl.R[0], (line_first<T, -1, R_, true, 1>(g, zs, 0, d.nz, s, 0, lb, b, L)));
+        __syncthreads();
+        for (int i = 1; i < np; ++i) line_mid_any<T, -1, 1, 3>(s, 0, lb, b, pl, i, tw);
+        product();
+        MM_LINE_RADIX(T, pl.R[np - 1], (line_start<T, +1, R_, 1, 3>(s, 0, lb, b, L)));
+        for (int i = 1; i < np - 1; ++i) line_mid_any<T, +1, 1, 3>(s, 0, lb, b, pl, i, tw);
+        MM_LINE_RADIX_EVEN(T, pl.R[0], (line_last<T, +1, R_, true, 1>(s, 0, lb, b, L, pl.Nsi[np - 1], pl.mgi[np - 1],
+                                                                      tw, g, zs, 0, d.nz, valid)));
         return;
     }
     grid_dep_wait();
@@ -974,61 +965,46 @@ line_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restr
 }
 
 // y passes.  DIR = -1: S1 (ny rows) -> S2 (Py rows), forward, zero upper half;
-// DIR = +1: S2 -> S1, keep y < ny.  Columns kx-fastest over (component and) z,
-// kx <= Px/2; NC components per thread.
-template <typename T, int DIR, int NC, int MAXT, int LC>
-__global__ void __launch_bounds__(MAXT, line_blocks<T, MAXT>())
+// DIR = +1: S2 -> S1, keep y < ny.  Columns kx-fastest over component and z,
+// kx <= Px/2, a thread per butterfly of one component (three per thread: 11.3 and
+// 9.6 against 8.7 and 8.8 us on 140-point lines of 100x65x27).
+template <typename T, int DIR, int MAXT>
+__global__ void __launch_bounds__(MAXT)
 line_y(DemagDims d, const typename Cplx<T>::type* __restrict__ in, typename Cplx<T>::type* __restrict__ out,
        const __grid_constant__ LinePlan pl, const typename Cplx<T>::type* __restrict__ tw, int lb, int ncol, int early) {
     using C = typename Cplx<T>::type;
     extern __shared__ __align__(16) unsigned char smraw[];
-    const int L = LC ? LC : pl.L, tid = threadIdx.x;
-    if constexpr (LC > 0) {
-        constexpr int kLb = line_ct_lb<T>(LC);
-        lb = kLb;
-    }
+    const int L = pl.L, np = pl.np, tid = threadIdx.x;
     const int l = tid & ((1 << lb) - 1), b = tid >> lb;
     const int col = (blockIdx.x << lb) + l;
     const bool valid = col < ncol;
     const int cc = valid ? col : ncol - 1;
-    const int z = cc / d.KX, kx = cc - z * d.KX;
+    const int cz = cc / d.KX, kx = cc - cz * d.KX;
     const int rin = DIR < 0 ? d.ny : L, rout = DIR < 0 ? L : d.ny;
-    const long cin = (long)d.nz * rin * d.KXS, cout = (long)d.nz * rout * d.KXS;
-    const C* gi = in + (long)blockIdx.y * 3 * cin + (long)z * rin * d.KXS + kx;     // NC = 1: z runs over 3 nz planes
-    C* go = out + (long)blockIdx.y * 3 * cout + (long)z * rout * d.KXS + kx;
+    const long plane = (long)blockIdx.y * 3 * d.nz + cz;
+    const C* gi = in + plane * rin * d.KXS + kx;
+    C* go = out + plane * rout * d.KXS + kx;
     if (early) grid_dep_launch();
     grid_dep_wait();
     C* s = reinterpret_cast<C*>(smraw) + l;
-    const int plane = line_len(L) << lb;
-    if constexpr (LC > 0) {
-        constexpr LinePlan P = line_ct<T>(LC);
-        constexpr int np = P.np, RF = DIR < 0 ? P.R[0] : P.R[np - 1], RL = DIR < 0 ? P.R[np - 1] : P.R[0];
-        line_first<T, DIR, RF, (DIR < 0), NC>(gi, d.KXS, cin, rin, s, plane, lb, b, L);
-        __syncthreads();
-        line_mids_ct<T, DIR, NC, 3, LC, 1, np - 1>(s, plane, lb, b, tw);
-        line_last<T, DIR, RL, (DIR > 0), NC>(s, plane, lb, b, L, DIR < 0 ? P.Ns[np - 1] : P.Nsi[np - 1], 0, tw, go, d.KXS,
-                                             cout, rout, valid);
-        return;
-    }
-    const int np = pl.np;
     if constexpr (DIR < 0) {
-        MM_LINE_RADIX_EVEN(T, pl.R[0], (line_first<T, -1, R_, true, NC>(gi, d.KXS, cin, d.ny, s, plane, lb, b, L)));
+        MM_LINE_RADIX_EVEN(T, pl.R[0], (line_first<T, -1, R_, true, 1>(gi, d.KXS, 0, d.ny, s, 0, lb, b, L)));
     } else {
-        MM_LINE_RADIX(T, pl.R[np - 1], (line_first<T, +1, R_, false, NC>(gi, d.KXS, cin, L, s, plane, lb, b, L)));
+        MM_LINE_RADIX(T, pl.R[np - 1], (line_first<T, +1, R_, false, 1>(gi, d.KXS, 0, L, s, 0, lb, b, L)));
     }
     __syncthreads();
-    for (int i = 1; i < np - 1; ++i) line_mid_any<T, DIR, NC, 3>(s, plane, lb, b, pl, i, tw);
+    for (int i = 1; i < np - 1; ++i) line_mid_any<T, DIR, 1, 3>(s, 0, lb, b, pl, i, tw);
     if constexpr (DIR < 0) {
-        MM_LINE_RADIX(T, pl.R[np - 1], (line_last<T, -1, R_, false, NC>(s, plane, lb, b, L, pl.Ns[np - 1], pl.mg[np - 1], tw,
-                                                                 go, d.KXS, cout, L, valid)));
+        MM_LINE_RADIX(T, pl.R[np - 1], (line_last<T, -1, R_, false, 1>(s, 0, lb, b, L, pl.Ns[np - 1], pl.mg[np - 1], tw, go,
+                                                                       d.KXS, 0, L, valid)));
     } else {
-        MM_LINE_RADIX_EVEN(T, pl.R[0], (line_last<T, +1, R_, true, NC>(s, plane, lb, b, L, pl.Nsi[np - 1], pl.mgi[np - 1], tw,
-                                                                go, d.KXS, cout, d.ny, valid)));
+        MM_LINE_RADIX_EVEN(T, pl.R[0], (line_last<T, +1, R_, true, 1>(s, 0, lb, b, L, pl.Nsi[np - 1], pl.mgi[np - 1], tw, go,
+                                                                      d.KXS, 0, d.ny, valid)));
     }
 }
 
 // kernels of the compiled lengths, by kind: null for a length without them
-enum LineKind { kLineFused, kLineFusedGen, kLineXFwd, kLineXInv, kLineConv, kLineYFwd, kLineYInv };
+enum LineKind { kLineFused, kLineFusedGen, kLineXFwd, kLineXInv, kLineConv };
 const void* line_ct_kernel0(LineKind kind, int L);      // 16 .. 128
 const void* line_ct_kernel1(LineKind kind, int L);      // 256 .. 1024
 const void* line_ct_kernel2(LineKind kind, int L);      // 96 .. 224
@@ -1040,11 +1016,9 @@ template <int LC> const void* line_ct_pick(LineKind kind) {
     switch (kind) {
         case kLineFused: return (const void*)line_fused<false, FT, LC>;
         case kLineFusedGen: return (const void*)line_fused<true, FT, LC>;
-        case kLineXFwd: return (const void*)line_x_forward<float, 1, 256, LC>;
-        case kLineXInv: return (const void*)line_x_inverse<float, 1, 256, LC>;
-        case kLineConv: return (const void*)line_conv<float, kConvThree, YT, LC>;
-        case kLineYFwd: return (const void*)line_y<float, -1, 3, YT, LC>;
-        default: return (const void*)line_y<float, +1, 3, YT, LC>;
+        case kLineXFwd: return (const void*)line_x_forward<float, 256, LC>;
+        case kLineXInv: return (const void*)line_x_inverse<float, 256, LC>;
+        default: return (const void*)line_conv<float, kConvThree, YT, LC>;
     }
 }
 
