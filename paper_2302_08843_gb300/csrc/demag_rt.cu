@@ -484,20 +484,34 @@ struct LineShape {
     long ctas;
 };
 
-// Radices are bounded by 8 (FP32, which shared-memory exchanges bound) or 4
-// (FP64, whose instructions bound it: small radices cost no more of them and
-// put more warps on them).  An FP64 grid that would leave quarter SMs idle
-// takes radix 2; the grids of a batch do not count, so that a grid's rounding
-// does not depend on the others.  Then as many columns per CTA (at least one 32-byte sector of
-// each row) as leave two CTAs for every SM.
+// The plan of a line, of which a launch has `lines`.  Radices are bounded by 8
+// (FP32, which shared-memory exchanges bound) or 4 (FP64, whose instructions
+// bound it: small radices cost no more of them and put more warps on them; the x
+// lines of 128x128x32 took 84 and 80 us with radix 4, 124 and 105 with 8).  An
+// FP64 length whose radix-4 plan keeps a radix-2 pass takes radices up to 8
+// instead: the wide first pass would idle half its threads in every other
+// (128x128x64's 128-point z lines 1351 -> 923 us, 256x256x64's 512-point lines
+// 1490 -> 1010 and 1486 -> 1056 along y, 988 -> 649 and 953 -> 631 along x).  An
+// FP64 grid that would leave quarter SMs idle takes radix 2; the grids of a batch
+// do not count, so that a grid's rounding does not depend on the others.
+template <typename T> LinePlan line_radices(int L, long lines, bool one) {
+    constexpr int kSms = 152;
+    if (sizeof(T) == 4) return host_plan(L, 8, one);
+    if (L > 2 && lines * (L / 4) < kSms * 128L) return host_plan(L, 2, one);
+    const LinePlan p = host_plan(L, 4, one);
+    if (one || p.rmin != 2) return p;
+    const LinePlan wide = host_plan(L, 8, one);
+    return wide.np > 1 ? wide : p;          // 6 and 8 points keep two passes
+}
+
+// As many columns per CTA (at least one 32-byte sector of each row) as leave two
+// CTAs for every SM.
 template <typename T> bool line_shape(int L, long ncol, int nb, int nc, bool conv, LineShape* o) {
     constexpr int kSms = 152;
     constexpr int full = 128 / (2 * sizeof(T)), sector = 32 / (2 * sizeof(T));
-    int rmax = sizeof(T) == 4 ? 8 : 4;
-    if (sizeof(T) == 8 && L > 2 && ncol * (L / 4) < kSms * 128L) rmax = 2;
     // FP32 z lines of up to 16 points stay in one thread's registers
     const bool one = conv && (L <= 2 || L == 4 || (sizeof(T) == 4 && (L == 6 || L == 8 || L == 12 || L == 16)));
-    o->pl = host_plan(L, rmax, one);
+    o->pl = line_radices<T>(L, ncol, one);
     const int M = L / o->pl.rmin;
     if (o->pl.np < 1 || o->pl.np > kLineMaxPass) return false;
     int lb = 0;
@@ -567,9 +581,7 @@ struct LineXShape {
 // pair (3: the fused stage's components).  FP64 radices as in line_shape.
 template <typename T> bool line_x_shape(int L, long pairs, int nb, int nc, long max_ctas, LineXShape* o) {
     constexpr int kSms = 152;
-    int rmax = line_rmax<T>();
-    if (sizeof(T) == 8 && pairs * (L / 4) < kSms * 128L) rmax = 2;
-    o->pl = host_plan(L, rmax, false);
+    o->pl = line_radices<T>(L, pairs, false);
     if (o->pl.np < 2) return false;
     o->nt = L / o->pl.rmin;
     const int per = nc * o->nt, most = nc == 3 ? 1024 : kLineThreads;

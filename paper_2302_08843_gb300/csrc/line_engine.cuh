@@ -25,8 +25,8 @@
 // radix-8 passes that multiply first.  FP64 instructions are what an FP64
 // pass spends its time on (one warp instruction per 19 cycles and SM; 64
 // cycles for a single warp of a quarter SM, dependent or not), so FP64 plans
-// take small radices and many threads; FP32 passes are bound by the
-// shared-memory exchanges and take radix 8.
+// take radix 4, many threads and, against a radix-2 pass left over, radix 8;
+// FP32 passes are bound by the shared-memory exchanges and take radix 8.
 #pragma once
 
 #include "common.cuh"
@@ -93,8 +93,8 @@ constexpr LinePlan line_plan(int L, int rmax) {
     }
     return p;
 }
-template <typename T> constexpr int line_rmax() { return sizeof(T) == 4 ? 8 : 4; }
-template <typename T> __host__ __device__ constexpr LinePlan line_ct(int L) { return line_plan(L, line_rmax<T>()); }
+// plan of an FP32 compiled length
+template <typename T> __host__ __device__ constexpr LinePlan line_ct(int L) { return line_plan(L, 8); }
 // FP64 z lines whose three components fit a CTA side by side take a thread per
 // butterfly and component (32x32x4: 9.5 -> 6.6 us, 128x128x32: 416 -> 393 us; in
 // FP32 the extra exchange costs more than the threads bring: 32 grids of
@@ -287,22 +287,22 @@ __device__ __forceinline__ void line_start(typename Cplx<T>::type* s, int plane,
 }
 
 // CALL with R_ = the radix; the FP64 plans hold none above 7 and no 6
-#define MM_LINE_RADIX(Tv, Rv, CALL)                                       \
+#define MM_LINE_RADIX(Rv, CALL)                                           \
     switch (Rv) {                                                         \
         case 2: { constexpr int R_ = 2; CALL; } break;                     \
         case 3: { constexpr int R_ = 3; CALL; } break;                     \
         case 4: { constexpr int R_ = 4; CALL; } break;                     \
         case 5: { constexpr int R_ = 5; CALL; } break;                     \
         case 7: { constexpr int R_ = 7; CALL; } break;                     \
-        case 6: { constexpr int R_ = sizeof(Tv) == 4 ? 6 : 2; CALL; } break; \
-        default: { constexpr int R_ = sizeof(Tv) == 4 ? 8 : 2; CALL; } break; \
+        case 6: { constexpr int R_ = 6; CALL; } break; \
+        default: { constexpr int R_ = 8; CALL; } break; \
     }
-#define MM_LINE_RADIX_EVEN(Tv, Rv, CALL)                                  \
+#define MM_LINE_RADIX_EVEN(Rv, CALL)                                      \
     switch (Rv) {                                                         \
         case 2: { constexpr int R_ = 2; CALL; } break;                     \
         case 4: { constexpr int R_ = 4; CALL; } break;                     \
-        case 6: { constexpr int R_ = sizeof(Tv) == 4 ? 6 : 2; CALL; } break; \
-        default: { constexpr int R_ = sizeof(Tv) == 4 ? 8 : 2; CALL; } break; \
+        case 6: { constexpr int R_ = 6; CALL; } break; \
+        default: { constexpr int R_ = 8; CALL; } break; \
     }
 
 template <typename T, int DIR, int NC, int SH>
@@ -311,7 +311,7 @@ __device__ __forceinline__ void line_mid_any(typename Cplx<T>::type* s, int plan
     const int R = DIR < 0 ? pl.R[i] : pl.R[pl.np - 1 - i];
     const int Ns = DIR < 0 ? pl.Ns[i] : pl.Nsi[i];
     const unsigned mg = DIR < 0 ? pl.mg[i] : pl.mgi[i];
-    MM_LINE_RADIX(T, R, (line_mid<T, DIR, R_, NC, SH>(s, plane, lb, b, pl.L, Ns, mg, tw)));
+    MM_LINE_RADIX(R, (line_mid<T, DIR, R_, NC, SH>(s, plane, lb, b, pl.L, Ns, mg, tw)));
 }
 
 // passes I .. END-1 of a compiled length

@@ -142,10 +142,10 @@ __device__ __forceinline__ void line_inverse(const typename Cplx<T>::type* sa, c
         line_x_last<T, P.R[0], NC>(s, plane, b, LC, P.Nsi[np - 1], 0, tw);
     } else {
         const int np = pl.np, L = pl.L;
-        MM_LINE_RADIX(T, pl.R[np - 1], (line_x_first<T, R_, NC>(sa, sb, cs, s, plane, b, L)));
+        MM_LINE_RADIX(pl.R[np - 1], (line_x_first<T, R_, NC>(sa, sb, cs, s, plane, b, L)));
         __syncthreads();
         for (int i = 1; i < np - 1; ++i) line_mid_any<T, +1, NC, 4>(s, plane, 0, b, pl, i, tw);
-        MM_LINE_RADIX_EVEN(T, pl.R[0], (line_x_last<T, R_, NC>(s, plane, b, L, pl.Nsi[np - 1], pl.mgi[np - 1], tw)));
+        MM_LINE_RADIX_EVEN(pl.R[0], (line_x_last<T, R_, NC>(s, plane, b, L, pl.Nsi[np - 1], pl.mgi[np - 1], tw)));
     }
 }
 
@@ -163,7 +163,7 @@ __device__ __forceinline__ void line_forward(typename Cplx<T>::type* s, int plan
         line_f_first<T, P.R[0], NC>(s, plane, b, LC, nx);
         line_mids_ct<T, -1, NC, 4, LC, 1, P.np>(s, plane, 0, b, tw);
     } else {
-        MM_LINE_RADIX_EVEN(T, pl.R[0], (line_f_first<T, R_, NC>(s, plane, b, L, nx)));
+        MM_LINE_RADIX_EVEN(pl.R[0], (line_f_first<T, R_, NC>(s, plane, b, L, nx)));
         for (int i = 1; i < pl.np; ++i) line_mid_any<T, -1, NC, 4>(s, plane, 0, b, pl, i, tw);
     }
     if (!on) return;
@@ -887,7 +887,7 @@ line_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restr
         // this thread's wave numbers u + 3 M i; their tensor entries (written long
         // before the previous pass) are on their way from the start
         static_assert(LC == 0 && sizeof(T) == 8, "the split form is FP64's");
-        constexpr int KP = 2;                           // the smallest radix of an FP64 plan is 4 at most
+        constexpr int KP = 3;                           // the smallest radix of a plan is 8 at most
         T t[KP][6];
 #pragma unroll
         for (int i = 0; i < KP; ++i) {
@@ -916,13 +916,13 @@ line_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restr
             __syncthreads();
         };
         const int np = pl.np;
-        MM_LINE_RADIX_EVEN(T, pl.R[0], (line_first<T, -1, R_, true, 1>(g, zs, 0, d.nz, s, 0, lb, b, L)));
+        MM_LINE_RADIX_EVEN(pl.R[0], (line_first<T, -1, R_, true, 1>(g, zs, 0, d.nz, s, 0, lb, b, L)));
         __syncthreads();
         for (int i = 1; i < np; ++i) line_mid_any<T, -1, 1, 3>(s, 0, lb, b, pl, i, tw);
         product();
-        MM_LINE_RADIX(T, pl.R[np - 1], (line_start<T, +1, R_, 1, 3>(s, 0, lb, b, L)));
+        MM_LINE_RADIX(pl.R[np - 1], (line_start<T, +1, R_, 1, 3>(s, 0, lb, b, L)));
         for (int i = 1; i < np - 1; ++i) line_mid_any<T, +1, 1, 3>(s, 0, lb, b, pl, i, tw);
-        MM_LINE_RADIX_EVEN(T, pl.R[0], (line_last<T, +1, R_, true, 1>(s, 0, lb, b, L, pl.Nsi[np - 1], pl.mgi[np - 1],
+        MM_LINE_RADIX_EVEN(pl.R[0], (line_last<T, +1, R_, true, 1>(s, 0, lb, b, L, pl.Nsi[np - 1], pl.mgi[np - 1],
                                                                       tw, g, zs, 0, d.nz, valid)));
         return;
     }
@@ -951,14 +951,14 @@ line_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restr
             line_mids_ct<T, +1, 3, 3, LC, 1, np - 1>(s, plane, lb, b, tw);
             line_last<T, +1, P.R[0], true, 3>(s, plane, lb, b, L, P.Nsi[np - 1], 0, tw, g, zs, cs, d.nz, valid);
         } else {
-            MM_LINE_RADIX_EVEN(T, pl.R[0], (line_first<T, -1, R_, true, 3>(g, zs, cs, d.nz, s, plane, lb, b, L)));
+            MM_LINE_RADIX_EVEN(pl.R[0], (line_first<T, -1, R_, true, 3>(g, zs, cs, d.nz, s, plane, lb, b, L)));
             __syncthreads();
             const int np = pl.np;
             for (int i = 1; i < np - 1; ++i) line_mid_any<T, -1, 3, 3>(s, plane, lb, b, pl, i, tw);
-            MM_LINE_RADIX(T, pl.R[np - 1], (line_product<T, R_>(s, plane, lb, b, L, pl.Ns[np - 1], pl.mg[np - 1], tw, tp,
+            MM_LINE_RADIX(pl.R[np - 1], (line_product<T, R_>(s, plane, lb, b, L, pl.Ns[np - 1], pl.mg[np - 1], tw, tp,
                                                                 tz, tc, up, d.yz_swap)));
             for (int i = 1; i < np - 1; ++i) line_mid_any<T, +1, 3, 3>(s, plane, lb, b, pl, i, tw);
-            MM_LINE_RADIX_EVEN(T, pl.R[0], (line_last<T, +1, R_, true, 3>(s, plane, lb, b, L, pl.Nsi[np - 1],
+            MM_LINE_RADIX_EVEN(pl.R[0], (line_last<T, +1, R_, true, 3>(s, plane, lb, b, L, pl.Nsi[np - 1],
                                                                           pl.mgi[np - 1], tw, g, zs, cs, d.nz, valid)));
         }
     }
@@ -988,17 +988,17 @@ line_y(DemagDims d, const typename Cplx<T>::type* __restrict__ in, typename Cplx
     grid_dep_wait();
     C* s = reinterpret_cast<C*>(smraw) + l;
     if constexpr (DIR < 0) {
-        MM_LINE_RADIX_EVEN(T, pl.R[0], (line_first<T, -1, R_, true, 1>(gi, d.KXS, 0, d.ny, s, 0, lb, b, L)));
+        MM_LINE_RADIX_EVEN(pl.R[0], (line_first<T, -1, R_, true, 1>(gi, d.KXS, 0, d.ny, s, 0, lb, b, L)));
     } else {
-        MM_LINE_RADIX(T, pl.R[np - 1], (line_first<T, +1, R_, false, 1>(gi, d.KXS, 0, L, s, 0, lb, b, L)));
+        MM_LINE_RADIX(pl.R[np - 1], (line_first<T, +1, R_, false, 1>(gi, d.KXS, 0, L, s, 0, lb, b, L)));
     }
     __syncthreads();
     for (int i = 1; i < np - 1; ++i) line_mid_any<T, DIR, 1, 3>(s, 0, lb, b, pl, i, tw);
     if constexpr (DIR < 0) {
-        MM_LINE_RADIX(T, pl.R[np - 1], (line_last<T, -1, R_, false, 1>(s, 0, lb, b, L, pl.Ns[np - 1], pl.mg[np - 1], tw, go,
+        MM_LINE_RADIX(pl.R[np - 1], (line_last<T, -1, R_, false, 1>(s, 0, lb, b, L, pl.Ns[np - 1], pl.mg[np - 1], tw, go,
                                                                        d.KXS, 0, L, valid)));
     } else {
-        MM_LINE_RADIX_EVEN(T, pl.R[0], (line_last<T, +1, R_, true, 1>(s, 0, lb, b, L, pl.Nsi[np - 1], pl.mgi[np - 1], tw, go,
+        MM_LINE_RADIX_EVEN(pl.R[0], (line_last<T, +1, R_, true, 1>(s, 0, lb, b, L, pl.Nsi[np - 1], pl.mgi[np - 1], tw, go,
                                                                       d.KXS, 0, d.ny, valid)));
     }
 }

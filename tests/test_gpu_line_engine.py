@@ -16,9 +16,15 @@ D = (2e-9, 3e-9, 2.5e-9)
 GRIDS = [(9, 8, 2), (9, 8, 3), (17, 6, 4), (33, 7, 6), (10, 12, 8), (5, 3, 49), (6, 4, 35), (7, 5, 63), (8, 9, 27),
          (3, 245, 1), (20, 257, 1), (5, 512, 1), (6, 525, 1), (2, 3, 1024), (1, 2, 700)]
 
+# FP64 lines whose radix-4 plan would end in a radix 2, enough of them to keep
+# whole warps busy: 32, 40, 56, 96, 128, 160, 200, 512, 1536 and 2400 points and the shortest
+# (6 and 8, which stay at two passes), and 56 points on both sides of the line
+# that parts few lines (radix 2) from many (19456 butterflies of radix 4)
+WIDE = [(256, 18, 8), (20, 28, 64), (16, 256, 10), (100, 40, 12), (48, 16, 40), (768, 38, 1), (62, 78, 4), (130, 100, 3),
+        (4, 1200, 4), (28, 30, 30), (57, 28, 8), (54, 28, 8)]
 
-@pytest.mark.parametrize("precision", ["fp64", "fp32"])
-@pytest.mark.parametrize("n", GRIDS)
+
+@pytest.mark.parametrize("n,precision", [(n, p) for n in GRIDS for p in ("fp64", "fp32")] + [(n, "fp64") for n in WIDE])
 def test_lines_match_oracle(n, precision):
     from oracle.demag import demag_fft, magnetization, rounding_sensitivity
     from oracle.newell import demag_tensor
