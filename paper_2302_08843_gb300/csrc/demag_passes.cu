@@ -2064,20 +2064,25 @@ template <int L> static bool launch_p5_tma(const DemagDims& d, const float2* S1,
 template <typename T, int L> static void launch_p3(const DemagDims& d, typename Cplx<T>::type* S2, const T* tens,
                                                    cudaStream_t st) {
     // Single FP32 grids with tiles enough for the persistent TMA passes (16
-    // columns of one ky each; two-factor lines: always) take those: 2304 tiles of
-    // 32-point lines 14.6 against 16.5 us, 128-point lines 43 against 70.  The line
-    // engine takes the others, where a tile's latency is what counts (33 tiles of
-    // a film's 256 points 8.6 -> 5.8 us, 640 of 32 points 10.5 -> 9.0; lines up to
-    // 16 points, one thread each, are level up to 8704 tiles), FP64 (64-point
-    // lines of 128x128x32 519 -> 393 us, 256 points of a 512x128x1 film 97 -> 44)
-    // and batches (16 grids of 100x100x8 63 -> 34 us).
+    // columns of one ky each; two-factor lines: always) take those; the longer the
+    // line, the fewer that is.  A step of RK4 and of Dormand-Prince, line engine
+    // against TMA: 128 points, 64 tiles 67 and 118 against 76 and 125 us, 192 tiles
+    // 104 and 170 against 98 and 180, 640 tiles 190 and 343 against 148 and 267; 64
+    // points, 480 tiles 98 and 169 against 101 and 176, 640 tiles 117 and 191 against
+    // 113 and 180; 256 points, 33 tiles 59 and 115 against 65 and 125, 64 tiles 92 and
+    // 142 against 86 and 151; 32 points, 640 tiles 81 and 147 against 88 and 155, 2304
+    // tiles 16.5 against 14.6 us a pass; lines up to 16 points, one thread each,
+    // are level up to 8704 tiles.  The line engine takes all others, FP64 (64-point
+    // lines of 128x128x32 519 -> 393 us, 256 points of a 512x128x1 film 97 -> 44) and
+    // batches (16 grids of 100x100x8 63 -> 34 us).
+    constexpr int kTmaTiles = L <= 16 ? 8192 : L < 64 ? 1024 : L < 128 ? 560 : L < 256 ? 144 : 48;
     if constexpr (sizeof(T) == 4 && L <= 256 && Fft<T, L, -1, (L > 1)>::NR <= 20) {
         if constexpr (z_two_r1<L>() > 0) {
             if (kZTwo && d.nb == 1 && launch_p3_two<L>(d, S2, tens, st)) return;
         }
         if constexpr (tma_len<L>()) {
             const long tiles = (long)((d.KX + 15) / 16) * d.LY;
-            if (d.nb == 1 && (d.classic || tiles >= (L <= 16 ? 8192 : 1024)) && launch_p3_tma<L>(d, S2, tens, st)) return;
+            if (d.nb == 1 && (d.classic || tiles >= kTmaTiles) && launch_p3_tma<L>(d, S2, tens, st)) return;
         }
     }
     if (!d.classic && launch_line_conv<T>(d, S2, tens, st)) return;

@@ -210,7 +210,7 @@ template <typename T> struct LineForward {
 template <typename T, int MAXT, int LC>
 __global__ void __launch_bounds__(MAXT)
 line_x_forward(DemagDims d, LineForward<T> f, typename Cplx<T>::type* __restrict__ S1,
-               const __grid_constant__ LinePlan pl, const typename Cplx<T>::type* __restrict__ tw, int nt, int lines, int early) {
+               const __grid_constant__ LinePlan pl, const typename Cplx<T>::type* __restrict__ tw, int nt, int lines) {
     constexpr int NC = 1;                            // components per line
     using C = typename Cplx<T>::type;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -223,7 +223,6 @@ line_x_forward(DemagDims d, LineForward<T> f, typename Cplx<T>::type* __restrict
     const LineRows r = line_rows<NC>(d, blockIdx.x * lines + t.l);
     const long rows = (long)d.ny * d.nz;             // rows of one component
     C* s = reinterpret_cast<C*>(smraw) + (size_t)t.l * NC * plane;
-    if (early) grid_dep_launch();
     grid_dep_wait();
     if (f.mask && !f.mask[g]) return;
     const T* Ms_b = static_cast<const T*>(d.Ms_b);
@@ -279,7 +278,7 @@ line_x_forward(DemagDims d, LineForward<T> f, typename Cplx<T>::type* __restrict
 template <typename T, int MAXT, int LC>
 __global__ void __launch_bounds__(MAXT)
 line_x_inverse(DemagDims d, const typename Cplx<T>::type* __restrict__ S1, T* __restrict__ h,
-               const __grid_constant__ LinePlan pl, const typename Cplx<T>::type* __restrict__ tw, int nt, int lines, int early) {
+               const __grid_constant__ LinePlan pl, const typename Cplx<T>::type* __restrict__ tw, int nt, int lines) {
     constexpr int NC = 1;                            // components per line
     using C = typename Cplx<T>::type;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -293,7 +292,6 @@ line_x_inverse(DemagDims d, const typename Cplx<T>::type* __restrict__ S1, T* __
     const long rows = (long)d.ny * d.nz, off = (long)blockIdx.y * 3 * rows;
     C* s = reinterpret_cast<C*>(smraw) + (size_t)t.l * NC * plane;
     const C* sa = S1 + (off + r.ra) * d.KXS;
-    if (early) grid_dep_launch();
     grid_dep_wait();
     line_inverse<T, NC, LC>(sa, r.two ? sa + d.KXS : sa, rows * d.KXS, s, plane, t.b, pl, tw);
     if (!r.on || !t.in) return;
@@ -594,7 +592,7 @@ template <bool GEN, int MAXT, int LC>
 __global__ void __launch_bounds__(MAXT, (line_fused_ctas<GEN, MAXT>()))
 line_fused(DemagDims d, float2* __restrict__ S1, const __grid_constant__ StageParams<float> p,
            const __grid_constant__ LineBatch bt, const __grid_constant__ LinePlan pl,
-           const float2* __restrict__ tw, int nt, int lines, int park_n, int fwd, int early) {
+           const float2* __restrict__ tw, int nt, int lines, int park_n, int fwd) {
     using C = float2;
     extern __shared__ __align__(16) unsigned char smraw[];
     if constexpr (LC > 0) {
@@ -610,7 +608,6 @@ line_fused(DemagDims d, float2* __restrict__ S1, const __grid_constant__ StagePa
     C* s = sp + c * plane;
     C* sa = S1 + (off + c * rows + r.ra) * d.KXS;
     C* sb = r.two ? sa + d.KXS : sa;
-    if (early) grid_dep_launch();
     grid_dep_wait();
     if (bt.mask && !bt.mask[g]) return;
     // Everything of the Runge-Kutta combination but the new derivative, summed
@@ -858,7 +855,7 @@ enum { kConvOne, kConvThree, kConvSplit };
 template <typename T, int FORM, int MAXT, int LC>
 __global__ void __launch_bounds__(MAXT, FORM == kConvSplit ? (MAXT <= 384 ? 2 : 1) : FORM == kConvOne ? 2 : LC > 0 && MAXT == kLineThreads32 ? 2 : line_blocks<T, MAXT>())
 line_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restrict__ tens,
-          const __grid_constant__ LinePlan pl, const typename Cplx<T>::type* __restrict__ tw, int lb, int ncol, int early) {
+          const __grid_constant__ LinePlan pl, const typename Cplx<T>::type* __restrict__ tw, int lb, int ncol) {
     using C = typename Cplx<T>::type;
     extern __shared__ __align__(16) unsigned char smraw[];
     const int L = LC ? LC : pl.L, tid = threadIdx.x;
@@ -882,7 +879,6 @@ line_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restr
     C* g = S2 + (long)blockIdx.y * 3 * cs + (long)ky * d.KXS + kx;
     const long tz = (long)KY2 * d.KXS, tc = (long)(L / 2 + 1) * tz;
     const T* tp = tens + (long)(up ? LY - ky : ky) * d.KXS + kx;
-    if (early) grid_dep_launch();
     if constexpr (FORM == kConvSplit) {
         // this thread's wave numbers u + 3 M i; their tensor entries (written long
         // before the previous pass) are on their way from the start
@@ -971,7 +967,7 @@ line_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restr
 template <typename T, int DIR, int MAXT>
 __global__ void __launch_bounds__(MAXT)
 line_y(DemagDims d, const typename Cplx<T>::type* __restrict__ in, typename Cplx<T>::type* __restrict__ out,
-       const __grid_constant__ LinePlan pl, const typename Cplx<T>::type* __restrict__ tw, int lb, int ncol, int early) {
+       const __grid_constant__ LinePlan pl, const typename Cplx<T>::type* __restrict__ tw, int lb, int ncol) {
     using C = typename Cplx<T>::type;
     extern __shared__ __align__(16) unsigned char smraw[];
     const int L = pl.L, np = pl.np, tid = threadIdx.x;
@@ -984,7 +980,6 @@ line_y(DemagDims d, const typename Cplx<T>::type* __restrict__ in, typename Cplx
     const long plane = (long)blockIdx.y * 3 * d.nz + cz;
     const C* gi = in + plane * rin * d.KXS + kx;
     C* go = out + plane * rout * d.KXS + kx;
-    if (early) grid_dep_launch();
     grid_dep_wait();
     C* s = reinterpret_cast<C*>(smraw) + l;
     if constexpr (DIR < 0) {
