@@ -304,7 +304,7 @@ mm_status mm_set_dmi(mm_state* s, mm_dmi_kind kind, double D, const double* D_ce
  * (h_k A_{k+1} + h_{k+1} A_k); energies use each cell's volume dx dy h_k.
  * The demag tensor must be built again (mm_demag_setup) after this call; h =
  * NULL returns to the equidistant grid.  Not with DMI (mm_set_dmi refuses
- * either order), not in the adjoint, always through the unfused stage path.
+ * either order), not in the adjoint.
  * MM_EINVAL unless nz equals the grid's nz, 2 <= nz <= 64 and every h is
  * finite and > 0. */
 mm_status mm_set_layers(mm_state* s, const double* h, int nz);

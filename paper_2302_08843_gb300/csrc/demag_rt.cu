@@ -695,7 +695,9 @@ bool launch_line_conv(const DemagDims& d, typename Cplx<T>::type* S2, const T* t
     if constexpr (sizeof(T) == 4) {
         if (o.pl.np > 1 && line_ct_use(kLineConv, d.LZ, &k)) line_ct_shape(d.LZ, ncol, &o);
     } else if (split) {
-        k = o.threads <= 384 ? line_conv<T, kConvSplit, 384, 0> : line_conv<T, kConvSplit, 768, 0>;
+        const bool wide = std::any_of(o.pl.R, o.pl.R + o.pl.np, [](int r) { return r == 6 || r == 8; });
+        if (wide) k = o.threads <= 384 ? line_conv<T, kConvSplitWide, 384, 0> : line_conv<T, kConvSplitWide, 768, 0>;
+        else k = o.threads <= 384 ? line_conv<T, kConvSplit, 384, 0> : line_conv<T, kConvSplit, 768, 0>;
     }
     const dim3 grid((unsigned)o.ctas, d.nb);
     line_launch(k, grid, o.threads, o.smem, st, d, S2, tens, o.pl, line_table<T>(o.pl), o.lb, (int)ncol);

@@ -286,32 +286,32 @@ __device__ __forceinline__ void line_start(typename Cplx<T>::type* s, int plane,
     __syncthreads();
 }
 
-// CALL with R_ = the radix; the FP64 plans hold none above 7 and no 6
-#define MM_LINE_RADIX(Rv, CALL)                                           \
+// CALL with R_ = the radix (Wv: plans with a 6 or an 8 come here too)
+#define MM_LINE_RADIX(Wv, Rv, CALL)                                           \
     switch (Rv) {                                                         \
         case 2: { constexpr int R_ = 2; CALL; } break;                     \
         case 3: { constexpr int R_ = 3; CALL; } break;                     \
         case 4: { constexpr int R_ = 4; CALL; } break;                     \
         case 5: { constexpr int R_ = 5; CALL; } break;                     \
         case 7: { constexpr int R_ = 7; CALL; } break;                     \
-        case 6: { constexpr int R_ = 6; CALL; } break; \
-        default: { constexpr int R_ = 8; CALL; } break; \
+        case 6: { constexpr int R_ = (Wv) ? 6 : 2; CALL; } break; \
+        default: { constexpr int R_ = (Wv) ? 8 : 2; CALL; } break; \
     }
-#define MM_LINE_RADIX_EVEN(Rv, CALL)                                      \
+#define MM_LINE_RADIX_EVEN(Wv, Rv, CALL)                                      \
     switch (Rv) {                                                         \
         case 2: { constexpr int R_ = 2; CALL; } break;                     \
         case 4: { constexpr int R_ = 4; CALL; } break;                     \
-        case 6: { constexpr int R_ = 6; CALL; } break; \
-        default: { constexpr int R_ = 8; CALL; } break; \
+        case 6: { constexpr int R_ = (Wv) ? 6 : 2; CALL; } break; \
+        default: { constexpr int R_ = (Wv) ? 8 : 2; CALL; } break; \
     }
 
-template <typename T, int DIR, int NC, int SH>
+template <typename T, int DIR, int NC, int SH, bool WIDE = true>
 __device__ __forceinline__ void line_mid_any(typename Cplx<T>::type* s, int plane, int lb, int b, const LinePlan& pl,
                                              int i, const typename Cplx<T>::type* tw) {
     const int R = DIR < 0 ? pl.R[i] : pl.R[pl.np - 1 - i];
     const int Ns = DIR < 0 ? pl.Ns[i] : pl.Nsi[i];
     const unsigned mg = DIR < 0 ? pl.mg[i] : pl.mgi[i];
-    MM_LINE_RADIX(R, (line_mid<T, DIR, R_, NC, SH>(s, plane, lb, b, pl.L, Ns, mg, tw)));
+    MM_LINE_RADIX(WIDE, R, (line_mid<T, DIR, R_, NC, SH>(s, plane, lb, b, pl.L, Ns, mg, tw)));
 }
 
 // passes I .. END-1 of a compiled length

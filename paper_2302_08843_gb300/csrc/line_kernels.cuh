@@ -142,10 +142,10 @@ __device__ __forceinline__ void line_inverse(const typename Cplx<T>::type* sa, c
         line_x_last<T, P.R[0], NC>(s, plane, b, LC, P.Nsi[np - 1], 0, tw);
     } else {
         const int np = pl.np, L = pl.L;
-        MM_LINE_RADIX(pl.R[np - 1], (line_x_first<T, R_, NC>(sa, sb, cs, s, plane, b, L)));
+        MM_LINE_RADIX(true, pl.R[np - 1], (line_x_first<T, R_, NC>(sa, sb, cs, s, plane, b, L)));
         __syncthreads();
         for (int i = 1; i < np - 1; ++i) line_mid_any<T, +1, NC, 4>(s, plane, 0, b, pl, i, tw);
-        MM_LINE_RADIX_EVEN(pl.R[0], (line_x_last<T, R_, NC>(s, plane, b, L, pl.Nsi[np - 1], pl.mgi[np - 1], tw)));
+        MM_LINE_RADIX_EVEN(true, pl.R[0], (line_x_last<T, R_, NC>(s, plane, b, L, pl.Nsi[np - 1], pl.mgi[np - 1], tw)));
     }
 }
 
@@ -163,7 +163,7 @@ __device__ __forceinline__ void line_forward(typename Cplx<T>::type* s, int plan
         line_f_first<T, P.R[0], NC>(s, plane, b, LC, nx);
         line_mids_ct<T, -1, NC, 4, LC, 1, P.np>(s, plane, 0, b, tw);
     } else {
-        MM_LINE_RADIX_EVEN(pl.R[0], (line_f_first<T, R_, NC>(s, plane, b, L, nx)));
+        MM_LINE_RADIX_EVEN(true, pl.R[0], (line_f_first<T, R_, NC>(s, plane, b, L, nx)));
         for (int i = 1; i < pl.np; ++i) line_mid_any<T, -1, NC, 4>(s, plane, 0, b, pl, i, tw);
     }
     if (!on) return;
@@ -850,10 +850,12 @@ __device__ __forceinline__ void line_product_one(typename Cplx<T>::type* g, long
 // slower, 90 against 80 us on 32 grids of 256x256x1: fewer CTAs per SM.)
 // FORM: kConvOne, a column in one thread's registers; kConvThree, a thread per
 // butterfly of all three components; kConvSplit, a thread per butterfly and
-// component, the product then taken wave number by wave number by all of them.
-enum { kConvOne, kConvThree, kConvSplit };
+// component, the product then taken wave number by wave number by all of them;
+// kConvSplitWide, that with radices 6 and 8 too, whose registers cost the plans
+// without them 1 to 3 % (film of 512x128x1: 47.5 -> 49.0 us).
+enum { kConvOne, kConvThree, kConvSplit, kConvSplitWide };
 template <typename T, int FORM, int MAXT, int LC>
-__global__ void __launch_bounds__(MAXT, FORM == kConvSplit ? (MAXT <= 384 ? 2 : 1) : FORM == kConvOne ? 2 : LC > 0 && MAXT == kLineThreads32 ? 2 : line_blocks<T, MAXT>())
+__global__ void __launch_bounds__(MAXT, FORM >= kConvSplit ? (MAXT <= 384 ? 2 : 1) : FORM == kConvOne ? 2 : LC > 0 && MAXT == kLineThreads32 ? 2 : line_blocks<T, MAXT>())
 line_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restrict__ tens,
           const __grid_constant__ LinePlan pl, const typename Cplx<T>::type* __restrict__ tw, int lb, int ncol) {
     using C = typename Cplx<T>::type;
@@ -867,8 +869,8 @@ line_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restr
         lb = kLb;
     }
     const int l = tid & ((1 << lb) - 1), u = tid >> lb;
-    const int c = FORM == kConvSplit ? min(u / M, 2) : 0;
-    const int b = FORM != kConvSplit ? u : u < 3 * M ? u - c * M : kLineIdle;
+    const int c = FORM >= kConvSplit ? min(u / M, 2) : 0;
+    const int b = FORM < kConvSplit ? u : u < 3 * M ? u - c * M : kLineIdle;
     const int col = (blockIdx.x << lb) + l;
     const bool valid = col < ncol;
     const int cc = valid ? col : ncol - 1;      // columns past the end follow the last one and store nothing
@@ -879,11 +881,12 @@ line_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restr
     C* g = S2 + (long)blockIdx.y * 3 * cs + (long)ky * d.KXS + kx;
     const long tz = (long)KY2 * d.KXS, tc = (long)(L / 2 + 1) * tz;
     const T* tp = tens + (long)(up ? LY - ky : ky) * d.KXS + kx;
-    if constexpr (FORM == kConvSplit) {
+    if constexpr (FORM >= kConvSplit) {
         // this thread's wave numbers u + 3 M i; their tensor entries (written long
         // before the previous pass) are on their way from the start
         static_assert(LC == 0 && sizeof(T) == 8, "the split form is FP64's");
-        constexpr int KP = 3;                           // the smallest radix of a plan is 8 at most
+        constexpr bool kWide = FORM == kConvSplitWide;
+        constexpr int KP = kWide ? 3 : 2;               // the smallest radix of a plan is 8, or 4, at most
         T t[KP][6];
 #pragma unroll
         for (int i = 0; i < KP; ++i) {
@@ -912,13 +915,13 @@ line_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restr
             __syncthreads();
         };
         const int np = pl.np;
-        MM_LINE_RADIX_EVEN(pl.R[0], (line_first<T, -1, R_, true, 1>(g, zs, 0, d.nz, s, 0, lb, b, L)));
+        MM_LINE_RADIX_EVEN(kWide, pl.R[0], (line_first<T, -1, R_, true, 1>(g, zs, 0, d.nz, s, 0, lb, b, L)));
         __syncthreads();
-        for (int i = 1; i < np; ++i) line_mid_any<T, -1, 1, 3>(s, 0, lb, b, pl, i, tw);
+        for (int i = 1; i < np; ++i) line_mid_any<T, -1, 1, 3, kWide>(s, 0, lb, b, pl, i, tw);
         product();
-        MM_LINE_RADIX(pl.R[np - 1], (line_start<T, +1, R_, 1, 3>(s, 0, lb, b, L)));
-        for (int i = 1; i < np - 1; ++i) line_mid_any<T, +1, 1, 3>(s, 0, lb, b, pl, i, tw);
-        MM_LINE_RADIX_EVEN(pl.R[0], (line_last<T, +1, R_, true, 1>(s, 0, lb, b, L, pl.Nsi[np - 1], pl.mgi[np - 1],
+        MM_LINE_RADIX(kWide, pl.R[np - 1], (line_start<T, +1, R_, 1, 3>(s, 0, lb, b, L)));
+        for (int i = 1; i < np - 1; ++i) line_mid_any<T, +1, 1, 3, kWide>(s, 0, lb, b, pl, i, tw);
+        MM_LINE_RADIX_EVEN(kWide, pl.R[0], (line_last<T, +1, R_, true, 1>(s, 0, lb, b, L, pl.Nsi[np - 1], pl.mgi[np - 1],
                                                                       tw, g, zs, 0, d.nz, valid)));
         return;
     }
@@ -947,14 +950,14 @@ line_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restr
             line_mids_ct<T, +1, 3, 3, LC, 1, np - 1>(s, plane, lb, b, tw);
             line_last<T, +1, P.R[0], true, 3>(s, plane, lb, b, L, P.Nsi[np - 1], 0, tw, g, zs, cs, d.nz, valid);
         } else {
-            MM_LINE_RADIX_EVEN(pl.R[0], (line_first<T, -1, R_, true, 3>(g, zs, cs, d.nz, s, plane, lb, b, L)));
+            MM_LINE_RADIX_EVEN(true, pl.R[0], (line_first<T, -1, R_, true, 3>(g, zs, cs, d.nz, s, plane, lb, b, L)));
             __syncthreads();
             const int np = pl.np;
             for (int i = 1; i < np - 1; ++i) line_mid_any<T, -1, 3, 3>(s, plane, lb, b, pl, i, tw);
-            MM_LINE_RADIX(pl.R[np - 1], (line_product<T, R_>(s, plane, lb, b, L, pl.Ns[np - 1], pl.mg[np - 1], tw, tp,
+            MM_LINE_RADIX(true, pl.R[np - 1], (line_product<T, R_>(s, plane, lb, b, L, pl.Ns[np - 1], pl.mg[np - 1], tw, tp,
                                                                 tz, tc, up, d.yz_swap)));
             for (int i = 1; i < np - 1; ++i) line_mid_any<T, +1, 3, 3>(s, plane, lb, b, pl, i, tw);
-            MM_LINE_RADIX_EVEN(pl.R[0], (line_last<T, +1, R_, true, 3>(s, plane, lb, b, L, pl.Nsi[np - 1],
+            MM_LINE_RADIX_EVEN(true, pl.R[0], (line_last<T, +1, R_, true, 3>(s, plane, lb, b, L, pl.Nsi[np - 1],
                                                                           pl.mgi[np - 1], tw, g, zs, cs, d.nz, valid)));
         }
     }
@@ -983,17 +986,17 @@ line_y(DemagDims d, const typename Cplx<T>::type* __restrict__ in, typename Cplx
     grid_dep_wait();
     C* s = reinterpret_cast<C*>(smraw) + l;
     if constexpr (DIR < 0) {
-        MM_LINE_RADIX_EVEN(pl.R[0], (line_first<T, -1, R_, true, 1>(gi, d.KXS, 0, d.ny, s, 0, lb, b, L)));
+        MM_LINE_RADIX_EVEN(true, pl.R[0], (line_first<T, -1, R_, true, 1>(gi, d.KXS, 0, d.ny, s, 0, lb, b, L)));
     } else {
-        MM_LINE_RADIX(pl.R[np - 1], (line_first<T, +1, R_, false, 1>(gi, d.KXS, 0, L, s, 0, lb, b, L)));
+        MM_LINE_RADIX(true, pl.R[np - 1], (line_first<T, +1, R_, false, 1>(gi, d.KXS, 0, L, s, 0, lb, b, L)));
     }
     __syncthreads();
     for (int i = 1; i < np - 1; ++i) line_mid_any<T, DIR, 1, 3>(s, 0, lb, b, pl, i, tw);
     if constexpr (DIR < 0) {
-        MM_LINE_RADIX(pl.R[np - 1], (line_last<T, -1, R_, false, 1>(s, 0, lb, b, L, pl.Ns[np - 1], pl.mg[np - 1], tw, go,
+        MM_LINE_RADIX(true, pl.R[np - 1], (line_last<T, -1, R_, false, 1>(s, 0, lb, b, L, pl.Ns[np - 1], pl.mg[np - 1], tw, go,
                                                                        d.KXS, 0, L, valid)));
     } else {
-        MM_LINE_RADIX_EVEN(pl.R[0], (line_last<T, +1, R_, true, 1>(s, 0, lb, b, L, pl.Nsi[np - 1], pl.mgi[np - 1], tw, go,
+        MM_LINE_RADIX_EVEN(true, pl.R[0], (line_last<T, +1, R_, true, 1>(s, 0, lb, b, L, pl.Nsi[np - 1], pl.mgi[np - 1], tw, go,
                                                                       d.KXS, 0, d.ny, valid)));
     }
 }
