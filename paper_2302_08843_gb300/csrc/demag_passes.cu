@@ -2112,14 +2112,22 @@ template <typename T, int L, int DIR> static void launch_y(const DemagDims& d, c
     if constexpr (sizeof(T) == 4 && L >= 16 && is_pow2(L)) {
         if (launch_py_tma<L, DIR>(d, in, out, st)) return;
     }
-    // FP64 lines of 16 points up take the line engine (128x128x32: 144 and 157 us
-    // -> 119 and 126 us); FP32 lines the compiled engines, which stay faster where
-    // exchanges and not FP64 instructions bound the pass (384 points: 29 and 33 us
-    // against 54 and 44)
-    if constexpr (sizeof(T) == 8 && L >= 16) {
+    // FP64 lines of 16 to 1024 points take the line engine (128x128x32: 144 and 157
+    // us -> 119 and 126 us; from 2048 points on a CTA holds one column of it, less
+    // than a sector: 49 against 44 us on 16x1024x4); FP32 lines the compiled
+    // engines, which stay faster where exchanges and not FP64 instructions bound
+    // the pass (384 points: 29 and 33 us against 54 and 44)
+    if constexpr (sizeof(T) == 8 && L >= 16 && L < 2048) {
         if (launch_line_y<T, DIR>(d, in, out, st)) return;
     }
     if constexpr (sizeof(T) == 4 || L < 16 || L >= 2048) launch_py<T, L, DIR>(d, in, out, st);
+}
+
+// FP64 x lines of 2048 points on stay on the compiled passes, whose four radix-8
+// passes need half the threads of a line (1024x1024x1: 244 and 233 us against 339
+// and 303, 1024x64x1 31 and 30 against 39 and 35)
+template <typename T, int L> constexpr bool line_x_use(const DemagDims& d) {
+    return !d.classic && (sizeof(T) == 4 || L < 2048);
 }
 
 template <typename T, int L> static void launch_x_fwd(const DemagDims& d, const T* m, const T* Ms_cell, T Ms,
@@ -2131,7 +2139,7 @@ template <typename T, int L> static void launch_x_fwd(const DemagDims& d, const 
     in.m = m;
     in.Ms_cell = Ms_cell;
     in.Ms = Ms;
-    if (!d.classic && launch_line_x_fwd<T>(d, in, S1, st)) return;
+    if (line_x_use<T, L>(d) && launch_line_x_fwd<T>(d, in, S1, st)) return;
     // lines too short or too long for the engine, and the classic FP32 passes
     if constexpr (sizeof(T) == 4 || L < 16 || L >= 2048) launch_p1<T, L>(d, m, Ms_cell, Ms, S1, st);
 }
@@ -2141,7 +2149,7 @@ template <typename T, int L> static void launch_x_inv(const DemagDims& d, const 
     if constexpr (sizeof(T) == 4 && L >= 16 && is_pow2(L)) {
         if (launch_p5_tma<L>(d, S1, h, st)) return;
     }
-    if (!d.classic && launch_line_x_inv<T>(d, S1, h, st)) return;
+    if (line_x_use<T, L>(d) && launch_line_x_inv<T>(d, S1, h, st)) return;
     if constexpr (sizeof(T) == 4 || L < 16 || L >= 2048) launch_p5<T, L>(d, S1, h, st);
 }
 
