@@ -124,6 +124,8 @@ template <typename T>
 bool launch_line_conv(const DemagDims& d, typename Cplx<T>::type* S2, const T* tens, cudaStream_t st);
 // copy the runtime-plan lengths' twiddle tables to the current device
 cudaError_t upload_twiddles_rt();
+// let a kernel be launched with `bytes` of dynamic shared memory on the current device (demag_rt.cu)
+void allow_shared(const void* kernel, size_t bytes);
 
 // diagnostic: one CTA whose bounded wait on a never-completed mbarrier runs out
 void launch_diag_wait(int* err, unsigned spins, cudaStream_t st);

@@ -1788,10 +1788,8 @@ template <typename T, int L> constexpr int g_p3() {
                       ? 1 : (int)(kP3Smem / ((size_t)3 * L * b_p3<T, L>() * sizeof(typename Cplx<T>::type))));
 }
 
-// raise a kernel's dynamic shared-memory limit when the request comes near the
-// 48 KB default (kernels may also hold a little static shared memory)
 template <typename K> static void set_smem(K kernel, size_t bytes) {
-    if (bytes > 40 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    allow_shared(reinterpret_cast<const void*>(kernel), bytes);
 }
 
 template <typename T, int L> static void launch_p1(const DemagDims& d, const T* m, const T* Ms_cell, T Ms,

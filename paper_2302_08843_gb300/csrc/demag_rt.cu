@@ -431,9 +431,41 @@ rt_z_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restr
 }
 
 // ------------------------------------------------------------- launchers ----
+// The limit belongs to a kernel and a device, not to a launch, and one kernel
+// serves lines of many lengths: it is raised once, to all that a CTA may have.
+// Set to each launch's own size, a thread with a shorter line would take it from
+// under another's longer one between that thread's two calls.  (Requests that
+// stay clear of the 48 KB every kernel may use, a little static shared memory
+// included, need nothing.)  A limit that could not be raised shows as the
+// launch's own error.
+void allow_shared(const void* kernel, size_t bytes) {
+    if (bytes <= 40 * 1024) return;
+    struct Raised { const void* kernel; int device; };
+    constexpr size_t kSlots = 2048;             // open addressing; when full, kernels are raised anew each time
+    static Raised raised[kSlots];
+    static std::mutex lock;
+    int dev = 0, most = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return;
+    const size_t h = ((reinterpret_cast<uintptr_t>(kernel) >> 4) * 0x9E3779B97F4A7C15ull >> 40) + dev;
+    std::lock_guard<std::mutex> guard(lock);
+    Raised* slot = nullptr;
+    for (size_t q = 0; q < 64 && !slot; ++q) {
+        Raised& r = raised[(h + q) % kSlots];
+        if (r.kernel == kernel && r.device == dev) return;
+        if (!r.kernel) slot = &r;
+    }
+    cudaFuncAttributes a;
+    if (cudaFuncGetAttributes(&a, kernel) != cudaSuccess ||
+        cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)a.sharedSizeBytes) !=
+            cudaSuccess)
+        return;
+    if (slot) *slot = Raised{kernel, dev};
+}
+
 namespace {
 template <typename K> void rt_smem(K kernel, size_t bytes) {
-    if (bytes > 40 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    allow_shared(reinterpret_cast<const void*>(kernel), bytes);
 }
 constexpr size_t kRtSmem = 200 * 1024;
 // lines (or columns) per CTA: up to `cap`, as many as two (or four) buffers of L complex values allow
@@ -538,7 +570,7 @@ template <typename T> bool line_shape(int L, long ncol, int nb, int nc, bool con
 // Dormand-Prince steps of the film 3080 us instead of 2831.
 template <typename... KArgs, typename... Args>
 void line_launch(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args&&... args) {
-    if (smem > 40 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_shared(reinterpret_cast<const void*>(kernel), smem);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)threads);
