@@ -50,7 +50,7 @@ template <typename T> __device__ __forceinline__ void axis_of(const AdjParams<T>
 template <typename T> __global__ void adj_prep_kernel(AdjParams<T> p) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= p.N) return;
-    const int N = p.N;
+    const long N = p.N;      // 64 bits: 3 N passes 2^31 from 716 million cells on
     const T mx = p.m[i], my = p.m[N + i], mz = p.m[2 * N + i];
     const T hx = p.h[i], hy = p.h[N + i], hz = p.h[2 * N + i];
     const T ux = p.u[i], uy = p.u[N + i], uz = p.u[2 * N + i];
@@ -78,7 +78,7 @@ template <typename T> __global__ void adj_prep_kernel(AdjParams<T> p) {
 template <typename T> __global__ void adj_finish_kernel(AdjParams<T> p) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= p.N) return;
-    const int N = p.N;
+    const long N = p.N;      // 64 bits: 3 N passes 2^31 from 716 million cells on
     const int x = i % p.nx, yz = i / p.nx, y = yz % p.ny, z = yz / p.ny;
     const T Ms = p.Ms_cell ? p.Ms_cell[i] : p.Ms;
     T lx = p.part[i], ly = p.part[N + i], lz = p.part[2 * N + i];
@@ -155,7 +155,7 @@ template <typename T> __global__ void adj_finish_kernel(AdjParams<T> p) {
 // u = dt b_last lambda_y (cotangent of the last stage derivative)
 template <typename T> __global__ void adj_renorm_kernel(const T* __restrict__ y, const T* __restrict__ lam,
                                                         T* __restrict__ lam_y, T* __restrict__ lam_acc,
-                                                        T* __restrict__ u, T cb, int N) {
+                                                        T* __restrict__ u, T cb, long N) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     const T a = y[i], b = y[N + i], c = y[2 * N + i];
@@ -174,15 +174,15 @@ template <typename T> __global__ void adj_renorm_kernel(const T* __restrict__ y,
 
 template <typename T>
 void launch_adj_prep(const AdjParams<T>& p, cudaStream_t st) {
-    adj_prep_kernel<T><<<(p.N + 255) / 256, 256, 0, st>>>(p);
+    adj_prep_kernel<T><<<(unsigned)((p.N + 255L) / 256), 256, 0, st>>>(p);
 }
 template <typename T>
 void launch_adj_finish(const AdjParams<T>& p, cudaStream_t st) {
-    adj_finish_kernel<T><<<(p.N + 255) / 256, 256, 0, st>>>(p);
+    adj_finish_kernel<T><<<(unsigned)((p.N + 255L) / 256), 256, 0, st>>>(p);
 }
 template <typename T>
 void launch_adj_renorm(const T* y, const T* lam, T* lam_y, T* lam_acc, T* u, double cb, int N, cudaStream_t st) {
-    adj_renorm_kernel<T><<<(N + 255) / 256, 256, 0, st>>>(y, lam, lam_y, lam_acc, u, (T)cb, N);
+    adj_renorm_kernel<T><<<(unsigned)((N + 255L) / 256), 256, 0, st>>>(y, lam, lam_y, lam_acc, u, (T)cb, N);
 }
 
 template void launch_adj_prep<float>(const AdjParams<float>&, cudaStream_t);

@@ -2376,6 +2376,9 @@ bool fused_stage(const DemagDims& d, float2* S1, const StageParams<float>& p, cu
 
 bool fused_stage_supported(const DemagDims& d, const StageParams<float>& p) {
     if (!d.err || d.LX < 16 || d.LX > 4096 || d.nx % 2 != 0) return false;
+    // k5_fused indexes the three components in 32 bits (64 cost 256x256x64 7531 -> 7744 us
+    // for five RK4 steps): 716 million cells and more take the separate passes
+    if (3L * d.nx * d.ny * d.nz >= 1L << 31) return false;
     if (fft_rt_length(d.LX)) return false;        // compiled engines only (powers of two, r 2^a)
     if (p.alpha_cell || p.zw || p.D_cell || (!p.Ms_cell && p.Ms == 0.f)) return false;
     if ((p.Ms_cell || p.A_cell || p.Ku_cell || p.lay) && p.dmi) return false;

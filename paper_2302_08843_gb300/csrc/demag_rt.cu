@@ -664,8 +664,14 @@ bool launch_line_x_inv(const DemagDims& d, const typename Cplx<T>::type* S1, T* 
     return true;
 }
 
+// The fused stage indexes the three components of a grid in 32 bits (in 64, five
+// RK4 steps of a 20x45x4 stack of layers took 461 us instead of 441): 716 million
+// cells and more take the separate passes, whose stage kernel has 64.
+static bool line_fused_fits(const DemagDims& d) { return 3L * d.nx * d.ny * d.nz < 1L << 31; }
+
 int line_fused_blocks(const DemagDims& d, long max_ctas) {
     LineXShape o;
+    if (!line_fused_fits(d)) return 0;
     if (d.nb > 65535 || !line_x_shape<float>(d.LX, line_fused_pairs(d), 1, 3, max_ctas, &o)) return 0;
     return (int)o.ctas;
 }
@@ -673,7 +679,8 @@ int line_fused_blocks(const DemagDims& d, long max_ctas) {
 bool launch_line_fused(const DemagDims& d, float2* S1, const StageParams<float>& p, const LineBatch* bt, bool gen,
                        bool fwd, long max_ctas, cudaStream_t st) {
     LineXShape o;
-    if (d.nb > 65535 || !line_x_shape<float>(d.LX, line_fused_pairs(d), 1, 3, max_ctas, &o)) return false;
+    if (!line_fused_fits(d) || d.nb > 65535 || !line_x_shape<float>(d.LX, line_fused_pairs(d), 1, 3, max_ctas, &o))
+        return false;
     LineBatch b{};
     if (bt) b = *bt;
     auto k = gen ? (o.threads <= 256 ? line_fused<true, 256, 0> : line_fused<true, 1024, 0>)

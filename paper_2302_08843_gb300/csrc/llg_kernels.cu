@@ -103,7 +103,7 @@ template <typename T, int VEC, bool UNI, bool DMI>
 __global__ void __launch_bounds__(kStageThreads, stage_min_blocks<T, DMI>()) stage_kernel(StageParams<T> p) {
     using LV = Vec<T, VEC>;
     const int nx = p.nx, ny = p.ny, nz = p.nz;
-    const int N = (int)p.N;
+    const long N = p.N;                // 64 bits: 3 N passes 2^31 from 716 million cells on
     const int x0 = (blockIdx.x * blockDim.x + threadIdx.x) * VEC;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
