@@ -346,7 +346,7 @@ __device__ __forceinline__ void line_acc_prod(float2& s, float a, float b) {
 // One item: the cells (x, ya) and (x, yb) of the line's two rows as the lanes
 // of paired FP32 instructions.  ia, ib: their indices in the grid (ib = ia for
 // a missing second row); v: the demag field in, Ms next out; rk: the known part
-// of next and of the error (line_known).
+// of the derivatives' sum and of the error (line_known).
 template <bool GEN>
 __device__ __forceinline__ void line_cells(const StageParams<float>& p, const LineBatch& bt, int g, long off, int x,
                                            int y, int z, bool two, const float2 (&rk)[6], float2 (&v)[3],
@@ -509,8 +509,12 @@ __device__ __forceinline__ void line_cells(const StageParams<float>& p, const Li
         st(p.acc_out, a, b, c);
     }
     if (p.next || p.want_err) {
-        const float2 dt = f2s(batch ? (float)bt.dt[g] : p.dtT), ck = f2mul(dt, f2s(p.ckT));
-        float2 ox = f2fma(ck, kx, rk[0]), oy = f2fma(ck, ky, rk[1]), oz = f2fma(ck, kz, rk[2]);
+        // m + dt (sum of all derivatives): one rounding at the size of m
+        const float2 dt = f2s(batch ? (float)bt.dt[g] : p.dtT), ck = f2s(p.ckT);
+        const float* mn = p.mn + off;
+        const float2 m0x = lds(mn), m0y = lds(mn + N), m0z = lds(mn + 2 * N);
+        float2 ox = f2fma(dt, f2fma(ck, kx, rk[0]), m0x), oy = f2fma(dt, f2fma(ck, ky, rk[1]), m0y),
+               oz = f2fma(dt, f2fma(ck, kz, rk[2]), m0z);
         if (p.want_err) {
             auto worst = [&](float e, float m0, float u) {
                 const float n = fabsf(e), sc = p.atolT + p.rtolT * fmaxf(fabsf(m0), fabsf(u));
@@ -518,8 +522,7 @@ __device__ __forceinline__ void line_cells(const StageParams<float>& p, const Li
                 if (n * red.ed > red.en * sc) { red.en = n; red.ed = sc; }
             };
             const bool on_next = p.err_on_next;
-            const float* mn = p.mn + off;
-            const float2 m0x = lds(mn), m0y = lds(mn + N), m0z = lds(mn + 2 * N), ebk = f2mul(dt, f2s(p.eb_kT));
+            const float2 ebk = f2mul(dt, f2s(p.eb_kT));
             const float2 eX = f2fma(ebk, kx, rk[3]), eY = f2fma(ebk, ky, rk[4]), eZ = f2fma(ebk, kz, rk[5]);
             worst(eX.x, m0x.x, on_next ? ox.x : mx.x); worst(eX.y, m0x.y, on_next ? ox.y : mx.y);
             worst(eY.x, m0y.x, on_next ? oy.x : my.x); worst(eY.y, m0y.y, on_next ? oy.y : my.y);
@@ -539,16 +542,15 @@ __device__ __forceinline__ void line_cells(const StageParams<float>& p, const Li
 }
 
 // The part of an item's Runge-Kutta combination that does not wait for the
-// field: mn + dt sum_j kc_j kin_j (w[0..2]) and dt sum_j eb_j kin_j (w[3..5]).
+// field: sum_j kc_j kin_j (w[0..2]) and dt sum_j eb_j kin_j (w[3..5]).  The state
+// is left to the cell update: added here it would be rounded once more.
 template <int NK>
 __device__ __forceinline__ void line_known(const StageParams<float>& p, float dtv, long off, int ia, int ib,
-                                           bool next, bool err, float2 (&w)[6]) {
+                                           float2 (&w)[6]) {
     const int N = (int)p.N;
-    float2 k[NK > 0 ? NK : 1][3], m0[3];
+    float2 k[NK > 0 ? NK : 1][3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const float* mn = p.mn + off + c * N;
-        m0[c] = next ? make_float2(__ldcg(mn + ia), __ldcg(mn + ib)) : f2s(0.f);
 #pragma unroll
         for (int q = 0; q < NK; ++q) {
             const float* a = p.kin[q] + off + c * N;
@@ -564,7 +566,7 @@ __device__ __forceinline__ void line_known(const StageParams<float>& p, float dt
             n = f2fma(f2s(p.kcT[q]), k[q][c], n);
             e = f2fma(f2s(p.ebT[q]), k[q][c], e);
         }
-        w[c] = f2fma(dt, n, m0[c]);
+        w[c] = n;
         w[3 + c] = f2mul(dt, e);
     }
 }
@@ -610,7 +612,7 @@ line_fused(DemagDims d, float2* __restrict__ S1, const __grid_constant__ StagePa
     C* sb = r.two ? sa + d.KXS : sa;
     grid_dep_wait();
     if (bt.mask && !bt.mask[g]) return;
-    // Everything of the Runge-Kutta combination but the new derivative, summed
+    // The Runge-Kutta combination of the derivatives that are there, summed
     // while the registers are free and all its loads can be in flight, and
     // parked in shared memory for this thread's cell updates: [next][err][3][nx]
     const bool next = p.next != nullptr, err = p.want_err != 0;
@@ -622,13 +624,13 @@ line_fused(DemagDims d, float2* __restrict__ S1, const __grid_constant__ StagePa
             const int ia = x + nx * (int)r.ra, ib = r.two ? ia + nx : ia;
             float2 w[6];
             switch (p.nk) {
-                case 0: line_known<0>(p, dtv, off * nx, ia, ib, next, err, w); break;
-                case 1: line_known<1>(p, dtv, off * nx, ia, ib, next, err, w); break;
-                case 2: line_known<2>(p, dtv, off * nx, ia, ib, next, err, w); break;
-                case 3: line_known<3>(p, dtv, off * nx, ia, ib, next, err, w); break;
-                case 4: line_known<4>(p, dtv, off * nx, ia, ib, next, err, w); break;
-                case 5: line_known<5>(p, dtv, off * nx, ia, ib, next, err, w); break;
-                default: line_known<6>(p, dtv, off * nx, ia, ib, next, err, w); break;
+                case 0: line_known<0>(p, dtv, off * nx, ia, ib, w); break;
+                case 1: line_known<1>(p, dtv, off * nx, ia, ib, w); break;
+                case 2: line_known<2>(p, dtv, off * nx, ia, ib, w); break;
+                case 3: line_known<3>(p, dtv, off * nx, ia, ib, w); break;
+                case 4: line_known<4>(p, dtv, off * nx, ia, ib, w); break;
+                case 5: line_known<5>(p, dtv, off * nx, ia, ib, w); break;
+                default: line_known<6>(p, dtv, off * nx, ia, ib, w); break;
             }
             float2* o = park + x;
             if (next) { o[0] = w[0]; o[nx] = w[1]; o[2 * nx] = w[2]; o += 3 * nx; }
