@@ -87,10 +87,9 @@ LinePlan host_plan(int L, int rmax, bool one) {
 
 }  // namespace
 
-// total entries of the concatenated twiddle tables (a compile-time bound for
-// the device arrays; checked against the host table at upload)
-constexpr int kTwRt = 173884;
-static __device__ double2 g_twrt64[kTwRt];
+// the concatenated twiddle tables (kTwRt, a compile-time bound, is checked against
+// the host table at upload)
+static __device__ double2 g_twrt64[2 * kTwRt];
 static __device__ float2 g_twrt32[kTwRt];
 
 // device addresses of the tables, per device (set by the upload)
@@ -151,7 +150,7 @@ cudaError_t upload_twiddles_rt() {
     static std::vector<double2> h64;
     static std::vector<float2> h32;
     if (h64.empty()) {
-        h64.resize(kTwRt);
+        h64.resize(2 * kTwRt);
         h32.resize(kTwRt);
         for (size_t i = 0; i < t.lengths.size(); ++i) {
             const int L = t.lengths[i];
@@ -159,11 +158,12 @@ cudaError_t upload_twiddles_rt() {
                 double c, sn;
                 twiddle_entry(L, m, &c, &sn);
                 h64[t.offsets[i] + m] = make_double2(c, sn);
+                h64[kTwRt + t.offsets[i] + m] = line_turn(m, L) ? make_double2(sn, -c / sn) : make_double2(c, sn / c);
                 h32[t.offsets[i] + m] = make_float2((float)c, (float)sn);
             }
         }
     }
-    cudaError_t e = cudaMemcpyToSymbol(g_twrt64, h64.data(), sizeof(double2) * kTwRt);
+    cudaError_t e = cudaMemcpyToSymbol(g_twrt64, h64.data(), sizeof(double2) * 2 * kTwRt);
     if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_twrt32, h32.data(), sizeof(float2) * kTwRt);
     int dev = 0;
     void *p64 = nullptr, *p32 = nullptr;

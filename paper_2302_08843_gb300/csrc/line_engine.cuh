@@ -20,9 +20,9 @@
 // half of a forward's input, and the dropped half of an inverse's output, are
 // the registers q >= R/2 of that pass.
 //
-// Twiddled radix-2 steps are folded into multiply-adds: X = a + w b (four) and,
-// in FP64, Y = 2 a - X (two), 3 instructions per point and level against 3.5 for
-// radix-8 passes that multiply first.  FP64 instructions are what an FP64
+// Twiddled radix-2 steps are folded into multiply-adds (LineTwiddle), in FP64 six
+// for both outputs: 3 instructions per point and level against 3.5 for radix-8
+// passes that multiply first.  FP64 instructions are what an FP64
 // pass spends its time on (one warp instruction per 19 cycles and SM; 64
 // cycles for a single warp of a quarter SM, dependent or not), so FP64 plans
 // take radix 4, many threads and, against a radix-2 pass left over, radix 8;
@@ -34,6 +34,14 @@
 namespace mm {
 
 constexpr int kLineMaxPass = 12;
+// entries of the concatenated tables W_L^m; behind them, in FP64, the same twiddles
+// as LineTwiddle takes them
+constexpr int kTwRt = 173884;
+// |Im W_L^m| > |Re W_L^m| (8 m mod 4 L between L and 3 L)
+__host__ __device__ __forceinline__ constexpr bool line_turn(int m, int L) {
+    const int q = 8 * m - (2 * m >= L ? 4 * L : 0);
+    return q > L && q < 3 * L;
+}
 constexpr int kLineIdle = 1 << 20;       // butterfly number of a thread without a line: past every pass's count
 
 struct LinePlan {
@@ -128,19 +136,56 @@ __device__ __forceinline__ int line_mod(int b, int Ns, unsigned mg) {
 template <int SH> __host__ __device__ __forceinline__ int line_place(int e) { return e + (e >> SH); }
 __host__ __device__ __forceinline__ int line_len(int L) { return L + (L >> 3) + 1; }
 
-// x = a + w b, y = a - w b.  FP64 forms y = 2 a - x (six instructions in all);
-// FP32, which is not bound by them, forms both directly: 2 a - x would carry the
-// rounding of a large x into a small y, as the spectrum of a nearly uniform
-// magnetisation has them side by side.
-template <typename C> __device__ __forceinline__ void bf2(C& a, C& b, C w) {
-    using T = decltype(C::x);
-    const C x = mk<C>(fma(w.x, b.x, fma(-w.y, b.y, a.x)), fma(w.x, b.y, fma(w.y, b.x, a.y)));
-    if constexpr (sizeof(T) == 4) b = mk<C>(fma(-w.x, b.x, fma(w.y, b.y, a.x)), fma(-w.x, b.y, fma(-w.y, b.x, a.y)));
-    else b = mk<C>(fma((T)2, a.x, -x.x), fma((T)2, a.y, -x.y));
-    a = x;
+// -v or v; FP64 on the integer side (FP64 instructions are what an FP64 pass is made of)
+__device__ __forceinline__ float line_flip(float v, bool neg) { return neg ? -v : v; }
+__device__ __forceinline__ double line_flip(double v, bool neg) {
+    return __hiloint2double(__double2hiint(v) ^ (neg ? (int)0x80000000 : 0), __double2loint(v));
 }
-// the same with w replaced by DIR i w
-template <int DIR, typename C> __device__ __forceinline__ void bf2i(C& a, C& b, C w) { bf2(a, b, mul_i<DIR>(w)); }
+
+// Twiddles of the folded butterflies and x = a + w b, y = a - w b, neither formed
+// from the other: y = 2 a - x would carry the rounding of a large x into a small
+// y, as the spectrum of a nearly uniform magnetisation has them side by side.
+//
+// FP32 takes w as it is, eight multiply-adds.
+template <typename T, int DIR> struct LineTwiddle {
+    float2 w;
+    __device__ __forceinline__ LineTwiddle(const float2* tw, int m, int) : w(__ldg(tw + m)) {
+        if (DIR > 0) w.y = -w.y;
+    }
+    __device__ __forceinline__ void bf2(float2& a, float2& b) const { bf2(a, b, w); }
+    __device__ __forceinline__ void bf2i(float2& a, float2& b) const { bf2(a, b, mul_i<DIR>(w)); }
+    static __device__ __forceinline__ void bf2(float2& a, float2& b, float2 w) {
+        const float2 x = make_float2(fma(w.x, b.x, fma(-w.y, b.y, a.x)), fma(w.x, b.y, fma(w.y, b.x, a.y)));
+        b = make_float2(fma(-w.x, b.x, fma(w.y, b.y, a.x)), fma(-w.x, b.y, fma(-w.y, b.x, a.y)));
+        a = x;
+    }
+};
+// FP64, whose instructions bound the pass, takes w = c (1 + i t), |t| <= 1, after
+// a quarter turn where |Im w| > |Re w| (Linzer and Feig 1993): w b costs two
+// multiply-adds up to the factor c, which the two sums take in, six in all.  The
+// turn costs selections on the integer side, which the twiddle's index decides:
+// kept with the twiddle they would wait for its load (32x32x4: 1342 against 1304 us
+// for ten RK4 steps).
+template <int DIR> struct LineTwiddle<double, DIR> {
+    double c, t;
+    bool turn;
+    __device__ __forceinline__ LineTwiddle(const double2* tw, int m, int L) : turn(line_turn(m, L)) {
+        const double2 e = __ldg(tw + kTwRt + m);
+        c = e.x;
+        t = e.y;
+    }
+    __device__ __forceinline__ void bf2(double2& a, double2& b) const { bf2(a, b, turn, false); }
+    __device__ __forceinline__ void bf2i(double2& a, double2& b) const { bf2(a, b, !turn, !turn); }
+    // u = b, or -DIR i b (quarter), or DIR i b (quarter and back)
+    __device__ __forceinline__ void bf2(double2& a, double2& b, bool quarter, bool back) const {
+        const double ux = quarter ? b.y : b.x, uy = quarter ? b.x : b.y;
+        const bool nx = quarter && (DIR < 0) != back, ny = quarter && (DIR > 0) != back;
+        const double px = line_flip(ux, nx), py = line_flip(uy, ny);
+        const double vx = fma(DIR < 0 ? -t : t, py, px), vy = fma(DIR < 0 ? t : -t, px, py);
+        b = make_double2(fma(-c, vx, a.x), fma(-c, vy, a.y));
+        a = make_double2(fma(c, vx, a.x), fma(c, vy, a.y));
+    }
+};
 
 // DFT of R values, no twiddles; HALF: the upper half of the inputs is zero
 template <int DIR, int R, bool HALF, typename C> __device__ __forceinline__ void line_dft(C (&x)[R]) {
@@ -181,41 +226,42 @@ template <typename T, int DIR, int R, int NC>
 __device__ __forceinline__ void line_butterfly(typename Cplx<T>::type (&x)[NC][R], const typename Cplx<T>::type* tw,
                                                int k, int step, int L) {
     using C = typename Cplx<T>::type;
+    using Tw = LineTwiddle<T, DIR>;
     auto W = [&](int m) {
         C w = __ldg(tw + m);
         if (DIR > 0) w.y = -w.y;
         return w;
     };
     if constexpr (R == 2) {
-        const C w = W(k * step);
+        const Tw w(tw, k * step, L);
 #pragma unroll
-        for (int c = 0; c < NC; ++c) bf2(x[c][0], x[c][1], w);
+        for (int c = 0; c < NC; ++c) w.bf2(x[c][0], x[c][1]);
     } else if constexpr (R == 4) {
-        const C w1 = W(k * step), w2 = W(2 * k * step);
+        const Tw w1(tw, k * step, L), w2(tw, 2 * k * step, L);
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
             C* a = x[c];
-            bf2(a[0], a[2], w2);          // t0, t1
-            bf2(a[1], a[3], w2);          // t2, t3
-            bf2(a[0], a[1], w1);          // X0, X2
-            bf2i<DIR>(a[2], a[3], w1);    // X1, X3
+            w2.bf2(a[0], a[2]);           // t0, t1
+            w2.bf2(a[1], a[3]);           // t2, t3
+            w1.bf2(a[0], a[1]);           // X0, X2
+            w1.bf2i(a[2], a[3]);          // X1, X3
             const C x1 = a[2];
             a[2] = a[1]; a[1] = x1;
         }
     } else if constexpr (R == 8) {
         // W_8 w1 = W_L^(k step + L/8)
-        const C w1 = W(k * step), w2 = W(2 * k * step), w4 = W(4 * k * step), u = W(k * step + L / 8);
+        const Tw w1(tw, k * step, L), w2(tw, 2 * k * step, L), w4(tw, 4 * k * step, L), u(tw, k * step + L / 8, L);
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
             C* a = x[c];
-            bf2(a[0], a[4], w4); bf2(a[2], a[6], w4);
-            bf2(a[0], a[2], w2); bf2i<DIR>(a[4], a[6], w2);     // E0 E2 | E1 E3 in a0 a2 a4 a6
-            bf2(a[1], a[5], w4); bf2(a[3], a[7], w4);
-            bf2(a[1], a[3], w2); bf2i<DIR>(a[5], a[7], w2);     // O0 O2 | O1 O3 in a1 a3 a5 a7
-            bf2(a[0], a[1], w1);            // X0, X4
-            bf2(a[4], a[5], u);             // X1, X5
-            bf2i<DIR>(a[2], a[3], w1);      // X2, X6
-            bf2i<DIR>(a[6], a[7], u);       // X3, X7
+            w4.bf2(a[0], a[4]); w4.bf2(a[2], a[6]);
+            w2.bf2(a[0], a[2]); w2.bf2i(a[4], a[6]);     // E0 E2 | E1 E3 in a0 a2 a4 a6
+            w4.bf2(a[1], a[5]); w4.bf2(a[3], a[7]);
+            w2.bf2(a[1], a[3]); w2.bf2i(a[5], a[7]);     // O0 O2 | O1 O3 in a1 a3 a5 a7
+            w1.bf2(a[0], a[1]);             // X0, X4
+            u.bf2(a[4], a[5]);              // X1, X5
+            w1.bf2i(a[2], a[3]);            // X2, X6
+            u.bf2i(a[6], a[7]);             // X3, X7
             const C x4 = a[1], x1 = a[4], x6 = a[3], x3 = a[6];
             a[1] = x1; a[3] = x3; a[4] = x4; a[6] = x6;
         }

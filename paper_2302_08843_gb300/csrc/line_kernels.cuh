@@ -763,12 +763,6 @@ __device__ __forceinline__ void line_last(const typename Cplx<T>::type* s, int p
     }
 }
 
-// -v or v; FP64 on the integer side (FP64 instructions are what an FP64 pass is made of)
-__device__ __forceinline__ float line_flip(float v, bool neg) { return neg ? -v : v; }
-__device__ __forceinline__ double line_flip(double v, bool neg) {
-    return __hiloint2double(__double2hiint(v) ^ (neg ? (int)0x80000000 : 0), __double2loint(v));
-}
-
 // h^ = T M^ of one wave number; t: the octant's xx, xy, xz, yy, yz, zz; ny, nz:
 // whether the odd components along y and along z change sign here
 template <typename T, typename C>
