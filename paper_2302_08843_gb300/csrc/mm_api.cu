@@ -667,7 +667,8 @@ mm_status adjoint_impl(mm_state* s, const void* m_n, const void* lam_np1, void* 
     T* Ahw = A[17];
     T* Apart = A[18];
     const T* ms[4] = {(const T*)m_n, Am[0], Am[1], Am[2]};
-    // forward recompute of the stage inputs, fields and derivatives
+    // forward recompute of the stage inputs, fields and derivatives (to rounding the
+    // step's own: DemagDims::classic is for the steps alone)
     const bool line = line_path<T>(s);
     for (int st = 0; st < 4; ++st) {
         StageParams<T> p;
