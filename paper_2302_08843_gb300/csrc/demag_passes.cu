@@ -2291,11 +2291,19 @@ static void launch_p3_layers(const DemagDims& d, typename Cplx<T>::type* S2, con
     k<<<grid, dim3(kLayCols, kLayRows), sm, st>>>(d, S2, tens);
 }
 
-// largest padded y extent of a 2-D grid (nz = 1) whose y transforms and tensor
-// multiply run as one pass of the z-pass kernels along y (32 served 256x256x1
-// grids: 88 us against 103 us for two y passes and the product; longer lines
-// leave a CTA of the line engine one column, less than a sector of each row)
-constexpr int k2dMaxPy = 1024, k2dClassicPy = 256;
+// Largest padded y extent of a 2-D grid (nz = 1) whose y transforms and tensor
+// multiply run as one pass of the z-pass kernels along y.  FP32 (32 served
+// 256x256x1 grids: 88 us against 103 us for two y passes and the product): up to
+// 1024 points, although a CTA holds one column from 258 butterflies of the widest
+// pass on, a quarter of a sector of each row (a stage of 512x512x1 40 against 47
+// us, 1000x500x1 99 against 134, 64x512x1 17 against 19; the few lengths of one
+// radix 2 and three or more odd ones above 685 points lose up to a seventh on
+// wide grids: 512x441x1 73 against 65 us).  FP64, where half a sector of each row
+// is twice the bytes and one column of three components is all a CTA holds: up to
+// 256 (a stage of 512x135x1 142 against 127 us, 512x343x1 784 against 558,
+// 1000x441x1 1287 against 974).
+template <typename T> constexpr int k2dMaxPy() { return sizeof(T) == 4 ? 1024 : 256; }
+constexpr int k2dClassicPy = 256;
 
 template <typename T>
 static void yzy(const DemagDims& d, typename Cplx<T>::type* S1, typename Cplx<T>::type* S2, const T* tens,
@@ -2318,7 +2326,7 @@ static void yzy(const DemagDims& d, typename Cplx<T>::type* S1, typename Cplx<T>
         }
         return;
     }
-    if (d.nz == 1 && d.LY > 1 && d.LY <= (d.classic ? k2dClassicPy : k2dMaxPy)) {
+    if (d.nz == 1 && d.LY > 1 && d.LY <= (d.classic ? k2dClassicPy : k2dMaxPy<T>())) {
         DemagDims d2 = d;
         d2.ny = 1; d2.nz = d.ny; d2.LY = 1; d2.LZ = d.LY; d2.yz_swap = 1;
         tm->begin(st, "p3_z_conv");
