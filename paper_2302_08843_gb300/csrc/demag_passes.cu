@@ -2294,8 +2294,8 @@ static void launch_p3_layers(const DemagDims& d, typename Cplx<T>::type* S2, con
 // Largest padded y extent of a 2-D grid (nz = 1) whose y transforms and tensor
 // multiply run as one pass of the z-pass kernels along y.  FP32 (32 served
 // 256x256x1 grids: 88 us against 103 us for two y passes and the product): up to
-// 1024 points, although a CTA holds one column from 258 butterflies of the widest
-// pass on, a quarter of a sector of each row (a stage of 512x512x1 40 against 47
+// 1024 points, although a CTA holds one column from 129 butterflies of the widest
+// pass on (513 of compiled lengths), a quarter of a sector of each row (a stage of 512x512x1 40 against 47
 // us, 1000x500x1 99 against 134, 64x512x1 17 against 19; the few lengths of one
 // radix 2 and three or more odd ones above 685 points lose up to a seventh on
 // wide grids: 512x441x1 73 against 65 us).  FP64, where half a sector of each row

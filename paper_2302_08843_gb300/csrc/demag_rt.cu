@@ -584,6 +584,11 @@ void line_launch(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, 
     cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
+// FP64 plans whose passes have unequal numbers of butterflies (line_warp_idle)
+template <typename T> bool line_idle(const LinePlan& pl) {
+    return sizeof(T) == 8 && std::any_of(pl.R, pl.R + pl.np, [&](int r) { return r != pl.rmin; });
+}
+
 // the kernel of a compiled length in place of the run-time one, if there is one
 template <typename... KArgs> bool line_ct_use(LineKind kind, int L, void (**kernel)(KArgs...)) {
     const void* k = line_ct_kernel0(kind, L);
@@ -645,7 +650,9 @@ bool launch_line_x_fwd(const DemagDims& d, const LineXIn<T>& in, typename Cplx<T
     if (d.nb > 65535 || !line_x_shape<T>(d.LX, line_x_pairs(d), d.nb, 1, kAnyCtas, &o)) return false;
     LineForward<T> f{in.m, in.Ms_cell, in.Ms, in.k, in.y, in.ca, in.dt_b, in.a, in.mask};
     auto k = o.threads <= 256 ? line_x_forward<T, 256, 0> : line_x_forward<T, kLineThreads, 0>;
-    if constexpr (sizeof(T) == 4) {
+    if constexpr (sizeof(T) == 8) {
+        if (line_idle<T>(o.pl)) k = o.threads <= 256 ? line_x_forward<T, 256, 0, true> : line_x_forward<T, kLineThreads, 0, true>;
+    } else {
         if (o.ct) line_ct_use(kLineXFwd, d.LX, &k);
     }
     line_launch(k, dim3((unsigned)o.ctas, d.nb), o.threads, o.smem, st, d, f, S1, o.pl, line_table<T>(o.pl), o.nt, o.lines);
@@ -657,7 +664,9 @@ bool launch_line_x_inv(const DemagDims& d, const typename Cplx<T>::type* S1, T* 
     LineXShape o;
     if (d.nb > 65535 || !line_x_shape<T>(d.LX, line_x_pairs(d), d.nb, 1, kAnyCtas, &o)) return false;
     auto k = o.threads <= 256 ? line_x_inverse<T, 256, 0> : line_x_inverse<T, kLineThreads, 0>;
-    if constexpr (sizeof(T) == 4) {
+    if constexpr (sizeof(T) == 8) {
+        if (line_idle<T>(o.pl)) k = o.threads <= 256 ? line_x_inverse<T, 256, 0, true> : line_x_inverse<T, kLineThreads, 0, true>;
+    } else {
         if (o.ct) line_ct_use(kLineXInv, d.LX, &k);
     }
     line_launch(k, dim3((unsigned)o.ctas, d.nb), o.threads, o.smem, st, d, S1, h, o.pl, line_table<T>(o.pl), o.nt, o.lines);
@@ -710,6 +719,9 @@ bool launch_line_y(const DemagDims& d, const typename Cplx<T>::type* in, typenam
     const long ncol = 3L * d.KX * d.nz;
     if (d.nb > 65535 || !line_shape<T>(d.LY, ncol, d.nb, 1, false, &o) || o.pl.np < 2) return false;
     auto k = o.threads <= 256 ? line_y<T, DIR, 256> : line_y<T, DIR, kLineThreads>;
+    if constexpr (sizeof(T) == 8) {
+        if (line_idle<T>(o.pl)) k = o.threads <= 256 ? line_y<T, DIR, 256, true> : line_y<T, DIR, kLineThreads, true>;
+    }
     line_launch(k, dim3((unsigned)o.ctas, d.nb), o.threads, o.smem, st, d, in, out, o.pl, line_table<T>(o.pl), o.lb,
                 (int)ncol);
     return true;
@@ -733,10 +745,27 @@ bool launch_line_conv(const DemagDims& d, typename Cplx<T>::type* S2, const T* t
              : o.threads > kSmall ? line_conv<T, kConvThree, kLineThreads, 0> : line_conv<T, kConvThree, kSmall, 0>;
     if constexpr (sizeof(T) == 4) {
         if (o.pl.np > 1 && line_ct_use(kLineConv, d.LZ, &k)) line_ct_shape(d.LZ, ncol, &o);
-    } else if (split) {
+    } else if (o.pl.np > 1) {
         const bool wide = std::any_of(o.pl.R, o.pl.R + o.pl.np, [](int r) { return r == 6 || r == 8; });
-        if (wide) k = o.threads <= 384 ? line_conv<T, kConvSplitWide, 384, 0> : line_conv<T, kConvSplitWide, 768, 0>;
-        else k = o.threads <= 384 ? line_conv<T, kConvSplit, 384, 0> : line_conv<T, kConvSplit, 768, 0>;
+        const bool idle = line_idle<T>(o.pl);
+        // components lie side by side in a CTA's threads, and whole warps are idle only
+        // where there are many of them (an RK4 step of 128x128x25: 4880 -> 4150 us)
+        while (split && idle && ((6 * M) << o.lb) <= 384 && (ncol >> (o.lb + 1)) >= 8 * 152) {
+            ++o.lb;
+            o.threads = (((3 * M) << o.lb) + 31) / 32 * 32;
+            o.smem *= 2;
+            o.ctas = (ncol + (1 << o.lb) - 1) >> o.lb;
+        }
+        const bool small = o.threads <= 384;
+        if (!split) {
+            if (idle) k = line_conv<T, kConvThree, kLineThreads, 0, true>;
+        } else if (idle) {
+            if (wide) k = small ? line_conv<T, kConvSplitWide, 384, 0, true> : line_conv<T, kConvSplitWide, 768, 0, true>;
+            else k = small ? line_conv<T, kConvSplit, 384, 0, true> : line_conv<T, kConvSplit, 768, 0, true>;
+        } else {
+            if (wide) k = small ? line_conv<T, kConvSplitWide, 384, 0> : line_conv<T, kConvSplitWide, 768, 0>;
+            else k = small ? line_conv<T, kConvSplit, 384, 0> : line_conv<T, kConvSplit, 768, 0>;
+        }
     }
     const dim3 grid((unsigned)o.ctas, d.nb);
     line_launch(k, grid, o.threads, o.smem, st, d, S2, tens, o.pl, line_table<T>(o.pl), o.lb, (int)ncol);

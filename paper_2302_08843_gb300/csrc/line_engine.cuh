@@ -332,6 +332,21 @@ __device__ __forceinline__ void line_start(typename Cplx<T>::type* s, int plane,
     __syncthreads();
 }
 
+// Whether a warp has no butterfly in a pass of radix R (IDLE kernels: FP64 plans of
+// unequal radices).  Plans of one radix 2 and odd ones have 2.5 to 3.5 times as
+// many threads as their odd passes have butterflies, and in FP64 idle threads'
+// instructions take the pipe from the others: with them an RK4 step of 64x32x245
+// (2 5 7 7) took 3307 us, without 1640.  FP32, bound by its exchanges, does without
+// the vote, and so do plans of equal radices (32x32x4 with the vote in its kernels:
+// 1342 against 1304 us).  Every warp is whole.
+template <bool IDLE> __device__ __forceinline__ bool line_warp_idle(const LinePlan& pl, int R, int b) {
+    return IDLE && !__any_sync(0xffffffffu, b * R < pl.L);
+}
+// the two barriers of a pass in place, for a warp that leaves it out
+__device__ __forceinline__ void line_pass_over() {
+    asm volatile("bar.sync 0;\n\tbar.sync 0;" ::: "memory");
+}
+
 // CALL with R_ = the radix (Wv: plans with a 6 or an 8 come here too)
 #define MM_LINE_RADIX(Wv, Rv, CALL)                                           \
     switch (Rv) {                                                         \
@@ -351,12 +366,13 @@ __device__ __forceinline__ void line_start(typename Cplx<T>::type* s, int plane,
         default: { constexpr int R_ = (Wv) ? 8 : 2; CALL; } break; \
     }
 
-template <typename T, int DIR, int NC, int SH, bool WIDE = true>
+template <typename T, int DIR, int NC, int SH, bool WIDE, bool IDLE>
 __device__ __forceinline__ void line_mid_any(typename Cplx<T>::type* s, int plane, int lb, int b, const LinePlan& pl,
                                              int i, const typename Cplx<T>::type* tw) {
     const int R = DIR < 0 ? pl.R[i] : pl.R[pl.np - 1 - i];
     const int Ns = DIR < 0 ? pl.Ns[i] : pl.Nsi[i];
     const unsigned mg = DIR < 0 ? pl.mg[i] : pl.mgi[i];
+    if (line_warp_idle<IDLE>(pl, R, b)) return line_pass_over();
     MM_LINE_RADIX(WIDE, R, (line_mid<T, DIR, R_, NC, SH>(s, plane, lb, b, pl.L, Ns, mg, tw)));
 }
 

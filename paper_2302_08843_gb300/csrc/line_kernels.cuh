@@ -129,7 +129,7 @@ __device__ __forceinline__ void line_f_first(typename Cplx<T>::type* s, int plan
 }
 
 // inverse of one line in shared memory (the first pass reads global memory); ends synchronised
-template <typename T, int NC, int LC>
+template <typename T, int NC, int LC, bool IDLE = false>
 __device__ __forceinline__ void line_inverse(const typename Cplx<T>::type* sa, const typename Cplx<T>::type* sb,
                                              long cs, typename Cplx<T>::type* s, int plane, int b,
                                              const LinePlan& pl, const typename Cplx<T>::type* tw) {
@@ -144,14 +144,15 @@ __device__ __forceinline__ void line_inverse(const typename Cplx<T>::type* sa, c
         const int np = pl.np, L = pl.L;
         MM_LINE_RADIX(true, pl.R[np - 1], (line_x_first<T, R_, NC>(sa, sb, cs, s, plane, b, L)));
         __syncthreads();
-        for (int i = 1; i < np - 1; ++i) line_mid_any<T, +1, NC, 4>(s, plane, 0, b, pl, i, tw);
+        for (int i = 1; i < np - 1; ++i) line_mid_any<T, +1, NC, 4, true, IDLE>(s, plane, 0, b, pl, i, tw);
+        if (line_warp_idle<IDLE>(pl, pl.R[0], b)) return line_pass_over();
         MM_LINE_RADIX_EVEN(true, pl.R[0], (line_x_last<T, R_, NC>(s, plane, b, L, pl.Nsi[np - 1], pl.mgi[np - 1], tw)));
     }
 }
 
 // forward of one line in shared memory and the r2c split into the two
 // spectrum rows; nt threads per line, this one b; called with the inputs in place and synchronised
-template <typename T, int NC, int LC>
+template <typename T, int NC, int LC, bool IDLE = false>
 __device__ __forceinline__ void line_forward(typename Cplx<T>::type* s, int plane, int b, int nt, int nx,
                                              const LinePlan& pl, const typename Cplx<T>::type* tw,
                                              typename Cplx<T>::type* sa, typename Cplx<T>::type* sb, long cs,
@@ -163,8 +164,9 @@ __device__ __forceinline__ void line_forward(typename Cplx<T>::type* s, int plan
         line_f_first<T, P.R[0], NC>(s, plane, b, LC, nx);
         line_mids_ct<T, -1, NC, 4, LC, 1, P.np>(s, plane, 0, b, tw);
     } else {
-        MM_LINE_RADIX_EVEN(true, pl.R[0], (line_f_first<T, R_, NC>(s, plane, b, L, nx)));
-        for (int i = 1; i < pl.np; ++i) line_mid_any<T, -1, NC, 4>(s, plane, 0, b, pl, i, tw);
+        if (line_warp_idle<IDLE>(pl, pl.R[0], b)) line_pass_over();
+        else MM_LINE_RADIX_EVEN(true, pl.R[0], (line_f_first<T, R_, NC>(s, plane, b, L, nx)));
+        for (int i = 1; i < pl.np; ++i) line_mid_any<T, -1, NC, 4, true, IDLE>(s, plane, 0, b, pl, i, tw);
     }
     if (!on) return;
     const T half = (T)0.5;
@@ -207,7 +209,7 @@ template <typename T> struct LineForward {
     const int* mask;      // grids to work on, or null
 };
 
-template <typename T, int MAXT, int LC>
+template <typename T, int MAXT, int LC, bool IDLE = false>
 __global__ void __launch_bounds__(MAXT)
 line_x_forward(DemagDims d, LineForward<T> f, typename Cplx<T>::type* __restrict__ S1,
                const __grid_constant__ LinePlan pl, const typename Cplx<T>::type* __restrict__ tw, int nt, int lines) {
@@ -271,11 +273,11 @@ line_x_forward(DemagDims d, LineForward<T> f, typename Cplx<T>::type* __restrict
     }
     __syncthreads();
     C* sa = S1 + (off + r.ra) * d.KXS;
-    line_forward<T, NC, LC>(s, plane, t.b, nt, nx, pl, tw, sa, sa + d.KXS, rows * d.KXS,
+    line_forward<T, NC, LC, IDLE>(s, plane, t.b, nt, nx, pl, tw, sa, sa + d.KXS, rows * d.KXS,
                         r.on && t.in, r.two);
 }
 
-template <typename T, int MAXT, int LC>
+template <typename T, int MAXT, int LC, bool IDLE = false>
 __global__ void __launch_bounds__(MAXT)
 line_x_inverse(DemagDims d, const typename Cplx<T>::type* __restrict__ S1, T* __restrict__ h,
                const __grid_constant__ LinePlan pl, const typename Cplx<T>::type* __restrict__ tw, int nt, int lines) {
@@ -293,7 +295,7 @@ line_x_inverse(DemagDims d, const typename Cplx<T>::type* __restrict__ S1, T* __
     C* s = reinterpret_cast<C*>(smraw) + (size_t)t.l * NC * plane;
     const C* sa = S1 + (off + r.ra) * d.KXS;
     grid_dep_wait();
-    line_inverse<T, NC, LC>(sa, r.two ? sa + d.KXS : sa, rows * d.KXS, s, plane, t.b, pl, tw);
+    line_inverse<T, NC, LC, IDLE>(sa, r.two ? sa + d.KXS : sa, rows * d.KXS, s, plane, t.b, pl, tw);
     if (!r.on || !t.in) return;
     for (int x = t.b; x < nx; x += nt) {
 #pragma unroll
@@ -850,7 +852,7 @@ __device__ __forceinline__ void line_product_one(typename Cplx<T>::type* g, long
 // kConvSplitWide, that with radices 6 and 8 too, whose registers cost the plans
 // without them 1 to 3 % (film of 512x128x1: 47.5 -> 49.0 us).
 enum { kConvOne, kConvThree, kConvSplit, kConvSplitWide };
-template <typename T, int FORM, int MAXT, int LC>
+template <typename T, int FORM, int MAXT, int LC, bool IDLE = false>
 __global__ void __launch_bounds__(MAXT, FORM >= kConvSplit ? (MAXT <= 384 ? 2 : 1) : FORM == kConvOne ? 2 : LC > 0 && MAXT == kLineThreads32 ? 2 : line_blocks<T, MAXT>())
 line_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restrict__ tens,
           const __grid_constant__ LinePlan pl, const typename Cplx<T>::type* __restrict__ tw, int lb, int ncol) {
@@ -913,10 +915,11 @@ line_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restr
         const int np = pl.np;
         MM_LINE_RADIX_EVEN(kWide, pl.R[0], (line_first<T, -1, R_, true, 1>(g, zs, 0, d.nz, s, 0, lb, b, L)));
         __syncthreads();
-        for (int i = 1; i < np; ++i) line_mid_any<T, -1, 1, 3, kWide>(s, 0, lb, b, pl, i, tw);
+        for (int i = 1; i < np; ++i) line_mid_any<T, -1, 1, 3, kWide, IDLE>(s, 0, lb, b, pl, i, tw);
         product();
-        MM_LINE_RADIX(kWide, pl.R[np - 1], (line_start<T, +1, R_, 1, 3>(s, 0, lb, b, L)));
-        for (int i = 1; i < np - 1; ++i) line_mid_any<T, +1, 1, 3, kWide>(s, 0, lb, b, pl, i, tw);
+        if (line_warp_idle<IDLE>(pl, pl.R[np - 1], b)) line_pass_over();
+        else MM_LINE_RADIX(kWide, pl.R[np - 1], (line_start<T, +1, R_, 1, 3>(s, 0, lb, b, L)));
+        for (int i = 1; i < np - 1; ++i) line_mid_any<T, +1, 1, 3, kWide, IDLE>(s, 0, lb, b, pl, i, tw);
         MM_LINE_RADIX_EVEN(kWide, pl.R[0], (line_last<T, +1, R_, true, 1>(s, 0, lb, b, L, pl.Nsi[np - 1], pl.mgi[np - 1],
                                                                       tw, g, zs, 0, d.nz, valid)));
         return;
@@ -949,10 +952,11 @@ line_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restr
             MM_LINE_RADIX_EVEN(true, pl.R[0], (line_first<T, -1, R_, true, 3>(g, zs, cs, d.nz, s, plane, lb, b, L)));
             __syncthreads();
             const int np = pl.np;
-            for (int i = 1; i < np - 1; ++i) line_mid_any<T, -1, 3, 3>(s, plane, lb, b, pl, i, tw);
-            MM_LINE_RADIX(true, pl.R[np - 1], (line_product<T, R_>(s, plane, lb, b, L, pl.Ns[np - 1], pl.mg[np - 1], tw, tp,
+            for (int i = 1; i < np - 1; ++i) line_mid_any<T, -1, 3, 3, true, IDLE>(s, plane, lb, b, pl, i, tw);
+            if (line_warp_idle<IDLE>(pl, pl.R[np - 1], b)) line_pass_over();
+            else MM_LINE_RADIX(true, pl.R[np - 1], (line_product<T, R_>(s, plane, lb, b, L, pl.Ns[np - 1], pl.mg[np - 1], tw, tp,
                                                                 tz, tc, up, d.yz_swap)));
-            for (int i = 1; i < np - 1; ++i) line_mid_any<T, +1, 3, 3>(s, plane, lb, b, pl, i, tw);
+            for (int i = 1; i < np - 1; ++i) line_mid_any<T, +1, 3, 3, true, IDLE>(s, plane, lb, b, pl, i, tw);
             MM_LINE_RADIX_EVEN(true, pl.R[0], (line_last<T, +1, R_, true, 3>(s, plane, lb, b, L, pl.Nsi[np - 1],
                                                                           pl.mgi[np - 1], tw, g, zs, cs, d.nz, valid)));
         }
@@ -963,7 +967,7 @@ line_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restr
 // DIR = +1: S2 -> S1, keep y < ny.  Columns kx-fastest over component and z,
 // kx <= Px/2, a thread per butterfly of one component (three per thread: 11.3 and
 // 9.6 against 8.7 and 8.8 us on 140-point lines of 100x65x27).
-template <typename T, int DIR, int MAXT>
+template <typename T, int DIR, int MAXT, bool IDLE = false>
 __global__ void __launch_bounds__(MAXT)
 line_y(DemagDims d, const typename Cplx<T>::type* __restrict__ in, typename Cplx<T>::type* __restrict__ out,
        const __grid_constant__ LinePlan pl, const typename Cplx<T>::type* __restrict__ tw, int lb, int ncol) {
@@ -987,7 +991,7 @@ line_y(DemagDims d, const typename Cplx<T>::type* __restrict__ in, typename Cplx
         MM_LINE_RADIX(true, pl.R[np - 1], (line_first<T, +1, R_, false, 1>(gi, d.KXS, 0, L, s, 0, lb, b, L)));
     }
     __syncthreads();
-    for (int i = 1; i < np - 1; ++i) line_mid_any<T, DIR, 1, 3>(s, 0, lb, b, pl, i, tw);
+    for (int i = 1; i < np - 1; ++i) line_mid_any<T, DIR, 1, 3, true, IDLE>(s, 0, lb, b, pl, i, tw);
     if constexpr (DIR < 0) {
         MM_LINE_RADIX(true, pl.R[np - 1], (line_last<T, -1, R_, false, 1>(s, 0, lb, b, L, pl.Ns[np - 1], pl.mg[np - 1], tw, go,
                                                                        d.KXS, 0, L, valid)));

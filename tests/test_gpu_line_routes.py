@@ -1,7 +1,11 @@
 """Routes of the z and y passes chosen by size, on both sides of their lines:
-FP64 2-D grids past the longest single pass."""
+FP64 plans of unequal radices, whose idle warps leave passes out, along every
+axis and with one, two and four columns per CTA; and FP64 2-D grids past the
+longest single pass.  Fields against the oracle."""
 import numpy as np
 import pytest
+
+from gpu_util import rel, to_host
 
 pytestmark = pytest.mark.gpu
 
@@ -11,6 +15,30 @@ D = (2e-9, 3e-9, 2.5e-9)
 def _m(n, seed=0):
     m = np.random.default_rng(seed).normal(size=(3,) + n[::-1])
     return m / np.linalg.norm(m, axis=0)
+
+
+def _field(n, precision, m, p):
+    from paper_2302_08843_gb300.binding import State
+    s = State(n, D, precision)
+    s.set_material(Ms=8e5, A=0.0, alpha=0.1)
+    s.demag_setup(p)
+    h = to_host(s.heff(m=m))
+    s.close()
+    return h
+
+
+# 490, 686 and 882 points (two, three and three idle passes) along z, y and x; 50, 70
+# and 98 points with few lines and with enough for four columns per CTA
+@pytest.mark.parametrize("n", [(4, 3, 245), (3, 5, 343), (5, 4, 441), (4, 245, 2), (9, 343, 1), (245, 6, 2), (441, 3, 2),
+                               (60, 40, 25), (70, 30, 35), (9, 5, 25), (62, 28, 49)])
+def test_fp64_plans_of_unequal_radices(n):
+    from oracle.demag import demag_fft, magnetization, rounding_sensitivity
+    from oracle.newell import demag_tensor
+    from paper_2302_08843_gb300.workloads import from_soa
+    m = _m(n)
+    M = magnetization(from_soa(m), 8e5)
+    tol = max(1e-10, rounding_sensitivity(n, D, 5, M))
+    assert rel(from_soa(_field(n, "fp64", m, 5)), demag_fft(demag_tensor(n, D, 5), M)) < tol
 
 
 @pytest.mark.parametrize("ny,one", [(128, True), (135, False), (343, False)])
