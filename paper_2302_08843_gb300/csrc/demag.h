@@ -57,6 +57,8 @@ struct DemagDims {
     // (gradients over 12 grids and 5 seeds: 3.3e-7 from FP64, and 3.4e-7 with the
     // replay on the step's own passes, at 5295 instead of 4455 us on 128x128x1).
     int classic = 0;
+    // the z pass may let the next kernel be placed while it runs (line_conv; set by yzy)
+    int early = 0;
     // non-equidistant layers (Sec. 4.4): no transform along z; the nz layers
     // are coupled densely at every lateral wave number (p3_layers).  lh holds
     // the nz thicknesses in the real type of the passes.

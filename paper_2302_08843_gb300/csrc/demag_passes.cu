@@ -2070,9 +2070,11 @@ template <typename T, int L> static void launch_p3(const DemagDims& d, typename 
     // 113 and 180; 256 points, 33 tiles 59 and 115 against 65 and 125, 64 tiles 92 and
     // 142 against 86 and 151; 32 points, 640 tiles 81 and 147 against 88 and 155, 2304
     // tiles 16.5 against 14.6 us a pass; lines up to 16 points, one thread each,
-    // are level up to 8704 tiles.  The line engine takes all others, FP64 (64-point
-    // lines of 128x128x32 519 -> 393 us, 256 points of a 512x128x1 film 97 -> 44) and
-    // batches (16 grids of 100x100x8 63 -> 34 us).
+    // are level up to 8704 tiles, but 16 points with y lines of 32 and 64 stay with TMA
+    // (256x16x8 101 against 94 us, 16x16x8 70 against 62, 64x32x8 75 against 71).  The
+    // line engine takes all others, FP64 (64-point lines of 128x128x32 519 -> 393 us,
+    // 256 points of a 512x128x1 film 97 -> 44) and batches (16 grids of 100x100x8 63 ->
+    // 34 us).
     constexpr int kTmaTiles = L <= 16 ? 8192 : L < 64 ? 1024 : L < 128 ? 560 : L < 256 ? 144 : 48;
     if constexpr (sizeof(T) == 4 && L <= 256 && Fft<T, L, -1, (L > 1)>::NR <= 20) {
         if constexpr (z_two_r1<L>() > 0) {
@@ -2080,10 +2082,19 @@ template <typename T, int L> static void launch_p3(const DemagDims& d, typename 
         }
         if constexpr (tma_len<L>()) {
             const long tiles = (long)((d.KX + 15) / 16) * d.LY;
-            if (d.nb == 1 && (d.classic || tiles >= kTmaTiles) && launch_p3_tma<L>(d, S2, tens, st)) return;
+            const bool short_y = L == 16 && (d.LY == 32 || d.LY == 64);
+            if (d.nb == 1 && (d.classic || short_y || tiles >= kTmaTiles) && launch_p3_tma<L>(d, S2, tens, st)) return;
         }
     }
-    if (!d.classic && launch_line_conv<T>(d, S2, tens, st)) return;
+    // FP32 lines of 1024 and 2048 points: a CTA of the line engine holds two columns
+    // and one, a part of a sector of each row, and pays where there are few.  An RK4
+    // step with the line engine and with the compiled pass below: 1024 points, 2112
+    // columns 545 and 608 us, 4160 columns 918 and 835; 2048 points, 1056 columns 880
+    // and 640.  (Of single states only: the passes of a batch must not depend on how
+    // many grids it launches.)
+    const bool part_rows = sizeof(T) == 4 && d.err && (L == 1024 || L == 2048) &&
+                           (long)d.KX * d.LY > (L == 1024 ? 3072 : 512);
+    if (!d.classic && !part_rows && launch_line_conv<T>(d, S2, tens, st)) return;
     constexpr int B = b_p3<T, L>(), G = g_p3<T, L>();
     using C = typename Cplx<T>::type;
     const int kyi = 2 * (d.LY / 2 + 1);
@@ -2341,7 +2352,18 @@ static void yzy(const DemagDims& d, typename Cplx<T>::type* S1, typename Cplx<T>
         tm->end(st);
     }
     tm->begin(st, "p3_z_conv");
-    MM_DISPATCH_RT(d.LZ, (launch_p3<T, L_>(d, S2e, tens, st)), (launch_rt_z<T>(d, S2e, tens, st)));
+    DemagDims dz = d;
+    if constexpr (sizeof(T) == 4) {
+        // The TMA y pass that follows has CTAs of 4 to 16 threads on lines up to 64
+        // points: placed while the z pass runs they are spared a start of 4 to 8 us (an
+        // RK4 step of 256x8x2 82 -> 56 us, 256x16x4 98 -> 66, 256x16x2 92 -> 63, 256x16x16
+        // 120 -> 95, 256x32x2 95 -> 65, 400x32x4 130 -> 102).  CTAs of longer lines, or of
+        // 64 points beside long z or x lines, crowd on the SMs that the z pass leaves
+        // first (64x32x32 81 -> 97 us, 768x32x2 97 -> 106, 512x64x2 77 -> 83).
+        const bool tma_y = d.err && d.nb == 1 && is_pow2(d.LY) && d.LY >= 16;
+        dz.early = tma_y && (d.LY <= 32 || (d.LY == 64 && d.LZ <= 16 && d.LX < 1024));
+    }
+    MM_DISPATCH_RT(d.LZ, (launch_p3<T, L_>(dz, S2e, tens, st)), (launch_rt_z<T>(dz, S2e, tens, st)));
     tm->end(st);
     if (d.LY > 1) {
         tm->begin(st, "p4_y_inverse");

@@ -563,7 +563,8 @@ template <typename T> bool line_shape(int L, long ncol, int nb, int nc, bool con
 }
 
 // Launched with programmatic stream serialisation, so that a kernel's set-up
-// overlaps the end of the previous one; none triggers the next one earlier.  CTAs
+// overlaps the end of the previous one; none but line_conv before a short y pass
+// (DemagDims::early) triggers the next one earlier.  CTAs
 // placed while the previous grid still runs crowd on the SMs that finish first:
 // with a trigger at the start of launches of at most 304 CTAs an RK4 step of
 // 512x128x1 in FP32 took 92 us instead of 59, 300x128x1 74 instead of 54, four FP64

@@ -925,6 +925,7 @@ line_conv(DemagDims d, typename Cplx<T>::type* __restrict__ S2, const T* __restr
         return;
     }
     grid_dep_wait();
+    if (d.early) grid_dep_launch();
     if constexpr (FORM == kConvOne) {
         if (!valid) return;
         switch (L) {

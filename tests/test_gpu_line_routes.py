@@ -1,11 +1,15 @@
 """Routes of the z and y passes chosen by size, on both sides of their lines:
 FP64 plans of unequal radices, whose idle warps leave passes out, along every
-axis and with one, two and four columns per CTA; and FP64 2-D grids past the
-longest single pass.  Fields against the oracle."""
+axis and with one, two and four columns per CTA; FP32 lines of 1024 and 2048
+points with few and with many columns; z passes that let a short y pass be
+placed while they run; and FP64 2-D grids past the longest single pass.
+Fields against the oracle where it is quick, else FP32 against FP64 fields with
+the FP32 bound of the demag tests; RK4 runs against FP64 ones with that bound
+for each step, and bit for bit against themselves."""
 import numpy as np
 import pytest
 
-from gpu_util import rel, to_host
+from gpu_util import FP32_TOL, rel, to_host
 
 pytestmark = pytest.mark.gpu
 
@@ -39,6 +43,31 @@ def test_fp64_plans_of_unequal_radices(n):
     M = magnetization(from_soa(m), 8e5)
     tol = max(1e-10, rounding_sensitivity(n, D, 5, M))
     assert rel(from_soa(_field(n, "fp64", m, 5)), demag_fft(demag_tensor(n, D, 5), M)) < tol
+
+
+@pytest.mark.parametrize("n", [(33, 40, 512), (33, 50, 512), (15, 16, 1024), (17, 20, 1024)])
+def test_fp32_long_z_lines(n):
+    m = _m(n)
+    assert rel(_field(n, "fp32", m, 1), _field(n, "fp64", m, 1)) < FP32_TOL
+
+
+@pytest.mark.parametrize("n", [(256, 8, 2), (256, 16, 4), (60, 16, 16), (400, 32, 4), (70, 32, 20), (256, 16, 8)])
+def test_short_y_lines_after_the_z_pass(n):
+    from paper_2302_08843_gb300.binding import State
+    out = []
+    steps = 12
+    for precision in ("fp64", "fp32", "fp32"):
+        s = State(n, D, precision)
+        s.set_material(Ms=8e5, A=1.3e-11, alpha=0.5, Ku1=1e5, ku_axis=(0.0, 0.6, 0.8))
+        s.demag_setup(2)
+        s.set_m(_m(n, 1))
+        t = 0.0
+        for _ in range(steps):
+            t, _ = s.step(2e-14, t, "rk4")
+        out.append(to_host(s.get_m()))
+        s.close()
+    assert rel(out[1], out[0]) < steps * FP32_TOL
+    assert np.array_equal(out[1], out[2])
 
 
 @pytest.mark.parametrize("ny,one", [(128, True), (135, False), (343, False)])
