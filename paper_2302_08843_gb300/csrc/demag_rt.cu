@@ -526,10 +526,13 @@ struct LineShape {
 // 1490 -> 1010 and 1486 -> 1056 along y, 988 -> 649 and 953 -> 631 along x).  An
 // FP64 grid that would leave quarter SMs idle takes radix 2; the grids of a batch
 // do not count, so that a grid's rounding does not depend on the others.
-template <typename T> LinePlan line_radices(int L, long lines, bool one) {
+bool line_few(int L, long lines) {
     constexpr int kSms = 152;
+    return L > 2 && lines * (L / 4) < kSms * 128L;
+}
+template <typename T> LinePlan line_radices(int L, long lines, bool one) {
     if (sizeof(T) == 4) return host_plan(L, 8, one);
-    if (L > 2 && lines * (L / 4) < kSms * 128L) return host_plan(L, 2, one);
+    if (line_few(L, lines)) return host_plan(L, 2, one);
     const LinePlan p = host_plan(L, 4, one);
     if (one || p.rmin != 2) return p;
     const LinePlan wide = host_plan(L, 8, one);
@@ -585,9 +588,16 @@ void line_launch(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, 
     cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
-// FP64 plans whose passes have unequal numbers of butterflies (line_warp_idle)
-template <typename T> bool line_idle(const LinePlan& pl) {
-    return sizeof(T) == 8 && std::any_of(pl.R, pl.R + pl.np, [&](int r) { return r != pl.rmin; });
+// FP64 plans whose passes have unequal numbers of butterflies (line_warp_idle);
+// lines: of all grids, as no result depends on it.
+// Where few lines leave the pipe idle anyway the vote pays from a third of the
+// threads without work on: an RK4 step of 16x16x49 (98 points, 52 % busy) 367 ->
+// 219 us, five of a 20x45x4 stack (40 and 90 points, 85 and 68 %) 979 -> 992.
+template <typename T> bool line_idle(const LinePlan& pl, long lines) {
+    if (sizeof(T) == 4) return false;
+    double busy = 0;
+    for (int i = 0; i < pl.np; ++i) busy += (double)pl.rmin / pl.R[i] / pl.np;
+    return busy < (line_few(pl.L, lines) ? 0.65 : 0.999);
 }
 
 // the kernel of a compiled length in place of the run-time one, if there is one
@@ -652,7 +662,8 @@ bool launch_line_x_fwd(const DemagDims& d, const LineXIn<T>& in, typename Cplx<T
     LineForward<T> f{in.m, in.Ms_cell, in.Ms, in.k, in.y, in.ca, in.dt_b, in.a, in.mask};
     auto k = o.threads <= 256 ? line_x_forward<T, 256, 0> : line_x_forward<T, kLineThreads, 0>;
     if constexpr (sizeof(T) == 8) {
-        if (line_idle<T>(o.pl)) k = o.threads <= 256 ? line_x_forward<T, 256, 0, true> : line_x_forward<T, kLineThreads, 0, true>;
+        if (line_idle<T>(o.pl, line_x_pairs(d) * d.nb))
+            k = o.threads <= 256 ? line_x_forward<T, 256, 0, true> : line_x_forward<T, kLineThreads, 0, true>;
     } else {
         if (o.ct) line_ct_use(kLineXFwd, d.LX, &k);
     }
@@ -666,7 +677,8 @@ bool launch_line_x_inv(const DemagDims& d, const typename Cplx<T>::type* S1, T* 
     if (d.nb > 65535 || !line_x_shape<T>(d.LX, line_x_pairs(d), d.nb, 1, kAnyCtas, &o)) return false;
     auto k = o.threads <= 256 ? line_x_inverse<T, 256, 0> : line_x_inverse<T, kLineThreads, 0>;
     if constexpr (sizeof(T) == 8) {
-        if (line_idle<T>(o.pl)) k = o.threads <= 256 ? line_x_inverse<T, 256, 0, true> : line_x_inverse<T, kLineThreads, 0, true>;
+        if (line_idle<T>(o.pl, line_x_pairs(d) * d.nb))
+            k = o.threads <= 256 ? line_x_inverse<T, 256, 0, true> : line_x_inverse<T, kLineThreads, 0, true>;
     } else {
         if (o.ct) line_ct_use(kLineXInv, d.LX, &k);
     }
@@ -721,7 +733,7 @@ bool launch_line_y(const DemagDims& d, const typename Cplx<T>::type* in, typenam
     if (d.nb > 65535 || !line_shape<T>(d.LY, ncol, d.nb, 1, false, &o) || o.pl.np < 2) return false;
     auto k = o.threads <= 256 ? line_y<T, DIR, 256> : line_y<T, DIR, kLineThreads>;
     if constexpr (sizeof(T) == 8) {
-        if (line_idle<T>(o.pl)) k = o.threads <= 256 ? line_y<T, DIR, 256, true> : line_y<T, DIR, kLineThreads, true>;
+        if (line_idle<T>(o.pl, ncol * d.nb)) k = o.threads <= 256 ? line_y<T, DIR, 256, true> : line_y<T, DIR, kLineThreads, true>;
     }
     line_launch(k, dim3((unsigned)o.ctas, d.nb), o.threads, o.smem, st, d, in, out, o.pl, line_table<T>(o.pl), o.lb,
                 (int)ncol);
@@ -748,7 +760,7 @@ bool launch_line_conv(const DemagDims& d, typename Cplx<T>::type* S2, const T* t
         if (o.pl.np > 1 && line_ct_use(kLineConv, d.LZ, &k)) line_ct_shape(d.LZ, ncol, &o);
     } else if (o.pl.np > 1) {
         const bool wide = std::any_of(o.pl.R, o.pl.R + o.pl.np, [](int r) { return r == 6 || r == 8; });
-        const bool idle = line_idle<T>(o.pl);
+        const bool idle = line_idle<T>(o.pl, ncol * d.nb);
         // components lie side by side in a CTA's threads, and whole warps are idle only
         // where there are many of them (an RK4 step of 128x128x25: 4880 -> 4150 us)
         while (split && idle && ((6 * M) << o.lb) <= 384 && (ncol >> (o.lb + 1)) >= 8 * 152) {
