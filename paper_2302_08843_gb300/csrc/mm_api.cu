@@ -878,7 +878,7 @@ struct mm_batch {
     void* D_d = nullptr;
     void* pc_d = nullptr;
     int* kind_d = nullptr;
-    std::vector<char> special;     // slots with DMI or Ms = 0: the general variant of the fused stage
+    std::vector<char> special;     // slots of the fused stage's general variant: bit 0 Ms = 0, bit 1 DMI
     std::vector<char> unstarted;   // loaded and not yet in an mm_batch_begin
     // per-slot controller state, on the device: status, steps, fresh, dt, t, torque
     int* ctl_i = nullptr;        // [3][cap] ints
@@ -1658,7 +1658,7 @@ mm_status mm_batch_set_slot(mm_batch* b, int slot, double Ms, double A, double a
     MM_TRY(batch_slot(b, slot, kSlotLoad, Ms, A, alpha, 0.0, 1.0, 0, dt0 > 0 ? dt0 : 1e-13));
     MM_CUDA(cudaStreamSynchronize(b->st));   // the caller may reuse m0
     b->status[slot] = 1;
-    b->special[slot] = Ms == 0.0 || (float)Ms == 0.f;
+    b->special[slot] = Ms == 0.0 || (float)Ms == 0.f ? 1 : 0;
     b->unstarted[slot] = 1;
     b->fresh_any = true;
     return MM_OK;
@@ -1675,7 +1675,7 @@ mm_status mm_batch_set_slot_terms(mm_batch* b, int slot, int dmi_kind, double D,
     const int kind = D != 0.0 ? dmi_kind : MM_DMI_NONE;
     MM_TRY(batch_slot(b, slot, kSlotTerms, 0.0, 0.0, 0.0, D, precession ? 1.0 : 0.0, kind, 0.0));
     MM_CUDA(cudaStreamSynchronize(b->st));
-    if (kind != MM_DMI_NONE) b->special[slot] = 1;
+    b->special[slot] = (char)((b->special[slot] & 1) | (kind != MM_DMI_NONE ? 2 : 0));
     return MM_OK;
 }
 
