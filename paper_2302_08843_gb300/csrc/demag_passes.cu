@@ -27,6 +27,7 @@
 #include "demag.h"
 #include "fft_engine.cuh"
 #include "fft_pair.cuh"
+#include "line_engine.cuh"
 #include "tma.cuh"
 
 namespace mm {
@@ -2113,6 +2114,8 @@ template <typename T, int L> static void launch_p3(const DemagDims& d, typename 
         auto k = p3_z_conv<T, L, B, G>;
         set_smem(k, sm);
         k<<<grid, B * G * tpl_of<T, L>(), sm, st>>>(d, S2, tens);
+    } else {
+        static_assert(L < 8 || line_holds_fp64(L), "the line engine has to take every line of this length");
     }
 }
 
@@ -2130,6 +2133,7 @@ template <typename T, int L, int DIR> static void launch_y(const DemagDims& d, c
         if (launch_line_y<T, DIR>(d, in, out, st)) return;
     }
     if constexpr (sizeof(T) == 4 || L < 16 || L >= 2048) launch_py<T, L, DIR>(d, in, out, st);
+    else static_assert(line_holds_fp64(L), "the line engine has to take every line of this length");
 }
 
 // FP64 x lines of 2048 points on stay on the compiled passes, whose four radix-8
@@ -2151,6 +2155,7 @@ template <typename T, int L> static void launch_x_fwd(const DemagDims& d, const 
     if (line_x_use<T, L>(d) && launch_line_x_fwd<T>(d, in, S1, st)) return;
     // lines too short or too long for the engine, and the classic FP32 passes
     if constexpr (sizeof(T) == 4 || L < 16 || L >= 2048) launch_p1<T, L>(d, m, Ms_cell, Ms, S1, st);
+    else static_assert(line_holds_fp64(L), "the line engine has to take every line of this length");
 }
 
 template <typename T, int L> static void launch_x_inv(const DemagDims& d, const typename Cplx<T>::type* S1, T* h,
@@ -2160,6 +2165,7 @@ template <typename T, int L> static void launch_x_inv(const DemagDims& d, const 
     }
     if (line_x_use<T, L>(d) && launch_line_x_inv<T>(d, S1, h, st)) return;
     if constexpr (sizeof(T) == 4 || L < 16 || L >= 2048) launch_p5<T, L>(d, S1, h, st);
+    else static_assert(line_holds_fp64(L), "the line engine has to take every line of this length");
 }
 
 // fused K5 launcher (see k5_fused): false if the shape or material does not qualify

@@ -101,6 +101,10 @@ constexpr LinePlan line_plan(int L, int rmax) {
     }
     return p;
 }
+// threads of a CTA at most.  FP32 passes wait on memory: three CTAs of 256
+// threads per SM (85 registers); the 512-thread variant takes the lines with
+// more butterflies.
+constexpr int kLineThreads = 512, kLineThreads32 = 256;
 // plan of an FP32 compiled length
 template <typename T> __host__ __device__ constexpr LinePlan line_ct(int L) { return line_plan(L, 8); }
 // FP64 z lines whose three components fit a CTA side by side take a thread per
@@ -134,7 +138,20 @@ __device__ __forceinline__ int line_mod(int b, int Ns, unsigned mg) {
 // (a warp reads eight elements of four lines), every sixteen where one line
 // does (a half warp reads sixteen elements).
 template <int SH> __host__ __device__ __forceinline__ int line_place(int e) { return e + (e >> SH); }
-__host__ __device__ __forceinline__ int line_len(int L) { return L + (L >> 3) + 1; }
+__host__ __device__ __forceinline__ constexpr int line_len(int L) { return L + (L >> 3) + 1; }
+
+// Whether a CTA holds an FP64 line of L points with every plan the launches may
+// choose (radices up to 2, 4 or 8), alone for the y and x passes and with its three
+// components for the z pass: the lengths whose launches have nothing else to turn
+// to.  (The one other reason to refuse, more than 65535 grids, is 16 times the
+// largest batch.)
+constexpr bool line_holds_fp64(int L) {
+    for (int rmax = 2; rmax <= 8; rmax *= 2) {
+        const LinePlan p = line_plan(L, rmax);
+        if (p.np < (rmax < 8 ? 2 : 1) || L / p.rmin > kLineThreads) return false;
+    }
+    return 3 * 2 * sizeof(double) * line_len(L) <= 160 * 1024;
+}
 
 // -v or v; FP64 on the integer side (FP64 instructions are what an FP64 pass is made of)
 __device__ __forceinline__ float line_flip(float v, bool neg) { return neg ? -v : v; }

@@ -22,10 +22,6 @@
 
 namespace mm {
 
-// threads of a CTA at most.  FP32 passes wait on memory: three CTAs of 256
-// threads per SM (85 registers); the 512-thread variant takes the lines with
-// more butterflies.
-constexpr int kLineThreads = 512, kLineThreads32 = 256;
 template <typename T, int MAXT> constexpr int line_blocks() { return sizeof(T) == 4 && MAXT == kLineThreads32 ? 3 : 1; }
 
 
