@@ -66,6 +66,10 @@ struct DemagDims {
     const void* lh = nullptr;
 };
 
+// SMs of the chip this library is written for; decides shapes of launches and the
+// FP64 radices of grids with few lines
+constexpr int kSms = 152;
+
 // most layers a non-equidistant stack may have (shared memory of p3_layers)
 constexpr int kMaxLayers = 64;
 

@@ -2265,8 +2265,6 @@ template <int L> static bool launch_k5(const DemagDims& d, float2* S1, const Sta
         MM_DISPATCH_L(Lv, CALL);         \
     }
 
-// P2 .. P4: S1 -> S1 through the tensor multiply.  A 2-D grid (nz = 1, Py <= 256)
-// runs the z-pass kernel along y in place on S1 instead (one pass, no S2).
 template <typename T>
 static bool launch_p3_layers_tma(const DemagDims& d, typename Cplx<T>::type* S2, const T* tens, cudaStream_t st) {
     using C = typename Cplx<T>::type;
@@ -2322,6 +2320,7 @@ static void launch_p3_layers(const DemagDims& d, typename Cplx<T>::type* S2, con
 template <typename T> constexpr int k2dMaxPy() { return sizeof(T) == 4 ? 1024 : 256; }
 constexpr int k2dClassicPy = 256;
 
+// P2 .. P4: S1 -> S1 through the tensor multiply
 template <typename T>
 static void yzy(const DemagDims& d, typename Cplx<T>::type* S1, typename Cplx<T>::type* S2, const T* tens,
                 cudaStream_t st, KernelTimer* tm) {

@@ -527,7 +527,6 @@ struct LineShape {
 // FP64 grid that would leave quarter SMs idle takes radix 2; the grids of a batch
 // do not count, so that a grid's rounding does not depend on the others.
 bool line_few(int L, long lines) {
-    constexpr int kSms = 152;
     return L > 2 && lines * (L / 4) < kSms * 128L;
 }
 template <typename T> LinePlan line_radices(int L, long lines, bool one) {
@@ -542,7 +541,6 @@ template <typename T> LinePlan line_radices(int L, long lines, bool one) {
 // As many columns per CTA (at least one 32-byte sector of each row) as leave two
 // CTAs for every SM.
 template <typename T> bool line_shape(int L, long ncol, int nb, int nc, bool conv, LineShape* o) {
-    constexpr int kSms = 152;
     constexpr int full = 128 / (2 * sizeof(T)), sector = 32 / (2 * sizeof(T));
     // FP32 z lines of up to 16 points stay in one thread's registers
     const bool one = conv && (L <= 2 || L == 4 || (sizeof(T) == 4 && (L == 6 || L == 8 || L == 12 || L == 16)));
@@ -629,7 +627,6 @@ struct LineXShape {
 // other grids); never more CTAs than max_ctas for each grid.  nc: lines of a row
 // pair (3: the fused stage's components).  FP64 radices as in line_shape.
 template <typename T> bool line_x_shape(int L, long pairs, int nb, int nc, long max_ctas, LineXShape* o) {
-    constexpr int kSms = 152;
     o->pl = line_radices<T>(L, pairs, false);
     if (o->pl.np < 2) return false;
     o->nt = L / o->pl.rmin;
@@ -749,7 +746,7 @@ bool launch_line_conv(const DemagDims& d, typename Cplx<T>::type* S2, const T* t
     const int M = o.pl.np ? d.LZ / o.pl.rmin : 0;
     const bool split = o.pl.np > 1 && line_split<T>(M);
     if (split) {
-        o.lb = line_split_lb<T>(M);
+        o.lb = line_split_lb(M);
         o.threads = (((3 * M) << o.lb) + 31) / 32 * 32;
         o.smem = (size_t)3 * line_len(d.LZ) * (2 * sizeof(T) << o.lb);
         o.ctas = (ncol + (1 << o.lb) - 1) >> o.lb;
@@ -763,7 +760,7 @@ bool launch_line_conv(const DemagDims& d, typename Cplx<T>::type* S2, const T* t
         const bool idle = line_idle<T>(o.pl, ncol * d.nb);
         // components lie side by side in a CTA's threads, and whole warps are idle only
         // where there are many of them (an RK4 step of 128x128x25: 4880 -> 4150 us)
-        while (split && idle && ((6 * M) << o.lb) <= 384 && (ncol >> (o.lb + 1)) >= 8 * 152) {
+        while (split && idle && ((6 * M) << o.lb) <= 384 && (ncol >> (o.lb + 1)) >= 8 * kSms) {
             ++o.lb;
             o.threads = (((3 * M) << o.lb) + 31) / 32 * 32;
             o.smem *= 2;

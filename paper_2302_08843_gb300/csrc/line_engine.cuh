@@ -113,8 +113,8 @@ template <typename T> __host__ __device__ constexpr LinePlan line_ct(int L) { re
 // 256x256x1 105 against 68 us).  M: butterflies of the widest pass.
 template <typename T> __host__ __device__ constexpr bool line_split(int M) { return sizeof(T) == 8 && M <= 128; }
 // their columns per CTA (log2): a sector of each row at least, and three warps
-template <typename T> __host__ __device__ constexpr int line_split_lb(int M) {
-    int lb = sizeof(T) == 4 ? 2 : 1;
+__host__ __device__ constexpr int line_split_lb(int M) {
+    int lb = 1;
     while (lb < 5 && ((3 * M) << lb) < 96) ++lb;
     return lb;
 }

@@ -209,7 +209,6 @@ template <typename T, int MAXT, int LC, bool IDLE = false>
 __global__ void __launch_bounds__(MAXT)
 line_x_forward(DemagDims d, LineForward<T> f, typename Cplx<T>::type* __restrict__ S1,
                const __grid_constant__ LinePlan pl, const typename Cplx<T>::type* __restrict__ tw, int nt, int lines) {
-    constexpr int NC = 1;                            // components per line
     using C = typename Cplx<T>::type;
     extern __shared__ __align__(16) unsigned char smraw[];
     if constexpr (LC > 0) {
@@ -218,9 +217,9 @@ line_x_forward(DemagDims d, LineForward<T> f, typename Cplx<T>::type* __restrict
     }
     const LineThread t = line_thread(nt, lines);
     const int g = blockIdx.y, nx = d.nx, plane = line_len(LC ? LC : pl.L);
-    const LineRows r = line_rows<NC>(d, blockIdx.x * lines + t.l);
+    const LineRows r = line_rows<1>(d, blockIdx.x * lines + t.l);
     const long rows = (long)d.ny * d.nz;             // rows of one component
-    C* s = reinterpret_cast<C*>(smraw) + (size_t)t.l * NC * plane;
+    C* s = reinterpret_cast<C*>(smraw) + (size_t)t.l * plane;
     grid_dep_wait();
     if (f.mask && !f.mask[g]) return;
     const T* Ms_b = static_cast<const T*>(d.Ms_b);
@@ -231,53 +230,45 @@ line_x_forward(DemagDims d, LineForward<T> f, typename Cplx<T>::type* __restrict
         // kBatch elements of both rows in flight per thread
         constexpr int kBatch = 4;
         for (int x0 = t.b; x0 < nx; x0 += kBatch * nt) {
-            C v[NC][kBatch];
+            C v[kBatch];
 #pragma unroll
-            for (int q = 0; q < kBatch; ++q)
-#pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    const int x = min(x0 + q * nt, nx - 1);
-                    const T* m = f.m + (off + r.ra + c * rows) * nx + x;
-                    v[c][q] = mk<C>(__ldcg(m), r.two ? __ldcg(m + nx) : (T)0);
-                    if (f.k) {
-                        const T* k = f.k + (m - f.m);
-                        v[c][q].x += ca * __ldcg(k);
-                        if (r.two) v[c][q].y += ca * __ldcg(k + nx);
-                    }
+            for (int q = 0; q < kBatch; ++q) {
+                const int x = min(x0 + q * nt, nx - 1);
+                const T* m = f.m + (off + r.ra) * nx + x;
+                v[q] = mk<C>(__ldcg(m), r.two ? __ldcg(m + nx) : (T)0);
+                if (f.k) {
+                    const T* k = f.k + (m - f.m);
+                    v[q].x += ca * __ldcg(k);
+                    if (r.two) v[q].y += ca * __ldcg(k + nx);
                 }
+            }
 #pragma unroll
             for (int q = 0; q < kBatch; ++q) {
                 const int x = x0 + q * nt;
                 if (x >= nx) break;
-#pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    const long row = r.ra + c * rows;
-                    if (f.k) {
-                        T* y = f.y + (off + row) * nx + x;
-                        y[0] = v[c][q].x;
-                        if (r.two) y[nx] = v[c][q].y;
-                    }
-                    T ma = msu, mb = msu;
-                    if (f.Ms_cell && !Ms_b) {
-                        ma = f.Ms_cell[(row % rows) * nx + x];
-                        mb = r.two ? f.Ms_cell[((row + 1) % rows) * nx + x] : (T)0;
-                    }
-                    s[c * plane + line_place<4>(x)] = mk<C>(ma * v[c][q].x, mb * v[c][q].y);
+                if (f.k) {
+                    T* y = f.y + (off + r.ra) * nx + x;
+                    y[0] = v[q].x;
+                    if (r.two) y[nx] = v[q].y;
                 }
+                T ma = msu, mb = msu;
+                if (f.Ms_cell && !Ms_b) {
+                    ma = f.Ms_cell[(r.ra % rows) * nx + x];
+                    mb = r.two ? f.Ms_cell[((r.ra + 1) % rows) * nx + x] : (T)0;
+                }
+                s[line_place<4>(x)] = mk<C>(ma * v[q].x, mb * v[q].y);
             }
         }
     }
     __syncthreads();
     C* sa = S1 + (off + r.ra) * d.KXS;
-    line_forward<T, NC, LC, IDLE>(s, plane, t.b, nt, nx, pl, tw, sa, sa + d.KXS, rows * d.KXS,
-                        r.on && t.in, r.two);
+    line_forward<T, 1, LC, IDLE>(s, plane, t.b, nt, nx, pl, tw, sa, sa + d.KXS, 0, r.on && t.in, r.two);
 }
 
 template <typename T, int MAXT, int LC, bool IDLE = false>
 __global__ void __launch_bounds__(MAXT)
 line_x_inverse(DemagDims d, const typename Cplx<T>::type* __restrict__ S1, T* __restrict__ h,
                const __grid_constant__ LinePlan pl, const typename Cplx<T>::type* __restrict__ tw, int nt, int lines) {
-    constexpr int NC = 1;                            // components per line
     using C = typename Cplx<T>::type;
     extern __shared__ __align__(16) unsigned char smraw[];
     if constexpr (LC > 0) {
@@ -286,21 +277,18 @@ line_x_inverse(DemagDims d, const typename Cplx<T>::type* __restrict__ S1, T* __
     }
     const LineThread t = line_thread(nt, lines);
     const int nx = d.nx, plane = line_len(LC ? LC : pl.L);
-    const LineRows r = line_rows<NC>(d, blockIdx.x * lines + t.l);
+    const LineRows r = line_rows<1>(d, blockIdx.x * lines + t.l);
     const long rows = (long)d.ny * d.nz, off = (long)blockIdx.y * 3 * rows;
-    C* s = reinterpret_cast<C*>(smraw) + (size_t)t.l * NC * plane;
+    C* s = reinterpret_cast<C*>(smraw) + (size_t)t.l * plane;
     const C* sa = S1 + (off + r.ra) * d.KXS;
     grid_dep_wait();
-    line_inverse<T, NC, LC, IDLE>(sa, r.two ? sa + d.KXS : sa, rows * d.KXS, s, plane, t.b, pl, tw);
+    line_inverse<T, 1, LC, IDLE>(sa, r.two ? sa + d.KXS : sa, 0, s, plane, t.b, pl, tw);
     if (!r.on || !t.in) return;
     for (int x = t.b; x < nx; x += nt) {
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-            const C v = s[c * plane + line_place<4>(x)];
-            T* o = h + (off + r.ra + c * rows) * nx + x;
-            o[0] = v.x;
-            if (r.two) o[nx] = v.y;
-        }
+        const C v = s[line_place<4>(x)];
+        T* o = h + (off + r.ra) * nx + x;
+        o[0] = v.x;
+        if (r.two) o[nx] = v.y;
     }
 }
 
@@ -1013,7 +1001,10 @@ template <int LC> const void* line_ct_pick(LineKind kind) {
         case kLineFusedGen: return (const void*)line_fused<true, FT, LC>;
         case kLineXFwd: return (const void*)line_x_forward<float, 256, LC>;
         case kLineXInv: return (const void*)line_x_inverse<float, 256, LC>;
-        default: return (const void*)line_conv<float, kConvThree, YT, LC>;
+        default:
+            // z lines of up to 16 points stay in one thread's registers
+            if constexpr (LC <= 16) return nullptr;
+            else return (const void*)line_conv<float, kConvThree, YT, LC>;
     }
 }
 

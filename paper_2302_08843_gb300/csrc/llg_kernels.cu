@@ -489,7 +489,6 @@ struct StageShape {
     dim3 block, grid;
 };
 template <typename T> static StageShape stage_shape(int nx, int ny, int nz, bool vec_ok) {
-    constexpr int kSms = 152;
     StageShape s;
     s.vec = vec_ok && nx % 2 == 0 ? 2 : 1;
     int bx = kBX, by = kBY;
