@@ -2073,7 +2073,7 @@ template <typename T, int L> static void launch_p3(const DemagDims& d, typename 
     // tiles 16.5 against 14.6 us a pass; lines up to 16 points, one thread each,
     // are level up to 8704 tiles, but 16 points with y lines of 32 and 64 stay with TMA
     // (256x16x8 101 against 94 us, 16x16x8 70 against 62, 64x32x8 75 against 71).  The
-    // line engine takes all others, FP64 (64-point lines of 128x128x32 519 -> 393 us,
+    // line engine takes all others, FP64 (64-point lines of 128x128x32 519 -> 382 us,
     // 256 points of a 512x128x1 film 97 -> 44) and batches (16 grids of 100x100x8 63 ->
     // 34 us).
     constexpr int kTmaTiles = L <= 16 ? 8192 : L < 64 ? 1024 : L < 128 ? 560 : L < 256 ? 144 : 48;
@@ -2125,7 +2125,7 @@ template <typename T, int L, int DIR> static void launch_y(const DemagDims& d, c
         if (launch_py_tma<L, DIR>(d, in, out, st)) return;
     }
     // FP64 lines of 16 to 1024 points take the line engine (128x128x32: 144 and 157
-    // us -> 119 and 126 us; from 2048 points on a CTA holds one column of it, less
+    // us -> 115 and 120 us; from 2048 points on a CTA holds one column of it, less
     // than a sector: 49 against 44 us on 16x1024x4); FP32 lines the compiled
     // engines, which stay faster where exchanges and not FP64 instructions bound
     // the pass (384 points: 29 and 33 us against 54 and 44)
@@ -2362,7 +2362,7 @@ static void yzy(const DemagDims& d, typename Cplx<T>::type* S1, typename Cplx<T>
         // The TMA y pass that follows has CTAs of 4 to 16 threads on lines up to 64
         // points: placed while the z pass runs they are spared a start of 4 to 8 us (an
         // RK4 step of 256x8x2 82 -> 56 us, 256x16x4 98 -> 66, 256x16x2 92 -> 63, 256x16x16
-        // 120 -> 95, 256x32x2 95 -> 65, 400x32x4 130 -> 102).  CTAs of longer lines, or of
+        // 120 -> 95, 256x32x2 95 -> 65, 400x32x4 130 -> 85).  CTAs of longer lines, or of
         // 64 points beside long z or x lines, crowd on the SMs that the z pass leaves
         // first (64x32x32 81 -> 97 us, 768x32x2 97 -> 106, 512x64x2 77 -> 83).
         const bool tma_y = d.err && d.nb == 1 && is_pow2(d.LY) && d.LY >= 16;

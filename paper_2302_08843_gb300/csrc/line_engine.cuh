@@ -108,7 +108,7 @@ constexpr int kLineThreads = 512, kLineThreads32 = 256;
 // plan of an FP32 compiled length
 template <typename T> __host__ __device__ constexpr LinePlan line_ct(int L) { return line_plan(L, 8); }
 // FP64 z lines whose three components fit a CTA side by side take a thread per
-// butterfly and component (32x32x4: 9.5 -> 6.6 us, 128x128x32: 416 -> 393 us; in
+// butterfly and component (32x32x4: 9.5 -> 6.6 us, 128x128x32: 416 -> 382 us; in
 // FP32 the extra exchange costs more than the threads bring: 32 grids of
 // 256x256x1 105 against 68 us).  M: butterflies of the widest pass.
 template <typename T> __host__ __device__ constexpr bool line_split(int M) { return sizeof(T) == 8 && M <= 128; }
@@ -352,7 +352,7 @@ __device__ __forceinline__ void line_start(typename Cplx<T>::type* s, int plane,
 // Whether a warp has no butterfly in a pass of radix R (IDLE kernels: FP64 plans of
 // unequal radices).  Plans of one radix 2 and odd ones have 2.5 to 3.5 times as
 // many threads as their odd passes have butterflies, and in FP64 idle threads'
-// instructions take the pipe from the others: with them an RK4 step of 64x32x245
+// instructions take the pipe from the others: with them an RK4 stage of 64x32x245
 // (2 5 7 7) took 3307 us, without 1640.  FP32, bound by its exchanges, does without
 // the vote, and so do plans of equal radices (32x32x4 with the vote in its kernels:
 // 1342 against 1304 us).  Every warp is whole.

@@ -558,7 +558,7 @@ __device__ __forceinline__ void line_known(const StageParams<float>& p, float dt
 }
 
 // threads of a fused CTA at most, and the CTAs per SM asked of the register
-// allocator: 64 registers a thread, 112 with every term (GEN).  The passes wait
+// allocator: 64 registers a thread, 128 with every term (GEN).  The passes wait
 // on memory and shared memory, so warps count for more than registers (one
 // thread for all three components: 80 registers, 19 warps per SM, 95 us on 32
 // grids of 256x256x1).
